@@ -141,7 +141,9 @@ typedef struct {
   int gmres_max_iter; /* NK: inner iterations per Newton step; default 300 */
   double gmres_rtol;  /* NK: inner relative-residual floor; default 1e-6 */
   int warm_start;     /* 1 = start from the case's last converged voltages */
-  int cluster_size;   /* single-solve launch: CTAs per cluster (0 = autotuned) */
+  int cluster_size;   /* single-solve launch: CTAs per cluster (0 = chosen by
+                         size); with block_threads and scen_per_cta 0 also the
+                         CTAs per scenario of a resident batch */
   int block_threads;  /* threads per CTA (0 = autotuned) */
   int scen_per_cta;   /* batched launch: scenarios per CTA (0 = autotuned) */
   int nk_fallback;    /* PF_NK through pf_solve / pf_solve_batch: redo every
@@ -152,6 +154,7 @@ typedef struct {
   int kernel_by_kernel; /* batched PF_NR: 1 = launch the phase kernels one by one
                            instead of as one CUDA graph (for profilers, which
                            cannot look inside a graph with a conditional node);
+                           no effect where the batch runs as one resident launch;
                            default 0 */
   int krylov;         /* PF_NK inner solver: 0 = restarted GMRES(gmres_restart)
                          (default), 1 = BiCGSTAB (the method of Sec. III.B;
@@ -290,8 +293,10 @@ int pf_solve(pf_case c, const pf_opts* opts, double* vmag, double* vang,
 
 /*
  * B scenarios of one topology solved together over the shared symbolic
- * pattern (Newton-Raphson: phase kernels in one CUDA graph whose loop ends on
- * the device when no scenario runs; Newton-Krylov: one persistent launch).
+ * pattern (Newton-Raphson: one launch with each scenario's factor in the
+ * shared memory of a CTA or cluster where it fits and the batch is small, else
+ * phase kernels in one CUDA graph whose loop ends on the device when no
+ * scenario runs; Newton-Krylov: one persistent launch).
  * Scenario b uses p_load[b][*], q_load[b][*] (per bus or per slot; a load
  * scale per bus and scenario is these arrays scaled) and, single phase
  * only, p_gen[b][n]; NULL = the case's own values.  Outputs vmag[b][*],
@@ -353,9 +358,11 @@ int pf_drain(pf_ctx ctx, int timeout_ms);
  * Counters of the context's serving runtime since it started (all zero before
  * the first pf_submit).  Newton-Raphson requests (no reactive limits, default
  * launch shape) run as group launches: one launch solves several queued
- * requests of any cases and sizes, one CTA each (a cluster of 2 CTAs for
- * grids of 4,000 buses or feeders of 2,000 nodes and more, of 4 CTAs from
- * 16,000 buses or 5,000 nodes, of 8 CTAs from 40,000 buses or 12,000 nodes),
+ * requests of any cases and sizes, on the cluster of a resident single solve
+ * of the case where its factor fits shared memory, else on one CTA each (a
+ * cluster of 2 CTAs for grids of 4,000 buses or feeders of 2,000 nodes and
+ * more, of 4 CTAs from 16,000 buses or 5,000 nodes, of 8 CTAs from 40,000
+ * buses or 12,000 nodes),
  * and each request retires when its own solve ends.  Runs of queued requests of one case are coalesced into batched
  * solves (pf_submit).  Newton-Krylov requests and requests with reactive
  * limits run as one launch each.
@@ -472,8 +479,10 @@ int pf_branch_flows(pf_case c, int B, const double* vmag, const double* vang, do
  * its own phase.  Later batch solves of that B with scen_per_cta == 0 and
  * block_threads == 0 use the stored shapes; *opts (in: method, precision;
  * out: the chosen shape, for PF_NR that of the factorisation, which alone
- * also applies to the sweeps when passed back explicitly).  Without tuning,
- * a batch uses about one CTA per SM (at most 8 scenarios per CTA).
+ * also applies to the sweeps when passed back explicitly), or 0, 0 where the
+ * resident solves were faster than the phase kernels in those shapes.
+ * Without tuning, a batch uses about one CTA per SM (at most 8 scenarios per
+ * CTA), or the resident solves (pf_solve_batch).
  * Blocking; allocates the batch workspace.
  */
 int pf_autotune(pf_case c, int B, pf_opts* opts);

@@ -1,6 +1,7 @@
 // C ABI of the power-flow library: contexts, cases, solves and inspection
 // calls.  Host code only; every numeric step runs in the CUDA kernels of
-// newton.cuh (single solves, Newton-Krylov, served requests), batch.cu
+// resident.cu (single-phase Newton-Raphson that fits shared memory),
+// newton.cuh (other single solves, Newton-Krylov, served requests), batch.cu
 // (batched Newton-Raphson), flows.cu and qlim.cu.
 #include <cuda_runtime.h>
 
@@ -158,6 +159,7 @@ int SysBuf::build(const CaseData& c, const Ybus& y, Ordering ord, bool fill) {
     }
     d.v_source = c.v_source;
   }
+  bus_type = bt;
   cudaError_t e = cudaSuccess;
 #define UP(vec, field) \
   if (e == cudaSuccess) e = upload(mem, vec, &d.field)
@@ -282,6 +284,118 @@ void SysBuf::finish_view(const std::array<const int8_t*, 2>& g, int threads, Dev
     --solo;
   }
   out.fac_solo_from = solo;
+}
+
+// Threads of a resident CTA: about one per row of its share.
+static int resident_threads(int n, int P) {
+  int t = 32;
+  while (t < 512 && t * P < n) t <<= 1;
+  return t;
+}
+
+// The fewest CTAs whose shared memory holds a scenario: the factor's blocks,
+// right-hand sides, the ring and tables, with room for the cut's imbalance.
+static int resident_least(const Symbolic& s, bool fp32) {
+  const double blocks = ((double)s.nnz_lu() * 4 + 2.0 * s.n) * (fp32 ? 4 : 8);
+  for (int P = 1; P <= 16; P <<= 1)
+    if ((P > 1 ? 1.15 : 1.0) * blocks / P + 36 * 1024 <= 224 * 1024) return P;
+  return 0;
+}
+
+// Single solves: latency, so more CTAs than memory asks for, one per 400
+// rows.  Measured (us, P = 1 / 2 / 4 / 8 / 16): 500 buses mixed 140 / 145 /
+// 133 / 140 / 180; 2,749 buses FP64 - / - / 770 / 657 / 641.
+int resident_single(const Symbolic& s, bool fp32) {
+  int P = resident_least(s, fp32);
+  while (P > 0 && P < 16 && s.n > 400 * P) P <<= 1;
+  return P;
+}
+
+// Batches: the fewest CTAs per scenario, as long as the clusters make at most
+// this many waves over the SMs; beyond, the phase kernels' 32 scenarios per
+// warp win.  Measured (ms, resident against phase kernels in their best
+// shape): 2,000 buses mixed x 256 0.69 / 1.94, x 1,000 2.40 / 3.47, x 3,000
+// 6.83 / 6.99; 5,000 mixed x 256 3.4 / 4.7, x 1,000 11.9 / 8.3; 500 FP64 x
+// 256 0.89 / 1.55, x 1,000 3.1 / 2.3; 100 FP64 x 1,000 0.48 / 0.81.
+int resident_batch(const Symbolic& s, bool fp32, int B, int num_sms) {
+  const int P = resident_least(s, fp32);
+  const double waves = fp32 || s.n <= 128 ? 8.0 : 3.5;
+  return P > 0 && (double)B * P <= waves * num_sms ? P : 0;
+}
+
+int SysBuf::resident_for(const Ybus& y, bool fp32, int P, const ResidentPlan** out) {
+  std::lock_guard<std::mutex> lk(g_mu);
+  *out = nullptr;
+  auto& slot = res_cache[2 * P + (fp32 ? 1 : 0)];
+  if (slot) {
+    if (slot->ok) *out = slot.get();
+    return PF_OK;
+  }
+  slot = std::make_unique<ResidentPlan>();
+  ResidentPlan& r = *slot;
+  ResPlanHost h;
+  if (y.ybs != 1 || !res_plan(sym, P, resident_threads(sym.n, P), h)) return PF_OK;
+  r.smem = res_smem(h, fp32 ? 4 : 8);
+  if (r.smem > 224 * 1024 || resident_clusters(fp32, P, h.threads, r.smem) < 1) return PF_OK;
+  auto val = [&](int e) { return &y.val[2 * (size_t)sym.y_src[e]]; };
+  std::vector<double2> ell_y(h.ell_y.size(), make_double2(0.0, 0.0));
+  for (size_t k = 0; k < ell_y.size(); ++k)
+    if (h.ell_y[k] >= 0) ell_y[k] = make_double2(val(h.ell_y[k])[0], val(h.ell_y[k])[1]);
+  std::vector<int4> row(h.row.size() / 4), jac(h.jac.size() / 4);
+  std::vector<float2> diag32(row.size(), make_float2(0.f, 0.f));
+  std::vector<float2> jy32;
+  std::vector<double2> jy64;
+  for (size_t k = 0; k < row.size(); ++k) {
+    const int* s = &h.row[4 * k];
+    row[k] = make_int4(s[0], s[1], s[2], 0);
+    if (s[0] >= 0) diag32[k] = make_float2((float)val(s[3])[0], (float)val(s[3])[1]);
+  }
+  for (size_t k = 0; k < jac.size(); ++k) {
+    const int* s = &h.jac[4 * k];
+    jac[k] = make_int4(s[0], s[1], s[2], bus_type[s[1]] | bus_type[s[2]] << 8);
+    if (fp32) jy32.push_back(make_float2((float)val(s[3])[0], (float)val(s[3])[1]));
+    else jy64.push_back(make_double2(val(s[3])[0], val(s[3])[1]));
+  }
+  std::vector<int2> rnd(h.rnd.size() / 2), gsrc(h.gsrc.size() / 2);
+  std::vector<uint2> rec(h.rec.size() / 2);
+  std::vector<int4> gat(h.gat.size() / 4);
+  for (size_t k = 0; k < rnd.size(); ++k) rnd[k] = make_int2(h.rnd[2 * k], h.rnd[2 * k + 1]);
+  for (size_t k = 0; k < gsrc.size(); ++k) gsrc[k] = make_int2(h.gsrc[2 * k], h.gsrc[2 * k + 1]);
+  for (size_t k = 0; k < rec.size(); ++k) rec[k] = make_uint2(h.rec[2 * k], h.rec[2 * k + 1]);
+  for (size_t k = 0; k < gat.size(); ++k)
+    gat[k] = make_int4(h.gat[4 * k], h.gat[4 * k + 1], h.gat[4 * k + 2], h.gat[4 * k + 3]);
+  ResDev& d = r.dev;
+  d.P = P;
+  d.threads = h.threads;
+  d.ngat_blk = h.ngat_blk;
+  d.ngat_vec = h.ngat_vec;
+  d.max_blk = h.max_blk;
+  d.max_vec = h.max_vec;
+  cudaError_t e = upload(mem, h.part, &d.part);
+  if (e == cudaSuccess) e = upload(mem, h.cta, &d.cta);
+  if (e == cudaSuccess) e = upload(mem, h.grp, &d.grp);
+  if (e == cudaSuccess) e = upload(mem, row, &d.row);
+  if (e == cudaSuccess) e = upload(mem, diag32, &d.diag32);
+  if (e == cudaSuccess) e = upload(mem, h.ell_col, &d.ell_col);
+  if (e == cudaSuccess) e = upload(mem, ell_y, &d.ell_y);
+  if (e == cudaSuccess) e = upload(mem, jac, &d.jac);
+  const float2* j32 = nullptr;
+  const double2* j64 = nullptr;
+  if (e == cudaSuccess) e = fp32 ? upload(mem, jy32, &j32) : upload(mem, jy64, &j64);
+  d.jac_y = fp32 ? (const void*)j32 : (const void*)j64;
+  if (e == cudaSuccess) e = upload(mem, rnd, &d.rnd);
+  if (e == cudaSuccess) e = upload(mem, rec, &d.rec);
+  if (e == cudaSuccess) e = upload(mem, h.bnd, &d.bnd);
+  if (e == cudaSuccess) e = upload(mem, gat, &d.gat);
+  if (e == cudaSuccess) e = upload(mem, gsrc, &d.gsrc);
+  if (e == cudaSuccess) e = upload(mem, std::vector<ResDev>(1, d), &r.d_dev);
+  if (e != cudaSuccess) {
+    res_cache.erase(2 * P + (fp32 ? 1 : 0));
+    return cuda_error(e, "uploading a resident plan");
+  }
+  r.ok = true;
+  *out = &r;
+  return PF_OK;
 }
 
 // ---------------------------------------------------------------------------
@@ -535,6 +649,15 @@ int pf_create_case(pf_ctx ctx, const pf_case_desc* desc, pf_case* out) {
     DevSys unused;
     rc = c->nr.lanes_for(pf::noalloc_threads(c->bs), 1, unused);
     if (rc != PF_OK) return rc;
+    // and the resident plans of single solves
+    for (int fp32 = 0; fp32 < 2 && c->data.kind == PF_SINGLE_PHASE; ++fp32) {
+      const ResidentPlan* plan = nullptr;
+      for (int P = resident_single(c->nr.sym, fp32 != 0); P > 0 && P <= 16 && !plan; P <<= 1) {
+        rc = c->nr.resident_for(c->y, fp32 != 0, P, &plan);
+        if (rc != PF_OK) return rc;
+      }
+      c->nr.res_single[fp32] = plan;
+    }
   }
   {
     const int ki = c->data.kind == PF_SINGLE_PHASE ? 0 : 1;
@@ -757,6 +880,14 @@ int pf_analyze(const pf_case_desc* desc, pf_case_stats* out) {
                 s->blev_ptr.size() + s->blev_rows.size() + s->perm.size());
     b += (long long)y.val.size() * 8 + (long long)d.n * (1 + 8 * 9);
   }
+  for (int fp32 = 0; fp32 < 2 && y.ybs == 1; ++fp32) {  // the plans of resident single solves
+    ResPlanHost h;
+    const int P = resident_single(nr, fp32 != 0);
+    if (P > 0 && res_plan(nr, P, resident_threads(nr.n, P), h))
+      b += 4LL * (long long)(h.row.size() + h.ell_col.size() + h.jac.size() + h.rnd.size() +
+                             h.rec.size() + h.bnd.size() + h.gat.size() + h.gsrc.size()) +
+           16LL * (long long)h.ell_y.size() + (fp32 ? 2LL : 4LL) * (long long)h.jac.size();
+  }
   out->device_bytes = b;
   return PF_OK;
 }
@@ -943,6 +1074,16 @@ int pf_launch_config(pf_case c, const pf_opts* opts, int B, int* grid, int* clus
   pf_opts o;
   if (opts) o = *opts; else pf_opts_default(&o);
   cudaSetDevice(c->ctx->device);
+  const ResidentPlan* plan = nullptr;
+  const int rc = resident_plan(c, o, B, RunMode::Solve, &plan);
+  if (rc != PF_OK) return rc;
+  if (plan) {
+    *grid = B * plan->dev.P;
+    *cluster = plan->dev.P;
+    *threads = plan->dev.threads;
+    *scen = 1;
+    return PF_OK;
+  }
   launch_shape(c, o, B, o.precision == PF_MIXED, grid, cluster, threads, scen);
   return PF_OK;
 }

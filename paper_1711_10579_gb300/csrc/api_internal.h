@@ -13,6 +13,7 @@
 
 #include "device.h"
 #include "host.h"
+#include "resident.h"
 
 namespace pf {
 
@@ -28,11 +29,20 @@ struct DevBuffer {
   cudaError_t alloc(void** out, size_t nbytes);
 };
 
+// A resident plan on the device.
+struct ResidentPlan {
+  ResDev dev{};
+  const ResDev* d_dev = nullptr;  // a copy in device memory (group launches)
+  size_t smem = 0;
+  bool ok = false;  // fits the device (else the case runs the other kernels)
+};
+
 // One ordering of a case: host symbolic analysis plus its device copy.
 struct SysBuf {
   Symbolic sym;
   DevSys view{};
   DevBuffer mem;
+  std::vector<int8_t> bus_type;  // in the ordering's numbering
   std::map<int, std::array<const int8_t*, 2>> g_cache;
   std::mutex g_mu;  // the serving thread and callers share g_cache
   int build(const CaseData& c, const Ybus& y, Ordering ord, bool fill);
@@ -40,8 +50,15 @@ struct SysBuf {
   // and cached); lanes_cached only looks them up and fails if absent.
   int lanes_for(int threads, int S, DevSys& out);
   int lanes_cached(int threads, int S, DevSys& out);
+  // The resident plan of P CTAs, built and uploaded on first use; null if the
+  // case does not fit it.
+  int resident_for(const Ybus& y, bool fp32, int P, const ResidentPlan** out);
+  // The plan of single solves (FP64, FP32), built with the case, or null.
+  const ResidentPlan* res_single[2] = {nullptr, nullptr};
 
  private:
+  std::map<int, std::unique_ptr<ResidentPlan>> res_cache;  // 2 P + fp32
+
   void finish_view(const std::array<const int8_t*, 2>& g, int threads, DevSys& out) const;
 };
 
@@ -123,12 +140,17 @@ struct pf_case_s {
   std::mutex mu;
   // autotuned batch shapes: (B, method, precision) -> (scenarios per CTA,
   // threads) of the factorisation (Newton-Krylov: the whole launch), then of
-  // the triangular sweeps of a Newton-Raphson batch
-  std::map<std::array<int, 3>, std::array<int, 4>> tuned;
+  // the triangular sweeps of a Newton-Raphson batch, then whether the
+  // resident solves were faster than both
+  std::map<std::array<int, 3>, std::array<int, 5>> tuned;
   std::mutex tuned_mu;
 };
 
 namespace pf {
+
+// CTAs of a resident solve (of one scenario of a batch of B), 0: none.
+int resident_single(const Symbolic& s, bool fp32);
+int resident_batch(const Symbolic& s, bool fp32, int B, int num_sms);
 
 enum class RunMode { Solve, Eval, Step };
 enum class InspectKind { Mismatch, Jacobian, Step };
@@ -136,6 +158,7 @@ enum class InspectKind { Mismatch, Jacobian, Step };
 // Launches one solve of B scenarios on `ws` (asynchronous on `st`).
 // Outputs go to out_vm / out_va / out_info when given, else to the
 // workspace's staging buffers.
+int resident_plan(pf_case c, const pf_opts& o, int B, RunMode mode, const ResidentPlan** out);
 int run_solve(pf_case c, const pf_opts& o, int B, const double* d_p_load,
               const double* d_q_load, const double* d_p_gen, Workspace* ws,
               cudaStream_t st, RunMode mode, double* out_vm, double* out_va,

@@ -147,6 +147,8 @@ struct DevWork {
   double* qus;               // [B] device time of the rounds
   pf_info* qinfo;            // [B] result of a scenario that failed
   int* nsw;                  // buses switched by the last check (one counter)
+  int by_scen;               // 1: the state is laid out [scenario][row] (resident
+                             // solves), else [row][scenario]
 };
 
 // Inputs and outputs of one batched call, read by the phase kernels from
@@ -185,11 +187,13 @@ size_t dynamic_smem_bytes(int bs, size_t tf, bool nk, int n, const DevOpts& o, i
 // One single-CTA solve of a group launch (several cases of different sizes
 // in one launch): its case, workspace and options, and the flag the CTA
 // raises (1) once its results are written.
+struct ResDev;
 struct GroupJob {
   DevSys S;
   DevWork w;
   DevOpts o;
   int* done;
+  const ResDev* res;  // resident solves: the plan (device memory)
 };
 constexpr int kGroupMax = 160;  // jobs of one group launch
 // The jobs of a launch: CTA b runs desc[job[b]].

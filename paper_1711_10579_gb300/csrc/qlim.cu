@@ -14,7 +14,8 @@
 // of the current-injection Newton (w.qg); a slot outside [q_min, q_max] is
 // held at the limit it crossed (w.qg fixed, its bit set in w.bt, |V| free)
 // and keeps the plain columns of Eq. 21-23 in the next round.
-// Rows are in the numbering of the solve's ordering; w.bt is [row][B].
+// Rows are in the numbering of the solve's ordering; the state is [row][B], or
+// [B][row] after resident solves (w.by_scen).
 
 #include <cuda_runtime.h>
 
@@ -26,11 +27,18 @@ namespace {
 
 constexpr int kThreads = 256;
 
+// Row and scenario of state index k.
+__device__ __forceinline__ void split(const DevSys& S, const DevWork& w, size_t k, int& i, int& gs) {
+  i = (int)(w.by_scen ? k % S.n : k / w.B);
+  gs = (int)(w.by_scen ? k / S.n : k % w.B);
+}
+
 __global__ void __launch_bounds__(kThreads) k_qlim_init(DevSys S, DevWork w, int three) {
   const size_t k = (size_t)blockIdx.x * kThreads + threadIdx.x;
   const int B = w.B;
   if (k >= (size_t)S.n * B) return;
-  const int i = (int)(k / B), gs = (int)(k % B);
+  int i, gs;
+  split(S, w, k, i, gs);
   if (three) {
     w.bt[k] = 0;  // no phase held
   } else {
@@ -55,7 +63,8 @@ __global__ void __launch_bounds__(kThreads) k_qlim_check(DevSys S, DevWork w, co
   const size_t k = (size_t)blockIdx.x * kThreads + threadIdx.x;
   const int B = w.B;
   if (k >= (size_t)S.n * B) return;
-  const int i = (int)(k / B), gs = (int)(k % B);
+  int i, gs;
+  split(S, w, k, i, gs);
   const int status = info[gs].status;
   if (w.qdone[gs]) return;  // failed in an earlier round
   if (i == 0) {
@@ -101,7 +110,8 @@ __global__ void __launch_bounds__(kThreads) k_qlim_check(DevSys S, DevWork w, co
   const double2* Y = reinterpret_cast<const double2*>(S.y_val);
   double2 I = make_double2(0.0, 0.0);
   for (int e = S.y_rowptr[i]; e < S.y_rowptr[i + 1]; ++e) {
-    const double2 y = Y[e], v = w.V[(size_t)S.y_col[e] * B + gs];
+    const size_t j = S.y_col[e];
+    const double2 y = Y[e], v = w.V[w.by_scen ? (size_t)gs * S.n + j : j * B + gs];
     I.x += y.x * v.x - y.y * v.y;
     I.y += y.x * v.y + y.y * v.x;
   }

@@ -1,0 +1,704 @@
+// Resident single-phase Newton-Raphson solves (resident.h): one scenario per
+// CTA or per cluster, its whole factor in shared memory.
+//
+// What bounds it: a solve is a chain of ~2 x 40-70 dependent levels per
+// Newton step, most of them a few dozen 2x2 blocks wide.  With the factor in
+// global memory (newton.cuh) a level cost two cluster barriers and two or
+// three dependent L2 round trips, 1.4 us of factorisation and 2 x 1.4 us of
+// sweeps; here it is one round of shared-memory reads, a few FMAs and a block
+// barrier.
+#include "kernels.cuh"
+#include "resident.h"
+
+namespace pf {
+
+namespace {
+
+// 8-byte asynchronous copy global -> shared.
+__device__ __forceinline__ void cp8(void* smem, const void* gmem) {
+  const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem) : "memory");
+}
+
+template <typename TF>
+struct Blk {
+  TF a, b, c, d;  // [a b; c d]
+};
+template <typename TF>
+struct Vec2;
+template <>
+struct Vec2<float> {
+  using T = float2;
+};
+template <>
+struct Vec2<double> {
+  using T = double2;
+};
+
+__device__ __forceinline__ Blk<float> ld_blk(const float* p) {
+  const float4 v = *reinterpret_cast<const float4*>(p);
+  return {v.x, v.y, v.z, v.w};
+}
+__device__ __forceinline__ Blk<double> ld_blk(const double* p) {
+  const double2 v = reinterpret_cast<const double2*>(p)[0], u = reinterpret_cast<const double2*>(p)[1];
+  return {v.x, v.y, u.x, u.y};
+}
+__device__ __forceinline__ void st_blk(float* p, const Blk<float>& v) {
+  *reinterpret_cast<float4*>(p) = make_float4(v.a, v.b, v.c, v.d);
+}
+__device__ __forceinline__ void st_blk(double* p, const Blk<double>& v) {
+  reinterpret_cast<double2*>(p)[0] = make_double2(v.a, v.b);
+  reinterpret_cast<double2*>(p)[1] = make_double2(v.c, v.d);
+}
+__device__ __forceinline__ float2 mk2(float x, float y) { return make_float2(x, y); }
+__device__ __forceinline__ double2 mk2(double x, double y) { return make_double2(x, y); }
+
+// a b + c d with the roundings written out: the kernels that inline a solve
+// (alone, and in a group launch) must not contract it differently, or a
+// served result would differ from the same solve alone.
+__device__ __forceinline__ float dot2(float a, float b, float c, float d) {
+  return __fmaf_rn(a, b, __fmul_rn(c, d));
+}
+__device__ __forceinline__ double dot2(double a, double b, double c, double d) {
+  return __fma_rn(a, b, __dmul_rn(c, d));
+}
+__device__ __forceinline__ float nmac2(float v, float a, float b, float c, float d) {  // v - a b - c d
+  return __fmaf_rn(-c, d, __fmaf_rn(-a, b, v));
+}
+__device__ __forceinline__ double nmac2(double v, double a, double b, double c, double d) {
+  return __fma_rn(-c, d, __fma_rn(-a, b, v));
+}
+
+// Inverse in closed form; false for a zero or non-finite determinant or
+// inverse (the rule of the batched factorisation).
+template <typename TF>
+__device__ __forceinline__ bool inv2(Blk<TF>& m) {
+  const TF det = dot2(m.a, m.d, -m.b, m.c);
+  const TF r = TF(1) / det;
+  const Blk<TF> v{m.d * r, -m.b * r, -m.c * r, m.a * r};
+  m = v;
+  return det != TF(0) && isfinite(v.a) && isfinite(v.b) && isfinite(v.c) && isfinite(v.d);
+}
+
+// Bus state: written by any CTA of the cluster (L2) or by this CTA alone.
+template <bool CL, typename T>
+__device__ __forceinline__ T ld_state(const T* p) {
+  if constexpr (CL) {
+    return __ldcg(p);
+  } else {
+    return *p;
+  }
+}
+
+enum { kFactor = 0, kForward = 1, kBackward = 2 };
+
+// The rounds tab[0 .. nr) of one part (blocks A, vector y).  A thread's items
+// of the next kResRing rounds are in flight by cp.async, so a round waits
+// for no global load.  Ends with a block barrier (nr > 0).
+template <int MODE, typename TF>
+__device__ __noinline__ void run_rounds(const int2* tab, int nr, const uint2* __restrict__ rec, TF* A,
+                                        TF* y, uint2* ring, int* flag) {
+  using V2 = typename Vec2<TF>::T;
+  constexpr int D = kResRing;
+  const int t = threadIdx.x, T = blockDim.x;
+  V2* yv = reinterpret_cast<V2*>(y);
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    if (d < nr) {
+      const int2 q = tab[d];
+      if (t < (q.y & 0xffff)) cp8(ring + d * T + t, rec + q.x + t);
+    }
+    cp_commit();
+  }
+  for (int r = 0; r < nr; ++r) {
+    const int2 q = tab[r];
+    cp_wait<D - 1>();
+    uint2* mine = ring + (r & (D - 1)) * T + t;
+    if (t < (q.y & 0xffff)) {
+      const uint2 it = *mine;
+      const int x = it.x & 0xffff;
+      if (x != kResNone) {
+        const int b = it.x >> 16, c = it.y & 0xffff, k = (it.y >> 16) & (kResMaxRows - 1);
+        if constexpr (MODE == kBackward) {
+          V2 v = yv[x];
+          if (b != kResNone) {
+            const Blk<TF> B = ld_blk(A + 4 * b);
+            const V2 u = yv[c];
+            v.x = nmac2(v.x, B.a, u.x, B.b, u.y);
+            v.y = nmac2(v.y, B.c, u.x, B.d, u.y);
+          }
+          if (it.y & kResFinal) {
+            const Blk<TF> Di = ld_blk(A + 4 * x);
+            v = mk2(dot2(Di.a, v.x, Di.b, v.y), dot2(Di.c, v.x, Di.d, v.y));
+          }
+          yv[x] = v;
+        } else {
+          const Blk<TF> B = ld_blk(A + 4 * b), Di = ld_blk(A + 4 * k);
+          if (MODE == kForward || (it.y & kResVec)) {
+            const V2 u = yv[k];
+            V2 v = yv[x];
+            const TF m0 = dot2(Di.a, u.x, Di.b, u.y), m1 = dot2(Di.c, u.x, Di.d, u.y);
+            v.x = nmac2(v.x, B.a, m0, B.b, m1);
+            v.y = nmac2(v.y, B.c, m0, B.d, m1);
+            yv[x] = v;
+          } else {
+            const Blk<TF> U = ld_blk(A + 4 * c);
+            Blk<TF> v = ld_blk(A + 4 * x);
+            const Blk<TF> m{dot2(Di.a, U.a, Di.b, U.c), dot2(Di.a, U.b, Di.b, U.d),
+                            dot2(Di.c, U.a, Di.d, U.c), dot2(Di.c, U.b, Di.d, U.d)};
+            v.a = nmac2(v.a, B.a, m.a, B.b, m.c);
+            v.b = nmac2(v.b, B.a, m.b, B.b, m.d);
+            v.c = nmac2(v.c, B.c, m.a, B.d, m.c);
+            v.d = nmac2(v.d, B.c, m.b, B.d, m.d);
+            if (it.y & kResFinal) {
+              if (!inv2(v)) *flag = 1;
+            }
+            st_blk(A + 4 * x, v);
+          }
+        }
+      }
+    }
+    if (r + D < nr) {
+      const int2 f = tab[r + D];
+      if (t < (f.y & 0xffff)) cp8(mine, rec + f.x + t);
+    }
+    cp_commit();
+    if (q.y < 0) __syncthreads();
+  }
+}
+
+// Off-diagonal Jacobian block (Eq. 10) of entry (i, j) of types ti, tj.
+template <bool CL>
+__device__ __forceinline__ Blk<float> jac_block(const DevWork& w, int i, int j, int ti, int tj,
+                                                float2 y) {
+  const double2 Vi = ld_state<CL>(w.V + i), Vj = ld_state<CL>(w.V + j);
+  Blk<float> o{0.f, 0.f, 0.f, 0.f};
+  if (ti == PF_SLACK || tj == PF_SLACK) return o;
+  const float vix = to_f32_trunc(Vi.x), viy = to_f32_trunc(Vi.y);
+  const float vjx = to_f32_trunc(Vj.x), vjy = to_f32_trunc(Vj.y);
+  const float yvx = dot2(y.x, vjx, -y.y, vjy), yvy = dot2(y.x, vjy, y.y, vjx);
+  const float cx = dot2(vix, yvx, viy, yvy), cy = dot2(viy, yvx, -vix, yvy);
+  o.a = cy;
+  o.c = -cx;
+  if (tj >= PF_PQ) {
+    const float rv = rsqrtf(dot2(vjx, vjx, vjy, vjy));
+    o.b = cx * rv;
+    o.d = cy * rv;
+  }
+  if (ti == PF_PV) o.c = o.d = 0.f;
+  return o;
+}
+template <bool CL>
+__device__ __forceinline__ Blk<double> jac_block(const DevWork& w, int i, int j, int ti, int tj,
+                                                 double2 y) {
+  const double2 Vi = ld_state<CL>(w.V + i), Uj = ld_state<CL>(w.U + j);
+  const double vmj = ld_state<CL>(w.vm + j);
+  Blk<double> o{0.0, 0.0, 0.0, 0.0};
+  if (ti == PF_SLACK || tj == PF_SLACK) return o;
+  const double yux = dot2(y.x, Uj.x, -y.y, Uj.y), yuy = dot2(y.x, Uj.y, y.y, Uj.x);
+  const double cx = dot2(Vi.x, yux, Vi.y, yuy), cy = dot2(Vi.y, yux, -Vi.x, yuy);
+  o.a = vmj * cy;
+  o.c = -vmj * cx;
+  if (tj >= PF_PQ) {
+    o.b = cx;
+    o.d = cy;
+  }
+  if (ti == PF_PV) o.c = o.d = 0.0;
+  return o;
+}
+
+// Diagonal Jacobian block of row i: V, I of the row, its mismatch power S and
+// loads, the Ybus diagonal.
+__device__ __forceinline__ Blk<float> diag_block(const DevSys& S, int i, int t, double2 Vi, double2,
+                                                 double vm, double2 I, double2, double pl, double ql,
+                                                 float2 y) {
+  if (t == PF_SLACK) return {1.f, 0.f, 0.f, 1.f};
+  const float vix = to_f32_trunc(Vi.x), viy = to_f32_trunc(Vi.y);
+  const float Ix = to_f32_trunc(I.x), Iy = to_f32_trunc(I.y);
+  const float rvi = rsqrtf(dot2(vix, vix, viy, viy));
+  const float uix = vix * rvi, uiy = viy * rvi;
+  const float yvx = dot2(y.x, vix, -y.y, viy), yvy = dot2(y.x, viy, y.y, vix);
+  const float scx = dot2(vix, Ix, viy, Iy), scy = dot2(viy, Ix, -vix, Iy);
+  const float dx = dot2(vix, yvx, viy, yvy), dy = dot2(viy, yvx, -vix, yvy);
+  const float ax = Ix + yvx, ay = Iy + yvy;
+  const float ex = dot2(uix, ax, uiy, ay), ey = dot2(uiy, ax, -uix, ay);
+  const float dshape = fmaf(2.f * S.zip32[3 * i + 2], to_f32_trunc(vm), S.zip32[3 * i + 1]);
+  Blk<float> o{-(scy - dy), fmaf(to_f32_trunc(pl), dshape, ex), scx - dx,
+               fmaf(to_f32_trunc(ql), dshape, ey)};
+  if (t == PF_PV) {
+    o.b = o.c = 0.f;
+    o.d = 1.f;
+  }
+  return o;
+}
+__device__ __forceinline__ Blk<double> diag_block(const DevSys& S, int i, int t, double2 Vi,
+                                                  double2 Ui, double vm, double2 I, double2 Sc,
+                                                  double pl, double ql, double2 y) {
+  if (t == PF_SLACK) return {1.0, 0.0, 0.0, 1.0};
+  const double dshape = fma(2.0 * S.zip[3 * i + 2], vm, S.zip[3 * i + 1]);
+  const double yvx = dot2(y.x, Vi.x, -y.y, Vi.y), yvy = dot2(y.x, Vi.y, y.y, Vi.x);
+  const double dx = dot2(Vi.x, yvx, Vi.y, yvy), dy = dot2(Vi.y, yvx, -Vi.x, yvy);
+  const double ax = I.x + yvx, ay = I.y + yvy;
+  const double ex = dot2(Ui.x, ax, Ui.y, ay), ey = dot2(Ui.y, ax, -Ui.x, ay);
+  Blk<double> o{-(Sc.y - dy), fma(pl, dshape, ex), Sc.x - dx, fma(ql, dshape, ey)};
+  if (t == PF_PV) {
+    o.b = o.c = 0.0;
+    o.d = 1.0;
+  }
+  return o;
+}
+
+// One scenario on the CTAs of a cluster (CL) or one CTA.  w: the scenario's
+// own state (B = 1).
+template <typename TF, bool CL>
+__device__ __forceinline__ void resident_solve(const DevSys& S, const DevWork& w, const DevOpts& o,
+                                               const ResDev& R, int lin) {
+  using V2 = typename Vec2<TF>::T;
+  const int P = CL ? (int)cg::this_cluster().num_blocks() : 1;
+  const int crank = CL ? (int)cg::this_cluster().block_rank() : 0;
+  const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarp = T >> 5;
+  extern __shared__ __align__(16) unsigned char dsm[];
+  TF* const A = reinterpret_cast<TF*>(dsm);
+  TF* const y = A + (size_t)R.max_blk * 4;
+  uint2* const ring = reinterpret_cast<uint2*>(
+      dsm + (((size_t)R.max_blk * 4 * sizeof(TF) + (size_t)R.max_vec * 2 * sizeof(TF) + 15) & ~(size_t)15));
+  int2* const tab = reinterpret_cast<int2*>(ring + (size_t)kResRing * T);
+  __shared__ ResPart sp[2];  // this CTA's part, and the top
+  __shared__ ResCta sc;
+  __shared__ unsigned long long sh_norm[16], sh_step[16], sh_red[32];
+  __shared__ int sh_flag;
+  if (tid == 0) {
+    sp[0] = R.part[crank];
+    sp[1] = R.part[CL ? P : 0];
+    sc = R.cta[crank];
+    sh_flag = 0;
+  }
+  const unsigned long long t_begin = global_ns();
+  __syncthreads();
+  const ResPart& part = sp[0];
+  const ResPart& top = sp[1];
+  const bool has_top = CL && crank == 0;
+  const int n_top_tab = has_top ? top.rb + top.nrb - top.rf : 0;
+  for (int k = tid; k < sc.ntab; k += T) tab[k] = R.rnd[sc.tab + k];
+  for (int k = tid; k < n_top_tab; k += T) tab[sc.ntab + k] = R.rnd[top.rf + k];
+  TF* const Ap = A + 4 * part.blk0;
+  TF* const yp = y + 2 * part.vec0;
+  TF* const At = A + 4 * top.blk0;
+  TF* const yt = y + 2 * top.vec0;
+  auto remote = [&](auto* p, int r) {
+    if constexpr (CL) {
+      return cg::this_cluster().map_shared_rank(p, r);
+    } else {
+      return p;
+    }
+  };
+  const bool prof = o.prof != nullptr && blockIdx.x == 0 && tid == 0;
+  unsigned long long t_last = prof ? t_begin : 0ull;
+  auto tick = [&](int phase) {
+    if (prof) {
+      const unsigned long long t = global_ns();
+      o.prof[phase] += t - t_last;
+      t_last = t;
+    }
+  };
+  // fn(row record) for this CTA's rows
+  auto rows = [&](auto fn) {
+    for (int g = warp; g < sc.ngrp; g += nwarp) {
+      const int4 r = __ldg(R.row + (size_t)(sc.grp + g) * 32 + lane);
+      if (r.x >= 0) fn(r.x & ~kResRowLevel0, r);
+    }
+  };
+  // largest value over the cluster into slot[] of every CTA (read after the
+  // next barrier)
+  auto spread = [&](unsigned long long m, unsigned long long* slot) {
+    for (int off = 16; off > 0; off >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, off));
+    if (lane == 0) sh_red[warp] = m;
+    __syncthreads();
+    if (tid < P) {
+      unsigned long long v = 0ull;
+      for (int q = 0; q < nwarp; ++q) v = max(v, sh_red[q]);
+      remote(slot, tid)[crank] = v;
+    }
+  };
+  auto widest = [&](const unsigned long long* slot) {
+    unsigned long long v = 0ull;
+    for (int q = 0; q < P; ++q) v = max(v, slot[q]);
+    return __longlong_as_double((long long)v);
+  };
+  auto put_info = [&](int st, int it, int passes, double nrm, double step) {
+    if (crank != 0 || tid != 0 || !w.out_info) return;
+    pf_info inf;
+    inf.status = st;
+    inf.iterations = it;
+    inf.linear_iterations = lin ? passes : 0;
+    inf.fallback = 0;
+    inf.mismatch = nrm;
+    inf.max_step = step;
+    inf.solve_us = 0.0;
+    inf.q_switched = 0;
+    inf.q_rounds = 1;
+    *w.out_info = inf;
+  };
+  rows([&](int i, const int4&) {
+    const int oi = S.perm[i];
+    setup_1ph(S, w, i, 0, w.in_p_load ? w.in_p_load[oi] : S.p_load0[i],
+              w.in_q_load ? w.in_q_load[oi] : S.q_load0[i],
+              w.in_p_gen ? w.in_p_gen[oi] : S.p_gen0[i]);
+  });
+  csync<CL>();
+  tick(kProfSetup);
+
+  int status = kRunning, passes = 0;
+  double prev = 0.0;
+  for (int it = 0;; ++it) {
+    // ---- mismatch (Eq. 8-9), right-hand side and Jacobian (Eq. 10) ----
+    for (int k = part.z0 + tid; k < part.nblk; k += T) st_blk(Ap + 4 * k, Blk<TF>{0, 0, 0, 0});
+    for (int k = part.np + tid; k < part.np + part.nb; k += T)
+      reinterpret_cast<V2*>(yp)[k] = mk2(TF(0), TF(0));
+    if (has_top)
+      for (int k = top.z0 + tid; k < top.nblk; k += T) st_blk(At + 4 * k, Blk<TF>{0, 0, 0, 0});
+    for (int e = tid; e < sc.njac; e += T) {
+      const int4 r = __ldg(R.jac + sc.jac + e);
+      const V2 yv = __ldg(reinterpret_cast<const V2*>(R.jac_y) + sc.jac + e);
+      const int ti = w.bt ? w.bt[r.y] : (r.w & 0xff), tj = w.bt ? w.bt[r.z] : (r.w >> 8);
+      st_blk(A + 4 * r.x, jac_block<CL>(w, r.y, r.z, ti, tj, yv));
+    }
+    unsigned long long m = 0ull;
+    for (int g = warp; g < sc.ngrp; g += nwarp) {
+      const ResGroup G = R.grp[sc.grp + g];
+      const size_t rl = (size_t)(sc.grp + g) * 32 + lane;
+      const int4 r = __ldg(R.row + rl);
+      const bool on = r.x >= 0;
+      const int i = on ? (r.x & ~kResRowLevel0) : 0;
+      const double2 Vi = ld_state<CL>(w.V + i);
+      const double vmi = ld_state<CL>(w.vm + i);
+      const double pl = w.spec[3 * (size_t)i], ql = w.spec[3 * (size_t)i + 1],
+                   pg = w.spec[3 * (size_t)i + 2];
+      const double zp = S.zip[3 * i], zi = S.zip[3 * i + 1], zz = S.zip[3 * i + 2];
+      const int t = w.bt ? w.bt[i] : S.btype[i];
+      double2 I = make_double2(0.0, 0.0), yd = make_double2(0.0, 0.0);
+#pragma unroll 4
+      for (int e = 0; e < G.width; ++e) {
+        const size_t q = (size_t)G.ell + 32 * e + lane;
+        const int j = __ldg(R.ell_col + q);
+        const double2 yv = __ldg(R.ell_y + q), v = ld_state<CL>(w.V + j);
+        if (sizeof(TF) == 8 && e == 0) yd = yv;
+        I.x = fma(yv.x, v.x, I.x);
+        I.x = fma(-yv.y, v.y, I.x);
+        I.y = fma(yv.x, v.y, I.y);
+        I.y = fma(yv.y, v.x, I.y);
+      }
+      if (!on) continue;
+      const double2 Sc = make_double2(dot2(Vi.x, I.x, Vi.y, I.y), dot2(Vi.y, I.x, -Vi.x, I.y));
+      const double shape = fma(fma(zz, vmi, zi), vmi, zp);
+      const double f0 = (t != PF_SLACK) ? fma(-pl, shape, pg) - Sc.x : 0.0;
+      const double qgen = (t == kPQLimit) ? w.qsw[i] : S.q_gen[i];
+      const double f1 = (t >= PF_PQ) ? fma(-ql, shape, qgen) - Sc.y : 0.0;
+      if (o.refine > 0) reinterpret_cast<double2*>(w.F)[i] = make_double2(f0, f1);
+      reinterpret_cast<V2*>(y)[r.z] = mk2((TF)f0, (TF)f1);
+      m = max(m, max(abs_bits(f0), abs_bits(f1)));
+      Blk<TF> D;
+      if constexpr (sizeof(TF) == 4) {
+        D = diag_block(S, i, t, Vi, Vi, vmi, I, Sc, pl, ql, __ldg(R.diag32 + rl));
+      } else {
+        D = diag_block(S, i, t, Vi, ld_state<CL>(w.U + i), vmi, I, Sc, pl, ql, yd);
+      }
+      bool ok = true;
+      if (r.x & kResRowLevel0) ok = inv2(D);
+      if (!ok)
+        for (int q = 0; q < P; ++q) *remote(&sh_flag, q) = 1;
+      st_blk(A + 4 * r.y, D);
+    }
+    spread(m, sh_norm);
+    csync<CL>();
+    tick(kProfMismatch);
+
+    // ---- stop test (every thread decides alike) ----
+    const double nrm = widest(sh_norm);
+    status = kRunning;
+    if (!(nrm <= 1e12)) status = PF_ERR_DIVERGED;
+    else if (nrm <= o.tol) status = PF_OK;
+    else if (it >= o.max_iter) status = PF_ERR_MAXITER;
+    if (status != kRunning) {
+      put_info(status, it, passes, nrm, it > 0 ? widest(sh_step) : 0.0);
+      break;
+    }
+    const bool refine = o.refine > 0 && refine_now(o, it, nrm, prev);
+    prev = nrm;
+    tick(kProfStop);
+
+    // ---- factorisation with the forward sweep, backward sweep; refinement ----
+    const int npass = refine ? o.refine : 0;
+    bool singular = false;
+    for (int pass = 0; pass <= npass; ++pass) {
+      if (pass == 0) {
+        run_rounds<kFactor, TF>(tab, part.nrf, R.rec, Ap, yp, ring, &sh_flag);
+      } else {
+        // FP64 residual of the step so far (matrix-free), then another solve
+        rows([&](int i, const int4&) { dv_row<false>(S, w, i, 0); });
+        csync<CL>();
+        rows([&](int i, const int4& r) {
+          resid_row<false>(S, w, i, 0);
+          reinterpret_cast<V2*>(y)[r.z] = mk2((TF)w.r[2 * i], (TF)w.r[2 * i + 1]);
+        });
+        for (int k = part.np + tid; k < part.np + part.nb; k += T)
+          reinterpret_cast<V2*>(yp)[k] = mk2(TF(0), TF(0));
+        __syncthreads();
+        tick(kProfResidual);
+        run_rounds<kForward, TF>(tab + (part.rw - part.rf), part.nrw, R.rec, Ap, yp, ring, &sh_flag);
+      }
+      if constexpr (CL) {
+        csync<CL>();
+        if (pass == 0 && tid == 0 && crank != 0 && sh_flag) *remote(&sh_flag, 0) = 1;
+        if (crank == 0) {
+          // the parts' Schur complements and right-hand sides, in their order
+          const int g0 = pass == 0 ? 0 : R.ngat_blk;
+          for (int k = g0 + tid; k < R.ngat_blk + R.ngat_vec; k += T) {
+            const int4 g = __ldg(R.gat + k);
+            if (k < R.ngat_blk) {
+              Blk<TF> v = ld_blk(At + 4 * g.x);
+              for (int q = g.y; q < g.z; ++q) {
+                const int2 s = __ldg(R.gsrc + q);
+                const Blk<TF> u = ld_blk(remote(A, s.x) + 4 * s.y);
+                v.a += u.a;
+                v.b += u.b;
+                v.c += u.c;
+                v.d += u.d;
+              }
+              if (g.w && !inv2(v)) sh_flag = 1;
+              st_blk(At + 4 * g.x, v);
+            } else {
+              V2 v = reinterpret_cast<V2*>(yt)[g.x];
+              for (int q = g.y; q < g.z; ++q) {
+                const int2 s = __ldg(R.gsrc + q);
+                const V2 u = reinterpret_cast<const V2*>(remote(y, s.x))[s.y];
+                v.x += u.x;
+                v.y += u.y;
+              }
+              reinterpret_cast<V2*>(yt)[g.x] = v;
+            }
+          }
+          __syncthreads();
+          const int2* tt = tab + sc.ntab;
+          if (pass == 0)
+            run_rounds<kFactor, TF>(tt, top.nrf, R.rec, At, yt, ring, &sh_flag);
+          else
+            run_rounds<kForward, TF>(tt + (top.rw - top.rf), top.nrw, R.rec, At, yt, ring, &sh_flag);
+          if (pass == 0) tick(kProfFactor);
+          run_rounds<kBackward, TF>(tt + (top.rb - top.rf), top.nrb, R.rec, At, yt, ring, &sh_flag);
+        }
+        csync<CL>();
+        if (pass == 0) singular = *remote(&sh_flag, 0) != 0;
+        const V2* xt = reinterpret_cast<const V2*>(remote(y, 0)) + top.vec0;
+        for (int k = tid; k < part.nb; k += T)
+          reinterpret_cast<V2*>(yp)[part.np + k] = xt[__ldg(R.bnd + part.bnd + k)];
+        __syncthreads();
+      } else {
+        if (pass == 0) tick(kProfFactor);
+      }
+      run_rounds<kBackward, TF>(tab + (part.rb - part.rf), part.nrb, R.rec, Ap, yp, ring, &sh_flag);
+      if (!CL && pass == 0) singular = sh_flag != 0;
+      ++passes;
+      if (npass > 0)
+        rows([&](int i, const int4& r) {
+          const V2 x = reinterpret_cast<const V2*>(y)[r.z];
+          double2* d = reinterpret_cast<double2*>(w.dx) + i;
+          *d = pass == 0 ? make_double2((double)x.x, (double)x.y)
+                         : make_double2(d->x + (double)x.x, d->y + (double)x.y);
+        });
+      tick(kProfSolve);
+      if (singular) break;
+    }
+    if (singular) {
+      status = PF_ERR_SINGULAR;
+      put_info(status, it, passes - 1, nrm, 0.0);
+      csync<CL>();
+      break;
+    }
+
+    // ---- voltage update ----
+    unsigned long long ms = 0ull;
+    rows([&](int i, const int4& r) {
+      double dd, dm;
+      if (npass > 0) {
+        const double2 q = reinterpret_cast<const double2*>(w.dx)[i];
+        dd = q.x;
+        dm = q.y;
+      } else {
+        const V2 q = reinterpret_cast<const V2*>(y)[r.z];
+        dd = (double)q.x;
+        dm = (double)q.y;
+      }
+      ms = max(ms, max(abs_bits(dd), abs_bits(dm)));
+      const double vm = w.vm[i] + dm, va = w.va[i] + dd;
+      w.vm[i] = vm;
+      w.va[i] = va;
+      double sn, cs;
+      sincos_tab(S.trig, va, &sn, &cs);
+      if (sizeof(TF) == 8) w.U[i] = make_double2(cs, sn);
+      w.V[i] = make_double2(vm * cs, vm * sn);
+    });
+    spread(ms, sh_step);
+    csync<CL>();
+    tick(kProfUpdate);
+  }
+
+  // ---- results in the caller's numbering ----
+  rows([&](int i, const int4&) { output_row<false>(S, w, i, 0, status == PF_OK); });
+  tick(kProfOutput);
+  if (crank == 0) {
+    __syncthreads();
+    if (tid == 0 && w.out_info) w.out_info->solve_us = (double)(global_ns() - t_begin) * 1e-3;
+  }
+}
+
+// Scenario gs of a state laid out [scenario][row].
+__device__ __forceinline__ DevWork scenario_of(DevWork w, int n, int gs) {
+  const size_t r = (size_t)gs * n;
+  w.B = 1;
+  if (w.in_p_load) w.in_p_load += r;
+  if (w.in_q_load) w.in_q_load += r;
+  if (w.in_p_gen) w.in_p_gen += r;
+  if (w.in_vm) w.in_vm += r;
+  if (w.in_va) w.in_va += r;
+  if (w.out_vm) w.out_vm += r;
+  if (w.out_va) w.out_va += r;
+  if (w.out_info) w.out_info += gs;
+  w.spec += 3 * r;
+  w.vm += r;
+  w.va += r;
+  w.V += r;
+  if (w.U) w.U += r;
+  w.dV += r;
+  w.F += 2 * r;
+  w.dx += 2 * r;
+  w.r += 2 * r;
+  if (w.bt) {
+    w.bt += r;
+    w.qsw += r;
+  }
+  return w;
+}
+
+template <typename TF, bool CL>
+__global__ void __launch_bounds__(512)
+    k_resident(DevSys S, DevWork w, DevOpts o, ResDev R, int lin) {
+  const int gs = CL ? blockIdx.x / (int)cg::this_cluster().num_blocks() : blockIdx.x;
+  resident_solve<TF, CL>(S, scenario_of(w, S.n, gs), o, R, lin);
+}
+
+// Several requests of any cases in one launch: cluster b solves desc[list.job[b]]
+// and raises its done flag (as newton_group_kernel).
+template <typename TF, bool CL>
+__global__ void __launch_bounds__(512) k_resident_group(const GroupJob* desc, GroupList list) {
+  const int csize = CL ? (int)cg::this_cluster().num_blocks() : 1;
+  const int crank = CL ? (int)cg::this_cluster().block_rank() : 0;
+  __shared__ GroupJob job;
+  __shared__ ResDev plan;
+  {
+    const GroupJob* src = desc + list.job[blockIdx.x / csize];
+    for (int k = threadIdx.x; k < (int)(sizeof(GroupJob) / 4); k += blockDim.x)
+      reinterpret_cast<unsigned*>(&job)[k] = reinterpret_cast<const unsigned*>(src)[k];
+    __syncthreads();
+    for (int k = threadIdx.x; k < (int)(sizeof(ResDev) / 4); k += blockDim.x)
+      reinterpret_cast<unsigned*>(&plan)[k] = reinterpret_cast<const unsigned*>(job.res)[k];
+  }
+  __syncthreads();
+  resident_solve<TF, CL>(job.S, job.w, job.o, plan, 0);
+  __threadfence_system();
+  csync<CL>();
+  if (crank == 0 && threadIdx.x == 0) {
+    __threadfence_system();
+    *reinterpret_cast<volatile int*>(job.done) = 1;
+  }
+}
+
+template <class Kern>
+cudaError_t configure(Kern kern, bool CL, int P, int threads, size_t smem, int B, cudaStream_t st,
+                      cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr) {
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess && P > 8)
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  cfg.gridDim = dim3(B * P);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  if (CL) {
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = P;
+    attr->val.clusterDim.y = 1;
+    attr->val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+  }
+  return e;
+}
+
+template <typename TF, bool CL>
+cudaError_t launch_res(const DevSys& S, const DevWork& w, const DevOpts& o, const ResDev& R,
+                       size_t smem, int B, int lin, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  const cudaError_t e = configure(k_resident<TF, CL>, CL, R.P, R.threads, smem, B, st, cfg, attr);
+  if (e != cudaSuccess) return e;
+  return cudaLaunchKernelEx(&cfg, k_resident<TF, CL>, S, w, o, R, lin);
+}
+
+template <typename TF, bool CL>
+cudaError_t launch_group(const GroupJob* desc, const GroupList& list, size_t smem, int P, int threads,
+                         cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  const cudaError_t e =
+      configure(k_resident_group<TF, CL>, CL, P, threads, smem, list.n, st, cfg, attr);
+  if (e != cudaSuccess) return e;
+  return cudaLaunchKernelEx(&cfg, k_resident_group<TF, CL>, desc, list);
+}
+
+template <typename TF, bool CL>
+int clusters_of(int P, int threads, size_t smem) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  int num = 0;
+  cudaError_t e = configure(k_resident<TF, CL>, CL, P, threads, smem, 1, nullptr, cfg, attr);
+  if (e == cudaSuccess) {
+    if (CL) {
+      e = cudaOccupancyMaxActiveClusters(&num, k_resident<TF, CL>, &cfg);
+    } else {
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&num, k_resident<TF, CL>, threads, smem);
+    }
+  }
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return 0;
+  }
+  return num;
+}
+
+}  // namespace
+
+cudaError_t launch_resident(bool fp32, const DevSys& S, const DevWork& w, const DevOpts& o,
+                            const ResDev& R, size_t smem, int B, int lin, cudaStream_t st) {
+  if (R.P > 1)
+    return fp32 ? launch_res<float, true>(S, w, o, R, smem, B, lin, st)
+                : launch_res<double, true>(S, w, o, R, smem, B, lin, st);
+  return fp32 ? launch_res<float, false>(S, w, o, R, smem, B, lin, st)
+              : launch_res<double, false>(S, w, o, R, smem, B, lin, st);
+}
+
+cudaError_t launch_resident_group(bool fp32, const GroupJob* desc, const GroupList& list, size_t smem,
+                                  int P, int threads, cudaStream_t st) {
+  if (list.n <= 0 || list.n > kGroupMax) return cudaErrorInvalidValue;
+  if (P > 1)
+    return fp32 ? launch_group<float, true>(desc, list, smem, P, threads, st)
+                : launch_group<double, true>(desc, list, smem, P, threads, st);
+  return fp32 ? launch_group<float, false>(desc, list, smem, P, threads, st)
+              : launch_group<double, false>(desc, list, smem, P, threads, st);
+}
+
+int resident_clusters(bool fp32, int P, int threads, size_t smem) {
+  if (P > 1) return fp32 ? clusters_of<float, true>(P, threads, smem) : clusters_of<double, true>(P, threads, smem);
+  return fp32 ? clusters_of<float, false>(P, threads, smem) : clusters_of<double, false>(P, threads, smem);
+}
+
+}  // namespace pf

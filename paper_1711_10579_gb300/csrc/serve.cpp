@@ -307,8 +307,9 @@ struct Server {
 
   // Stages job k (dispatcher thread, lock not held: it may allocate): its
   // workspace, pinned inputs and descriptor; returns the dynamic shared
-  // memory its solve needs.
-  int stage(int k, size_t* smem) {
+  // memory its solve needs and its resident plan (null: the group kernel of
+  // newton.cuh).
+  int stage(int k, size_t* smem, const ResidentPlan** plan) {
     Job& J = jobs[k];
     Request* r = J.req;
     pf_case c = r->c;
@@ -364,6 +365,10 @@ struct Server {
     g.done = h_done + k;
     h_done[k] = 0;
     *smem = d.y_in_smem ? (size_t)n * bs * tf : 0;
+    // the plan a single solve of the case runs on (built with the case)
+    *plan = kind == PF_SINGLE_PHASE ? c->nr.res_single[fp32 ? 1 : 0] : nullptr;
+    g.res = *plan ? (*plan)->d_dev : nullptr;
+    if (*plan) *smem = (*plan)->smem;
     return PF_OK;
   }
 
@@ -423,36 +428,43 @@ struct Server {
       any = true;
     }
     if (claimed.empty()) return any;
+    // one launch per kernel and launch shape
     struct Group {
       GroupList list;
       size_t smem = 0;
       int bs = 2;
       bool fp32 = true;
       int cluster = 1;
+      int threads = 0;  // resident solves: threads per CTA, else 0
     };
-    Group grp[16];
-    for (Group& g : grp) g.list.n = 0;
+    std::vector<Group> grp;
     std::vector<std::pair<int, int>> failed;  // (job, status)
     lk.unlock();
     for (int k : claimed) {
       Request* r = jobs[k].req;
       size_t smem = 0;
-      const int rc = stage(k, &smem);
+      const ResidentPlan* plan = nullptr;
+      const int rc = stage(k, &smem, &plan);
       if (rc != PF_OK) {
         failed.push_back({k, rc});
         continue;
       }
-      const int tier = size_tier(*r);
-      Group& g = grp[(r->c->bs == 2 ? 0 : 2) + (r->o.precision == PF_MIXED ? 0 : 1) + 4 * tier];
-      g.bs = r->c->bs;
-      g.fp32 = r->o.precision == PF_MIXED;
-      g.cluster = kTierCluster[tier];
-      g.smem = std::max(g.smem, smem);
-      g.list.job[g.list.n++] = k;
+      Group want;
+      want.bs = r->c->bs;
+      want.fp32 = r->o.precision == PF_MIXED;
+      want.cluster = plan ? plan->dev.P : kTierCluster[size_tier(*r)];
+      want.threads = plan ? plan->dev.threads : 0;
+      want.list.n = 0;
+      auto it = std::find_if(grp.begin(), grp.end(), [&](const Group& g) {
+        return g.bs == want.bs && g.fp32 == want.fp32 && g.cluster == want.cluster &&
+               g.threads == want.threads;
+      });
+      if (it == grp.end()) it = grp.insert(grp.end(), want);
+      it->smem = std::max(it->smem, smem);
+      it->list.job[it->list.n++] = k;
     }
     std::string err;
     for (Group& g : grp) {
-      if (g.list.n == 0) continue;
       // the next idle stream (round robin), else the next one
       int sidx = gnext;
       for (int q = 0; q < kGroupStreams; ++q) {
@@ -464,7 +476,9 @@ struct Server {
       }
       gnext = (sidx + 1) % kGroupStreams;
       const cudaError_t e =
-          launch_newton_group(g.bs, g.fp32, h_desc, g.list, g.smem, g.cluster, gst[sidx]);
+          g.threads ? launch_resident_group(g.fp32, h_desc, g.list, g.smem, g.cluster, g.threads,
+                                            gst[sidx])
+                    : launch_newton_group(g.bs, g.fp32, h_desc, g.list, g.smem, g.cluster, gst[sidx]);
       for (int q = 0; q < g.list.n; ++q) {
         if (e == cudaSuccess) jobs[g.list.job[q]].stream = sidx;
         else failed.push_back({g.list.job[q], PF_ERR_CUDA});

@@ -110,6 +110,28 @@ void launch_shape(pf_case c, const pf_opts& o, int B, bool fp32, int* grid, int*
   }
 }
 
+// The resident plan a solve runs on, or null: single-phase Newton-Raphson
+// whose factor fits the shared memory of a cluster, with no explicit shape of
+// the other kernels asked for.
+int resident_plan(pf_case c, const pf_opts& o, int B, RunMode mode, const ResidentPlan** out) {
+  *out = nullptr;
+  if (mode != RunMode::Solve || o.method != PF_NR || c->data.kind != PF_SINGLE_PHASE ||
+      o.block_threads || o.scen_per_cta)
+    return PF_OK;
+  const bool fp32 = o.precision == PF_MIXED;
+  if (B > 1) {
+    std::lock_guard<std::mutex> lk(c->tuned_mu);
+    auto it = c->tuned.find({B, o.method, o.precision});
+    if (it != c->tuned.end() && !it->second[4]) return PF_OK;
+  }
+  if (B == 1 && !o.cluster_size) {
+    *out = c->nr.res_single[fp32 ? 1 : 0];
+    return PF_OK;
+  }
+  const int P = o.cluster_size ? o.cluster_size : resident_batch(c->nr.sym, fp32, B, c->ctx->num_sms);
+  return P ? c->nr.resident_for(c->y, fp32, P, out) : PF_OK;
+}
+
 int run_solve(pf_case c, const pf_opts& o, int B, const double* d_p_load, const double* d_q_load,
               const double* d_p_gen, Workspace* ws, cudaStream_t st, RunMode mode, double* out_vm,
               double* out_va, pf_info* out_info, unsigned long long* prof, const double* d_vm0,
@@ -124,6 +146,9 @@ int run_solve(pf_case c, const pf_opts& o, int B, const double* d_p_load, const 
   SysBuf& sb = nk ? c->nk : c->nr;
   // inspection of the Jacobian reads the factor array as FP64
   const bool fp32 = (o.precision == PF_MIXED) && mode != RunMode::Eval;
+  const ResidentPlan* plan = nullptr;
+  rc = resident_plan(c, o, B, mode, &plan);
+  if (rc != PF_OK) return rc;
   int threads, cluster, S, grid;
   launch_shape(c, o, B, fp32, &grid, &cluster, &threads, &S);
   // a batch of Newton-Raphson solves runs its sweeps in a shape of their own
@@ -142,6 +167,7 @@ int run_solve(pf_case c, const pf_opts& o, int B, const double* d_p_load, const 
   if (rc != PF_OK) return rc;
   DevWork w = ws->w;
   w.B = B;
+  w.by_scen = plan ? 1 : 0;
   if (fp32) w.U = nullptr;  // the mixed-precision Jacobian reads V alone
   w.in_p_load = d_p_load;
   w.in_q_load = d_q_load;
@@ -179,6 +205,12 @@ int run_solve(pf_case c, const pf_opts& o, int B, const double* d_p_load, const 
   d.max_lin = o.gmres_max_iter;
   d.rtol = o.gmres_rtol;
   d.krylov = o.krylov;
+  if (plan) {
+    const cudaError_t e =
+        launch_resident(fp32, sys, w, d, plan->dev, plan->smem, B, B > 1 ? 1 : 0, st);
+    if (e != cudaSuccess) return cuda_error(e, "launching the resident Newton kernel");
+    return PF_OK;
+  }
   // single solves keep the triangular-solve vector in shared memory when it fits
   const size_t tf = fp32 ? 4 : 8;
   d.y_in_smem = 0;
@@ -242,6 +274,10 @@ int run_solve_q(pf_case c, const pf_opts& o, int B, const double* d_p_load, cons
   const DevSys& sys = (nk ? c->nk : c->nr).view;
   DevWork w = ws->w;
   w.B = B;
+  const ResidentPlan* plan = nullptr;
+  rc = resident_plan(c, o, B, RunMode::Solve, &plan);
+  if (rc != PF_OK) return rc;
+  w.by_scen = plan ? 1 : 0;
   const bool three = cd.kind != PF_SINGLE_PHASE;
   int npv = 0;  // buses, or phase slots, that can switch
   for (size_t i = 0; i < cd.bus_type.size(); ++i)
@@ -365,6 +401,8 @@ int solve_noalloc(pf_case c, const pf_opts& o, const double* d_p_load, const dou
   const int threads = noalloc_threads(bs);
   int cluster = o.cluster_size;
   if (!cluster) cluster = max_cluster(bs, fp32, false, threads);
+  // the resident plan uploaded when the case was created
+  const ResidentPlan* plan = o.cluster_size ? nullptr : c->nr.res_single[fp32 ? 1 : 0];
   // the lane tables of this launch shape, uploaded when the case was created
   DevSys sys;
   rc = c->nr.lanes_cached(threads, 1, sys);
@@ -452,7 +490,12 @@ int solve_noalloc(pf_case c, const pf_opts& o, const double* d_p_load, const dou
   d.max_lin = o.gmres_max_iter;
   d.rtol = o.gmres_rtol;
   d.y_in_smem = ((size_t)n * bs * tf <= 200 * 1024) ? 1 : 0;
-  e = launch_newton(bs, fp32, false, sys, w, d, cluster, cluster, threads, st);
+  if (plan) {
+    w.by_scen = 1;
+    e = launch_resident(fp32, sys, w, d, plan->dev, plan->smem, 1, 0, st);
+  } else {
+    e = launch_newton(bs, fp32, false, sys, w, d, cluster, cluster, threads, st);
+  }
   if (e != cudaSuccess) return cuda_error(e, "launching the Newton kernel");
   return PF_OK;
 }
@@ -535,11 +578,44 @@ int autotune(pf_case c, int B, pf_opts* io) {
   if (rc != PF_OK) return rc;
   {
     std::lock_guard<std::mutex> lk(c->tuned_mu);
-    c->tuned[{B, o.method, o.precision}] = {bestS, bestT, bestS_s, bestT_s};
+    c->tuned[{B, o.method, o.precision}] = {bestS, bestT, bestS_s, bestT_s, 0};
   }
   io->scen_per_cta = bestS;
   io->block_threads = bestT;
-  return PF_OK;
+  // the phase kernels in those shapes against the resident solves
+  pf_opts t = o;
+  t.scen_per_cta = t.block_threads = 0;
+  const ResidentPlan* plan = nullptr;
+  const int P = nr && c->data.kind == PF_SINGLE_PHASE
+                    ? resident_batch(c->nr.sym, o.precision == PF_MIXED, B, c->ctx->num_sms)
+                    : 0;
+  if (P) rc = c->nr.resident_for(c->y, o.precision == PF_MIXED, P, &plan);
+  if (rc != PF_OK || !plan) return rc;
+  float ms[2] = {1e30f, 1e30f};
+  e = cudaEventCreate(&e0);
+  if (e == cudaSuccess) e = cudaEventCreate(&e1);
+  for (int k = 0; k < 4 && rc == PF_OK && e == cudaSuccess; ++k) {
+    {
+      std::lock_guard<std::mutex> lk(c->tuned_mu);
+      c->tuned[{B, o.method, o.precision}][4] = k & 1;
+    }
+    e = cudaEventRecord(e0, st);
+    if (e == cudaSuccess)
+      rc = run_solve(c, t, B, nullptr, nullptr, nullptr, ws, st, RunMode::Solve, nullptr, nullptr);
+    if (rc == PF_OK && e == cudaSuccess) e = cudaEventRecord(e1, st);
+    if (rc == PF_OK && e == cudaSuccess) e = cudaEventSynchronize(e1);
+    if (rc == PF_OK && e == cudaSuccess) e = cudaEventElapsedTime(&ms[k & 1], e0, e1);
+  }
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+  if (rc == PF_OK && e != cudaSuccess) rc = cuda_error(e, "timing the resident solves");
+  const bool resident = rc == PF_OK && ms[1] < ms[0];
+  {
+    std::lock_guard<std::mutex> lk(c->tuned_mu);
+    c->tuned[{B, o.method, o.precision}][4] = resident ? 1 : 0;
+  }
+  if (resident) io->scen_per_cta = io->block_threads = 0;  // the stored choice
+  return rc;
 }
 
 int profile_solve(pf_case c, int B, const pf_opts& o, double* phase_us, pf_info* info) {

@@ -1,0 +1,152 @@
+"""Resident solves (csrc/resident.cpp, csrc/resident.cu): the host schedule
+executed on the CPU, and the kernels against the FP64 oracle at the sizes
+where the cut into CTAs, the groups of 32 rows and the rounds have edges."""
+import ctypes as C
+import dataclasses
+import os
+import subprocess
+import tempfile
+
+import numpy as np
+import pytest
+
+from oracle import pf_oracle as O
+from paper_1711_10579_gb300 import build, cases
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+CSRC = os.path.join(os.path.dirname(HERE), "paper_1711_10579_gb300", "csrc")
+
+
+def mesh(n, seed=1):
+    if n == 1:
+        return dataclasses.replace(
+            cases.two_bus_case(0.0, 0.0, 0.1, 0.1), n_bus=1, br_from=np.zeros(0, np.int32),
+            br_to=np.zeros(0, np.int32), br_r=np.zeros(0), br_x=np.zeros(0), br_b=np.zeros(0),
+            **{k: getattr(cases.two_bus_case(0.0, 0.0, 0.1, 0.1), k)[:1] for k in
+               ("bus_type", "v_set", "p_gen", "q_gen", "p_load", "q_load", "zip")})
+    if n == 2:
+        return cases.two_bus_case(0.9, 0.3, 0.02, 0.15)
+    m = max(n - 1, int(1.35 * n)) if n > 4 else n - 1
+    return cases.transmission_case(n, m, max(1, n // 5), seed, max_angle=0.06)
+
+
+# ----------------------------------------------------------------------------
+# the schedule, on the CPU
+# ----------------------------------------------------------------------------
+
+@pytest.fixture(scope="module")
+def host():
+    so = os.path.join(tempfile.mkdtemp(prefix="resident"), "resident_host.so")
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-shared", "-fPIC",
+                           "-I", os.path.join(build._cuda_home(), "include"), "-o", so,
+                           os.path.join(HERE, "resident_host.cpp"),
+                           os.path.join(CSRC, "resident.cpp"), os.path.join(CSRC, "symbolic.cpp")])
+    return C.CDLL(so)
+
+
+@pytest.mark.parametrize("P,threads", [(1, 32), (1, 512), (2, 64), (4, 128), (16, 512)])
+@pytest.mark.parametrize("n", [1, 2, 3, 14, 33, 300, 2000])
+def test_schedule_solves_the_system(host, n, P, threads):
+    """Residuals of a diagonally dominant random system in FP64: a few ulps of
+    the entries times the row length."""
+    g = mesh(n)
+    f, t = (np.ascontiguousarray(a, np.int32) for a in (g.br_from, g.br_to))
+    err, parts = C.c_double(-1.0), C.c_int(0)
+    rc = host.resident_check(n, len(f), f.ctypes.data_as(C.c_void_p), t.ctypes.data_as(C.c_void_p),
+                             P, threads, C.byref(err), C.byref(parts))
+    assert rc == 0
+    assert 0.0 <= err.value <= 1e-13
+    if n == 2000 and P > 1:
+        assert parts.value == P + 1  # every CTA has its own subtrees, and there is a top
+
+
+def test_schedule_of_a_tree_and_of_a_star(host):
+    feeder = cases.feeder_case(700, 3)
+    star = (np.zeros(299, np.int32), np.arange(1, 300, dtype=np.int32))
+    for f, t, n in ((feeder.br_from, feeder.br_to, 700), (*star, 300)):
+        f, t = (np.ascontiguousarray(a, np.int32) for a in (f, t))
+        for P in (1, 4):
+            err, parts = C.c_double(-1.0), C.c_int(0)
+            assert host.resident_check(n, len(f), f.ctypes.data_as(C.c_void_p),
+                                       t.ctypes.data_as(C.c_void_p), P, 128, C.byref(err),
+                                       C.byref(parts)) == 0
+            assert 0.0 <= err.value <= 1e-13
+
+
+# ----------------------------------------------------------------------------
+# the kernels
+# ----------------------------------------------------------------------------
+
+@pytest.fixture(scope="module")
+def env():
+    import __graft_entry__
+
+    __graft_entry__.build()
+    from paper_1711_10579_gb300 import pf
+
+    ctx = pf.pf_ctx_create(0)
+    yield pf, ctx
+    pf.pf_ctx_destroy(ctx)
+
+
+def _loads(case, B, seed):
+    if case.n_bus <= 2:
+        s = np.linspace(1.0, 0.5, B)[:, None]
+        return case.p_load[None] * s, case.q_load[None] * s, np.repeat(case.p_gen[None], B, 0)
+    return cases.scenario_loads(case, B, seed=seed)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+@pytest.mark.parametrize("n,P", [(1, 1), (2, 1), (3, 2), (14, 1), (31, 1), (33, 4), (129, 2), (500, 1),
+                                 (500, 16), (2000, 8)])
+def test_resident_matches_oracle(env, n, P, prec):
+    """Single solves and a ragged batch on P CTAs, ZIP loads and a PQ bus with
+    generation among them, with and without FP64 refinement: within 1e-6 of
+    the oracle's solution, as every solve (the stop test's mismatch of 1e-8)."""
+    pf, ctx = env
+    case = mesh(n)
+    if n > 2:
+        zipf = np.tile([1.0, 0.0, 0.0], (n, 1))
+        zipf[1::2] = [0.4, 0.35, 0.25]
+        qg = np.zeros(n)
+        qg[np.flatnonzero(case.bus_type == cases.PQ)[0]] = 1e-3
+        case = dataclasses.replace(case, zip=zipf, q_gen=qg)
+    pl, ql, pg = _loads(case, 3, seed=5)
+    refs = [O.newton_polar(case.with_loads(pl[b], ql[b], pg[b])) if n > 1 else
+            {"vm": case.v_set, "va": np.zeros(1)} for b in range(3)]
+    c = pf.pf_create_case(ctx, case)
+    try:
+        for rs in (0.1, 0.0):
+            o = pf.make_opts(precision=pf.PF_FP64 if prec == "fp64" else pf.PF_MIXED,
+                             cluster_size=P, refine_stall=rs)
+            shape = pf.pf_launch_config(c, o, 3)
+            assert shape["cluster"] == P and shape["grid"] == 3 * P
+            vm, va, info = pf.pf_solve_batch(c, pl, ql, pg, o)
+            vm1, va1, info1 = pf.pf_solve_batch(c, pl[:1], ql[:1], pg[:1], o)
+            assert np.all(info["status"] == 0) and np.all(info["mismatch"] <= 1e-8)
+            # the same launch shape: the scenario alone is the same bit for bit
+            assert np.array_equal(vm[0], vm1[0]) and np.array_equal(va[0], va1[0])
+            assert np.all(info["linear_iterations"] >= info["iterations"])
+            for b, r in enumerate(refs):
+                assert np.max(np.abs(vm[b] - r["vm"])) <= 1e-6
+                assert np.max(np.abs(va[b] - r["va"])) <= 1e-6
+    finally:
+        pf.pf_destroy_case(c)
+
+
+@pytest.mark.gpu
+def test_resident_reports_failures(env):
+    """A scenario past the loading nose next to one that converges, and an
+    iteration limit."""
+    pf, ctx = env
+    case = cases.two_bus_case(50.0, 20.0, 0.02, 0.15)
+    c = pf.pf_create_case(ctx, case)
+    pl = np.array([[0.0, 50.0], [0.0, 0.9]])
+    ql = np.array([[0.0, 20.0], [0.0, 0.3]])
+    _, _, info = pf.pf_solve_batch(c, pl, ql, None, pf.make_opts(max_iter=20))
+    assert info["status"][0] in (pf.PF_ERR_MAXITER, pf.PF_ERR_DIVERGED, pf.PF_ERR_SINGULAR)
+    assert info["status"][1] == 0
+    _, _, info = pf.pf_solve_batch(c, pl, ql, None, pf.make_opts(max_iter=0))
+    assert np.all(info["status"] == pf.PF_ERR_MAXITER) and np.all(info["iterations"] == 0)
+    pf.pf_destroy_case(c)
