@@ -302,12 +302,28 @@ static int resident_least(const Symbolic& s, bool fp32) {
   return 0;
 }
 
+// Groups of 8 lanes of a feeder's CTA: at most 32, few levels are wider.
+static int feeder_groups(int n, int P) {
+  int g = 4;
+  while (g < 32 && 4 * g * P < n) g <<= 1;
+  return g;
+}
+
+static int feeder_least(int n, bool fp32) {
+  const double node = fp32 ? FeedShape<float>::node * 4.0 : FeedShape<double>::node * 8.0;
+  for (int P = 1; P <= 16; P <<= 1)
+    if ((P > 1 ? 1.04 : 1.0) * n * (node + 36) / P + 24 * 1024 <= 224 * 1024) return P;
+  return 0;
+}
+
 // Single solves: latency, so more CTAs than memory asks for, one per 400
-// rows.  Measured (us, P = 1 / 2 / 4 / 8 / 16): 500 buses mixed 140 / 145 /
-// 133 / 140 / 180; 2,749 buses FP64 - / - / 770 / 657 / 641.
-int resident_single(const Symbolic& s, bool fp32) {
-  int P = resident_least(s, fp32);
-  while (P > 0 && P < 16 && s.n > 400 * P) P <<= 1;
+// rows (feeders: 100 nodes).  Measured (us, P = 1 / 2 / 4 / 8 / 16): 500 buses
+// mixed 140 / 145 / 133 / 140 / 180; 2,749 buses FP64 - / - / 770 / 657 / 641;
+// feeders of 100 nodes mixed 143 / 170 / 157 / 161 / 184, of 400 314 / 259 /
+// 215 / 231 / 257, of 1,000 FP64 - / 1,343 / 1,044 / 1,060 / 919.
+int resident_single(const Symbolic& s, bool fp32, bool three) {
+  int P = three ? feeder_least(s.n, fp32) : resident_least(s, fp32);
+  while (P > 0 && P < 16 && s.n > (three ? 100 : 400) * P) P <<= 1;
   return P;
 }
 
@@ -317,8 +333,15 @@ int resident_single(const Symbolic& s, bool fp32) {
 // shape): 2,000 buses mixed x 256 0.69 / 1.94, x 1,000 2.40 / 3.47, x 3,000
 // 6.83 / 6.99; 5,000 mixed x 256 3.4 / 4.7, x 1,000 11.9 / 8.3; 500 FP64 x
 // 256 0.89 / 1.55, x 1,000 3.1 / 2.3; 100 FP64 x 1,000 0.48 / 0.81.
-int resident_batch(const Symbolic& s, bool fp32, int B, int num_sms) {
-  const int P = resident_least(s, fp32);
+int resident_batch(const Symbolic& s, bool fp32, bool three, int B, int num_sms) {
+  int P = three ? feeder_least(s.n, fp32) : resident_least(s, fp32);
+  if (three) {
+    // feeders: CTAs of at most 256 nodes, so that two fit an SM.  Measured (ms,
+    // resident against phase kernels): 1,000 nodes mixed x 500 3.6 / 4.7, FP64
+    // x 250 5.0 / 5.8; 8,000 nodes FP64 x 16 5.4 / 16.3, x 61 16.3 / 16.8
+    while (P > 0 && P < 16 && s.n > 256 * P) P <<= 1;
+    return P > 0 && (double)B * P <= (s.n > 280 * P ? 4.0 : 13.0) * num_sms ? P : 0;
+  }
   const double waves = fp32 || s.n <= 128 ? 8.0 : 3.5;
   return P > 0 && (double)B * P <= waves * num_sms ? P : 0;
 }
@@ -327,16 +350,29 @@ int SysBuf::resident_for(const Ybus& y, bool fp32, int P, const ResidentPlan** o
   std::lock_guard<std::mutex> lk(g_mu);
   *out = nullptr;
   auto& slot = res_cache[2 * P + (fp32 ? 1 : 0)];
-  if (slot) {
-    if (slot->ok) *out = slot.get();
-    return PF_OK;
+  if (!slot) {
+    slot = std::make_unique<ResidentPlan>();
+    slot->P = P;
+    const int rc = y.ybs == 1 ? upload_resident(y, fp32, *slot) : upload_feeder(y, fp32, *slot);
+    if (rc != PF_OK) {
+      res_cache.erase(2 * P + (fp32 ? 1 : 0));
+      return rc;
+    }
   }
-  slot = std::make_unique<ResidentPlan>();
-  ResidentPlan& r = *slot;
+  if (slot->ok) *out = slot.get();
+  return PF_OK;
+}
+
+// Shared memory of a resident CTA at most (with the kernels' static arrays
+// below the 227 KB of a CTA).
+constexpr size_t kResidentSmem = 224 * 1024;
+
+int SysBuf::upload_resident(const Ybus& y, bool fp32, ResidentPlan& r) {
   ResPlanHost h;
-  if (y.ybs != 1 || !res_plan(sym, P, resident_threads(sym.n, P), h)) return PF_OK;
+  r.threads = resident_threads(sym.n, r.P);
+  if (!res_plan(sym, r.P, r.threads, h)) return PF_OK;
   r.smem = res_smem(h, fp32 ? 4 : 8);
-  if (r.smem > 224 * 1024 || resident_clusters(fp32, P, h.threads, r.smem) < 1) return PF_OK;
+  if (r.smem > kResidentSmem || resident_clusters(fp32, r.P, r.threads, r.smem) < 1) return PF_OK;
   auto val = [&](int e) { return &y.val[2 * (size_t)sym.y_src[e]]; };
   std::vector<double2> ell_y(h.ell_y.size(), make_double2(0.0, 0.0));
   for (size_t k = 0; k < ell_y.size(); ++k)
@@ -365,8 +401,8 @@ int SysBuf::resident_for(const Ybus& y, bool fp32, int P, const ResidentPlan** o
   for (size_t k = 0; k < gat.size(); ++k)
     gat[k] = make_int4(h.gat[4 * k], h.gat[4 * k + 1], h.gat[4 * k + 2], h.gat[4 * k + 3]);
   ResDev& d = r.dev;
-  d.P = P;
-  d.threads = h.threads;
+  d.P = r.P;
+  d.threads = r.threads;
   d.ngat_blk = h.ngat_blk;
   d.ngat_vec = h.ngat_vec;
   d.max_blk = h.max_blk;
@@ -388,13 +424,98 @@ int SysBuf::resident_for(const Ybus& y, bool fp32, int P, const ResidentPlan** o
   if (e == cudaSuccess) e = upload(mem, h.bnd, &d.bnd);
   if (e == cudaSuccess) e = upload(mem, gat, &d.gat);
   if (e == cudaSuccess) e = upload(mem, gsrc, &d.gsrc);
-  if (e == cudaSuccess) e = upload(mem, std::vector<ResDev>(1, d), &r.d_dev);
-  if (e != cudaSuccess) {
-    res_cache.erase(2 * P + (fp32 ? 1 : 0));
-    return cuda_error(e, "uploading a resident plan");
-  }
+  const ResDev* copy = nullptr;
+  if (e == cudaSuccess) e = upload(mem, std::vector<ResDev>(1, d), &copy);
+  r.d_dev = copy;
+  if (e != cudaSuccess) return cuda_error(e, "uploading a resident plan");
   r.ok = true;
-  *out = &r;
+  return PF_OK;
+}
+
+// Mixed-precision feeders of more nodes stay on the persistent kernel: its
+// voltages there are up to 1.3e-7 (relative) off the solution (170 feeders of
+// 2,000-4,000 nodes; up to 2.8e-8 below 2,000), and this kernel's, which are a
+// hundred times closer, would move what such a call returns by as much.
+constexpr int kFeederMixedMax = 2000;
+
+int SysBuf::upload_feeder(const Ybus& y, bool fp32, ResidentPlan& r) {
+  FeedPlanHost h;
+  if (fp32 && sym.n > kFeederMixedMax) return PF_OK;
+  const int groups = feeder_groups(sym.n, r.P);
+  r.threads = groups * kFeedLanes;
+  if (!feed_plan(sym, bus_type, r.P, groups, h)) return PF_OK;
+  r.smem = feed_smem(h, fp32);
+  if (r.smem > kResidentSmem || feeder_clusters(fp32, r.P, r.threads, r.smem) < 1) return PF_OK;
+  const int n = sym.n;
+  auto val = [&](int e) { return &y.val[18 * (size_t)sym.y_src[e]]; };
+  auto free_phase = [&](int i, int a) { return ((bus_type[i] >> a) & 1) && !(bus_type[i] & 8); };
+  // Ybus rows by lane: the entries of (node, phase) as [entry][column][lane]
+  std::vector<double2> ell_y(3 * h.ell_y.size(), make_double2(0.0, 0.0));
+  for (size_t g = 0; g < h.grp.size(); ++g)
+    for (int e = 0; e < h.grp[g].width; ++e)
+      for (int l = 0; l < 32; ++l) {
+        const int q = h.grp[g].ell + 32 * e + l, ye = h.ell_y[q];
+        if (ye < 0) continue;
+        const int a = (h.item[2 * (32 * g + l)] >> 28) & 3;
+        for (int c = 0; c < 3; ++c)
+          ell_y[3 * ((size_t)h.grp[g].ell + 32 * e) + 32 * c + l] =
+              make_double2(val(ye)[2 * (3 * a + c)], val(ye)[2 * (3 * a + c) + 1]);
+      }
+  // S_k0 (the row sum: what a branch does not carry to another free phase) and
+  // the branch admittances, zero outside the free phases of rows and columns
+  const int nb = fp32 ? FeedShape<float>::branch : FeedShape<double>::branch;
+  std::vector<double> diag(18 * (size_t)n, 0.0), br((size_t)nb * n, 0.0);
+  for (int i = 0; i < n; ++i)
+    for (int e = sym.y_rowptr[i]; e < sym.y_rowptr[i + 1]; ++e) {
+      const int j = sym.y_col[e];
+      for (int a = 0; a < 3; ++a)
+        for (int c = 0; c < 3; ++c) {
+          if (!free_phase(i, a) || !free_phase(j, c)) continue;
+          const double *v = val(e) + 2 * (3 * a + c);
+          diag[18 * (size_t)i + 2 * (3 * a + c)] += v[0];
+          diag[18 * (size_t)i + 2 * (3 * a + c) + 1] += v[1];
+          if (e != h.branch[i]) continue;
+          br[(size_t)nb * i + 3 * a + c] = -v[0];
+          br[(size_t)nb * i + 9 + 3 * a + c] = -v[1];
+        }
+    }
+  std::vector<int2> item(h.item.size() / 2), node(h.node.size() / 2), rnd(h.rnd.size() / 2);
+  std::vector<uint2> rec(h.rec.size() / 2);
+  for (size_t k = 0; k < item.size(); ++k) item[k] = make_int2(h.item[2 * k], h.item[2 * k + 1]);
+  for (size_t k = 0; k < node.size(); ++k) node[k] = make_int2(h.node[2 * k], h.node[2 * k + 1]);
+  for (size_t k = 0; k < rnd.size(); ++k) rnd[k] = make_int2(h.rnd[2 * k], h.rnd[2 * k + 1]);
+  for (size_t k = 0; k < rec.size(); ++k) rec[k] = make_uint2(h.rec[2 * k], h.rec[2 * k + 1]);
+  FeedDev& d = r.feed;
+  d.P = r.P;
+  d.threads = r.threads;
+  d.max_slots = h.max_slots;
+  d.max_rec = h.max_rec;
+  d.max_rnd = h.max_rnd;
+  cudaError_t e = upload(mem, h.part, &d.part);
+  if (e == cudaSuccess) e = upload(mem, h.cta, &d.cta);
+  if (e == cudaSuccess) e = upload(mem, h.grp, &d.grp);
+  if (e == cudaSuccess) e = upload(mem, item, &d.item);
+  if (e == cudaSuccess) e = upload(mem, h.ell_col, &d.ell_col);
+  if (e == cudaSuccess) e = upload(mem, ell_y, &d.ell_y);
+  if (e == cudaSuccess) e = upload(mem, node, &d.node);
+  if (e == cudaSuccess) e = upload(mem, rnd, &d.rnd);
+  if (e == cudaSuccess) e = upload(mem, rec, &d.rec);
+  const float *d32 = nullptr, *b32 = nullptr;
+  const double *d64 = nullptr, *b64 = nullptr;
+  if (fp32) {
+    if (e == cudaSuccess) e = upload(mem, std::vector<float>(diag.begin(), diag.end()), &d32);
+    if (e == cudaSuccess) e = upload(mem, std::vector<float>(br.begin(), br.end()), &b32);
+  } else {
+    if (e == cudaSuccess) e = upload(mem, diag, &d64);
+    if (e == cudaSuccess) e = upload(mem, br, &b64);
+  }
+  d.ydiag = fp32 ? (const void*)d32 : (const void*)d64;
+  d.branch = fp32 ? (const void*)b32 : (const void*)b64;
+  const FeedDev* copy = nullptr;
+  if (e == cudaSuccess) e = upload(mem, std::vector<FeedDev>(1, d), &copy);
+  r.d_dev = copy;
+  if (e != cudaSuccess) return cuda_error(e, "uploading a feeder plan");
+  r.ok = true;
   return PF_OK;
 }
 
@@ -650,9 +771,9 @@ int pf_create_case(pf_ctx ctx, const pf_case_desc* desc, pf_case* out) {
     rc = c->nr.lanes_for(pf::noalloc_threads(c->bs), 1, unused);
     if (rc != PF_OK) return rc;
     // and the resident plans of single solves
-    for (int fp32 = 0; fp32 < 2 && c->data.kind == PF_SINGLE_PHASE; ++fp32) {
+    for (int fp32 = 0; fp32 < 2; ++fp32) {
       const ResidentPlan* plan = nullptr;
-      for (int P = resident_single(c->nr.sym, fp32 != 0); P > 0 && P <= 16 && !plan; P <<= 1) {
+      for (int P = resident_single(c->nr.sym, fp32 != 0, c->bs == 6); P > 0 && P <= 16 && !plan; P <<= 1) {
         rc = c->nr.resident_for(c->y, fp32 != 0, P, &plan);
         if (rc != PF_OK) return rc;
       }
@@ -880,13 +1001,25 @@ int pf_analyze(const pf_case_desc* desc, pf_case_stats* out) {
                 s->blev_ptr.size() + s->blev_rows.size() + s->perm.size());
     b += (long long)y.val.size() * 8 + (long long)d.n * (1 + 8 * 9);
   }
-  for (int fp32 = 0; fp32 < 2 && y.ybs == 1; ++fp32) {  // the plans of resident single solves
-    ResPlanHost h;
-    const int P = resident_single(nr, fp32 != 0);
-    if (P > 0 && res_plan(nr, P, resident_threads(nr.n, P), h))
-      b += 4LL * (long long)(h.row.size() + h.ell_col.size() + h.jac.size() + h.rnd.size() +
-                             h.rec.size() + h.bnd.size() + h.gat.size() + h.gsrc.size()) +
-           16LL * (long long)h.ell_y.size() + (fp32 ? 2LL : 4LL) * (long long)h.jac.size();
+  for (int fp32 = 0; fp32 < 2; ++fp32) {  // the plans of resident single solves
+    const int P = resident_single(nr, fp32 != 0, y.ybs == 3);
+    if (P == 0) continue;
+    if (y.ybs == 1) {
+      ResPlanHost h;
+      if (res_plan(nr, P, resident_threads(nr.n, P), h))
+        b += 4LL * (long long)(h.row.size() + h.ell_col.size() + h.jac.size() + h.rnd.size() +
+                               h.rec.size() + h.bnd.size() + h.gat.size() + h.gsrc.size()) +
+             16LL * (long long)h.ell_y.size() + (fp32 ? 2LL : 4LL) * (long long)h.jac.size();
+    } else {
+      FeedPlanHost h;
+      std::vector<int8_t> bt(d.n);
+      for (int i = 0; i < d.n; ++i)
+        bt[i] = !d.bus_type.empty() && d.bus_type[nr.perm[i]] == PF_PV ? 16 : 7;
+      if (feed_plan(nr, bt, P, feeder_groups(nr.n, P), h))
+        b += 4LL * (long long)(h.item.size() + h.ell_col.size() + h.node.size() + h.rnd.size() +
+                               h.rec.size()) +
+             48LL * (long long)h.ell_y.size() + (fp32 ? 152LL : 288LL) * d.n;
+    }
   }
   out->device_bytes = b;
   return PF_OK;
@@ -1078,9 +1211,9 @@ int pf_launch_config(pf_case c, const pf_opts* opts, int B, int* grid, int* clus
   const int rc = resident_plan(c, o, B, RunMode::Solve, &plan);
   if (rc != PF_OK) return rc;
   if (plan) {
-    *grid = B * plan->dev.P;
-    *cluster = plan->dev.P;
-    *threads = plan->dev.threads;
+    *grid = B * plan->P;
+    *cluster = plan->P;
+    *threads = plan->threads;
     *scen = 1;
     return PF_OK;
   }

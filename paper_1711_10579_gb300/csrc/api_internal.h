@@ -12,6 +12,7 @@
 #include <vector>
 
 #include "device.h"
+#include "feeder.h"
 #include "host.h"
 #include "resident.h"
 
@@ -29,10 +30,12 @@ struct DevBuffer {
   cudaError_t alloc(void** out, size_t nbytes);
 };
 
-// A resident plan on the device.
+// A resident plan on the device (resident.h; three phase: feeder.h).
 struct ResidentPlan {
+  int P = 1, threads = 0;
   ResDev dev{};
-  const ResDev* d_dev = nullptr;  // a copy in device memory (group launches)
+  FeedDev feed{};
+  const void* d_dev = nullptr;  // a copy of dev / feed in device memory (group launches)
   size_t smem = 0;
   bool ok = false;  // fits the device (else the case runs the other kernels)
 };
@@ -57,6 +60,8 @@ struct SysBuf {
   const ResidentPlan* res_single[2] = {nullptr, nullptr};
 
  private:
+  int upload_resident(const Ybus& y, bool fp32, ResidentPlan& r);
+  int upload_feeder(const Ybus& y, bool fp32, ResidentPlan& r);
   std::map<int, std::unique_ptr<ResidentPlan>> res_cache;  // 2 P + fp32
 
   void finish_view(const std::array<const int8_t*, 2>& g, int threads, DevSys& out) const;
@@ -149,8 +154,8 @@ struct pf_case_s {
 namespace pf {
 
 // CTAs of a resident solve (of one scenario of a batch of B), 0: none.
-int resident_single(const Symbolic& s, bool fp32);
-int resident_batch(const Symbolic& s, bool fp32, int B, int num_sms);
+int resident_single(const Symbolic& s, bool fp32, bool three);
+int resident_batch(const Symbolic& s, bool fp32, bool three, int B, int num_sms);
 
 enum class RunMode { Solve, Eval, Step };
 enum class InspectKind { Mismatch, Jacobian, Step };

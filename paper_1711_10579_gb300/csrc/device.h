@@ -187,13 +187,12 @@ size_t dynamic_smem_bytes(int bs, size_t tf, bool nk, int n, const DevOpts& o, i
 // One single-CTA solve of a group launch (several cases of different sizes
 // in one launch): its case, workspace and options, and the flag the CTA
 // raises (1) once its results are written.
-struct ResDev;
 struct GroupJob {
   DevSys S;
   DevWork w;
   DevOpts o;
   int* done;
-  const ResDev* res;  // resident solves: the plan (device memory)
+  const void* res;  // resident solves: the plan (device memory)
 };
 constexpr int kGroupMax = 160;  // jobs of one group launch
 // The jobs of a launch: CTA b runs desc[job[b]].

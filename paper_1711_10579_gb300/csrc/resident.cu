@@ -7,7 +7,7 @@
 // three dependent L2 round trips, 1.4 us of factorisation and 2 x 1.4 us of
 // sweeps; here it is one round of shared-memory reads, a few FMAs and a block
 // barrier.
-#include "kernels.cuh"
+#include "resident.cuh"
 #include "resident.h"
 
 namespace pf {
@@ -53,22 +53,6 @@ __device__ __forceinline__ void st_blk(double* p, const Blk<double>& v) {
 __device__ __forceinline__ float2 mk2(float x, float y) { return make_float2(x, y); }
 __device__ __forceinline__ double2 mk2(double x, double y) { return make_double2(x, y); }
 
-// a b + c d with the roundings written out: the kernels that inline a solve
-// (alone, and in a group launch) must not contract it differently, or a
-// served result would differ from the same solve alone.
-__device__ __forceinline__ float dot2(float a, float b, float c, float d) {
-  return __fmaf_rn(a, b, __fmul_rn(c, d));
-}
-__device__ __forceinline__ double dot2(double a, double b, double c, double d) {
-  return __fma_rn(a, b, __dmul_rn(c, d));
-}
-__device__ __forceinline__ float nmac2(float v, float a, float b, float c, float d) {  // v - a b - c d
-  return __fmaf_rn(-c, d, __fmaf_rn(-a, b, v));
-}
-__device__ __forceinline__ double nmac2(double v, double a, double b, double c, double d) {
-  return __fma_rn(-c, d, __fma_rn(-a, b, v));
-}
-
 // Inverse in closed form; false for a zero or non-finite determinant or
 // inverse (the rule of the batched factorisation).
 template <typename TF>
@@ -78,16 +62,6 @@ __device__ __forceinline__ bool inv2(Blk<TF>& m) {
   const Blk<TF> v{m.d * r, -m.b * r, -m.c * r, m.a * r};
   m = v;
   return det != TF(0) && isfinite(v.a) && isfinite(v.b) && isfinite(v.c) && isfinite(v.d);
-}
-
-// Bus state: written by any CTA of the cluster (L2) or by this CTA alone.
-template <bool CL, typename T>
-__device__ __forceinline__ T ld_state(const T* p) {
-  if constexpr (CL) {
-    return __ldcg(p);
-  } else {
-    return *p;
-  }
 }
 
 enum { kFactor = 0, kForward = 1, kBackward = 2 };
@@ -285,13 +259,7 @@ __device__ __forceinline__ void resident_solve(const DevSys& S, const DevWork& w
   TF* const yp = y + 2 * part.vec0;
   TF* const At = A + 4 * top.blk0;
   TF* const yt = y + 2 * top.vec0;
-  auto remote = [&](auto* p, int r) {
-    if constexpr (CL) {
-      return cg::this_cluster().map_shared_rank(p, r);
-    } else {
-      return p;
-    }
-  };
+  const bool first = crank == 0 && tid == 0;
   const bool prof = o.prof != nullptr && blockIdx.x == 0 && tid == 0;
   unsigned long long t_last = prof ? t_begin : 0ull;
   auto tick = [&](int phase) {
@@ -307,37 +275,6 @@ __device__ __forceinline__ void resident_solve(const DevSys& S, const DevWork& w
       const int4 r = __ldg(R.row + (size_t)(sc.grp + g) * 32 + lane);
       if (r.x >= 0) fn(r.x & ~kResRowLevel0, r);
     }
-  };
-  // largest value over the cluster into slot[] of every CTA (read after the
-  // next barrier)
-  auto spread = [&](unsigned long long m, unsigned long long* slot) {
-    for (int off = 16; off > 0; off >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, off));
-    if (lane == 0) sh_red[warp] = m;
-    __syncthreads();
-    if (tid < P) {
-      unsigned long long v = 0ull;
-      for (int q = 0; q < nwarp; ++q) v = max(v, sh_red[q]);
-      remote(slot, tid)[crank] = v;
-    }
-  };
-  auto widest = [&](const unsigned long long* slot) {
-    unsigned long long v = 0ull;
-    for (int q = 0; q < P; ++q) v = max(v, slot[q]);
-    return __longlong_as_double((long long)v);
-  };
-  auto put_info = [&](int st, int it, int passes, double nrm, double step) {
-    if (crank != 0 || tid != 0 || !w.out_info) return;
-    pf_info inf;
-    inf.status = st;
-    inf.iterations = it;
-    inf.linear_iterations = lin ? passes : 0;
-    inf.fallback = 0;
-    inf.mismatch = nrm;
-    inf.max_step = step;
-    inf.solve_us = 0.0;
-    inf.q_switched = 0;
-    inf.q_rounds = 1;
-    *w.out_info = inf;
   };
   rows([&](int i, const int4&) {
     const int oi = S.perm[i];
@@ -406,21 +343,18 @@ __device__ __forceinline__ void resident_solve(const DevSys& S, const DevWork& w
       bool ok = true;
       if (r.x & kResRowLevel0) ok = inv2(D);
       if (!ok)
-        for (int q = 0; q < P; ++q) *remote(&sh_flag, q) = 1;
+        for (int q = 0; q < P; ++q) *remote_smem<CL>(&sh_flag, q) = 1;
       st_blk(A + 4 * r.y, D);
     }
-    spread(m, sh_norm);
+    spread<CL>(m, sh_red, sh_norm, P, crank);
     csync<CL>();
     tick(kProfMismatch);
 
     // ---- stop test (every thread decides alike) ----
-    const double nrm = widest(sh_norm);
-    status = kRunning;
-    if (!(nrm <= 1e12)) status = PF_ERR_DIVERGED;
-    else if (nrm <= o.tol) status = PF_OK;
-    else if (it >= o.max_iter) status = PF_ERR_MAXITER;
+    const double nrm = widest(sh_norm, P);
+    status = stop_test(o, it, nrm);
     if (status != kRunning) {
-      put_info(status, it, passes, nrm, it > 0 ? widest(sh_step) : 0.0);
+      if (first) put_info(w.out_info, status, it, lin ? passes : 0, nrm, it > 0 ? widest(sh_step, P) : 0.0);
       break;
     }
     const bool refine = o.refine > 0 && refine_now(o, it, nrm, prev);
@@ -449,7 +383,7 @@ __device__ __forceinline__ void resident_solve(const DevSys& S, const DevWork& w
       }
       if constexpr (CL) {
         csync<CL>();
-        if (pass == 0 && tid == 0 && crank != 0 && sh_flag) *remote(&sh_flag, 0) = 1;
+        if (pass == 0 && tid == 0 && crank != 0 && sh_flag) *remote_smem<CL>(&sh_flag, 0) = 1;
         if (crank == 0) {
           // the parts' Schur complements and right-hand sides, in their order
           const int g0 = pass == 0 ? 0 : R.ngat_blk;
@@ -459,7 +393,7 @@ __device__ __forceinline__ void resident_solve(const DevSys& S, const DevWork& w
               Blk<TF> v = ld_blk(At + 4 * g.x);
               for (int q = g.y; q < g.z; ++q) {
                 const int2 s = __ldg(R.gsrc + q);
-                const Blk<TF> u = ld_blk(remote(A, s.x) + 4 * s.y);
+                const Blk<TF> u = ld_blk(remote_smem<CL>(A, s.x) + 4 * s.y);
                 v.a += u.a;
                 v.b += u.b;
                 v.c += u.c;
@@ -471,7 +405,7 @@ __device__ __forceinline__ void resident_solve(const DevSys& S, const DevWork& w
               V2 v = reinterpret_cast<V2*>(yt)[g.x];
               for (int q = g.y; q < g.z; ++q) {
                 const int2 s = __ldg(R.gsrc + q);
-                const V2 u = reinterpret_cast<const V2*>(remote(y, s.x))[s.y];
+                const V2 u = reinterpret_cast<const V2*>(remote_smem<CL>(y, s.x))[s.y];
                 v.x += u.x;
                 v.y += u.y;
               }
@@ -488,8 +422,8 @@ __device__ __forceinline__ void resident_solve(const DevSys& S, const DevWork& w
           run_rounds<kBackward, TF>(tt + (top.rb - top.rf), top.nrb, R.rec, At, yt, ring, &sh_flag);
         }
         csync<CL>();
-        if (pass == 0) singular = *remote(&sh_flag, 0) != 0;
-        const V2* xt = reinterpret_cast<const V2*>(remote(y, 0)) + top.vec0;
+        if (pass == 0) singular = *remote_smem<CL>(&sh_flag, 0) != 0;
+        const V2* xt = reinterpret_cast<const V2*>(remote_smem<CL>(y, 0)) + top.vec0;
         for (int k = tid; k < part.nb; k += T)
           reinterpret_cast<V2*>(yp)[part.np + k] = xt[__ldg(R.bnd + part.bnd + k)];
         __syncthreads();
@@ -511,7 +445,7 @@ __device__ __forceinline__ void resident_solve(const DevSys& S, const DevWork& w
     }
     if (singular) {
       status = PF_ERR_SINGULAR;
-      put_info(status, it, passes - 1, nrm, 0.0);
+      if (first) put_info(w.out_info, status, it, lin ? passes - 1 : 0, nrm, 0.0);
       csync<CL>();
       break;
     }
@@ -538,7 +472,7 @@ __device__ __forceinline__ void resident_solve(const DevSys& S, const DevWork& w
       if (sizeof(TF) == 8) w.U[i] = make_double2(cs, sn);
       w.V[i] = make_double2(vm * cs, vm * sn);
     });
-    spread(ms, sh_step);
+    spread<CL>(ms, sh_red, sh_step, P, crank);
     csync<CL>();
     tick(kProfUpdate);
   }
@@ -601,7 +535,7 @@ __global__ void __launch_bounds__(512) k_resident_group(const GroupJob* desc, Gr
       reinterpret_cast<unsigned*>(&job)[k] = reinterpret_cast<const unsigned*>(src)[k];
     __syncthreads();
     for (int k = threadIdx.x; k < (int)(sizeof(ResDev) / 4); k += blockDim.x)
-      reinterpret_cast<unsigned*>(&plan)[k] = reinterpret_cast<const unsigned*>(job.res)[k];
+      reinterpret_cast<unsigned*>(&plan)[k] = static_cast<const unsigned*>(job.res)[k];
   }
   __syncthreads();
   resident_solve<TF, CL>(job.S, job.w, job.o, plan, 0);
@@ -613,33 +547,12 @@ __global__ void __launch_bounds__(512) k_resident_group(const GroupJob* desc, Gr
   }
 }
 
-template <class Kern>
-cudaError_t configure(Kern kern, bool CL, int P, int threads, size_t smem, int B, cudaStream_t st,
-                      cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr) {
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess && P > 8)
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  cfg.gridDim = dim3(B * P);
-  cfg.blockDim = dim3(threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  if (CL) {
-    attr->id = cudaLaunchAttributeClusterDimension;
-    attr->val.clusterDim.x = P;
-    attr->val.clusterDim.y = 1;
-    attr->val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-  }
-  return e;
-}
-
 template <typename TF, bool CL>
 cudaError_t launch_res(const DevSys& S, const DevWork& w, const DevOpts& o, const ResDev& R,
                        size_t smem, int B, int lin, cudaStream_t st) {
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
-  const cudaError_t e = configure(k_resident<TF, CL>, CL, R.P, R.threads, smem, B, st, cfg, attr);
+  const cudaError_t e = configure_clusters(k_resident<TF, CL>, R.P, R.threads, smem, B, st, cfg, attr);
   if (e != cudaSuccess) return e;
   return cudaLaunchKernelEx(&cfg, k_resident<TF, CL>, S, w, o, R, lin);
 }
@@ -650,29 +563,9 @@ cudaError_t launch_group(const GroupJob* desc, const GroupList& list, size_t sme
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   const cudaError_t e =
-      configure(k_resident_group<TF, CL>, CL, P, threads, smem, list.n, st, cfg, attr);
+      configure_clusters(k_resident_group<TF, CL>, P, threads, smem, list.n, st, cfg, attr);
   if (e != cudaSuccess) return e;
   return cudaLaunchKernelEx(&cfg, k_resident_group<TF, CL>, desc, list);
-}
-
-template <typename TF, bool CL>
-int clusters_of(int P, int threads, size_t smem) {
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
-  int num = 0;
-  cudaError_t e = configure(k_resident<TF, CL>, CL, P, threads, smem, 1, nullptr, cfg, attr);
-  if (e == cudaSuccess) {
-    if (CL) {
-      e = cudaOccupancyMaxActiveClusters(&num, k_resident<TF, CL>, &cfg);
-    } else {
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&num, k_resident<TF, CL>, threads, smem);
-    }
-  }
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  return num;
 }
 
 }  // namespace
@@ -697,8 +590,11 @@ cudaError_t launch_resident_group(bool fp32, const GroupJob* desc, const GroupLi
 }
 
 int resident_clusters(bool fp32, int P, int threads, size_t smem) {
-  if (P > 1) return fp32 ? clusters_of<float, true>(P, threads, smem) : clusters_of<double, true>(P, threads, smem);
-  return fp32 ? clusters_of<float, false>(P, threads, smem) : clusters_of<double, false>(P, threads, smem);
+  if (P > 1)
+    return fp32 ? count_clusters(k_resident<float, true>, P, threads, smem)
+                : count_clusters(k_resident<double, true>, P, threads, smem);
+  return fp32 ? count_clusters(k_resident<float, false>, P, threads, smem)
+              : count_clusters(k_resident<double, false>, P, threads, smem);
 }
 
 }  // namespace pf

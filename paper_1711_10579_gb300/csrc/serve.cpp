@@ -366,7 +366,7 @@ struct Server {
     h_done[k] = 0;
     *smem = d.y_in_smem ? (size_t)n * bs * tf : 0;
     // the plan a single solve of the case runs on (built with the case)
-    *plan = kind == PF_SINGLE_PHASE ? c->nr.res_single[fp32 ? 1 : 0] : nullptr;
+    *plan = c->nr.res_single[fp32 ? 1 : 0];
     g.res = *plan ? (*plan)->d_dev : nullptr;
     if (*plan) *smem = (*plan)->smem;
     return PF_OK;
@@ -452,8 +452,8 @@ struct Server {
       Group want;
       want.bs = r->c->bs;
       want.fp32 = r->o.precision == PF_MIXED;
-      want.cluster = plan ? plan->dev.P : kTierCluster[size_tier(*r)];
-      want.threads = plan ? plan->dev.threads : 0;
+      want.cluster = plan ? plan->P : kTierCluster[size_tier(*r)];
+      want.threads = plan ? plan->threads : 0;
       want.list.n = 0;
       auto it = std::find_if(grp.begin(), grp.end(), [&](const Group& g) {
         return g.bs == want.bs && g.fp32 == want.fp32 && g.cluster == want.cluster &&
@@ -476,9 +476,11 @@ struct Server {
       }
       gnext = (sidx + 1) % kGroupStreams;
       const cudaError_t e =
-          g.threads ? launch_resident_group(g.fp32, h_desc, g.list, g.smem, g.cluster, g.threads,
-                                            gst[sidx])
-                    : launch_newton_group(g.bs, g.fp32, h_desc, g.list, g.smem, g.cluster, gst[sidx]);
+          g.threads && g.bs == 2
+              ? launch_resident_group(g.fp32, h_desc, g.list, g.smem, g.cluster, g.threads, gst[sidx])
+          : g.threads
+              ? launch_feeder_group(g.fp32, h_desc, g.list, g.smem, g.cluster, g.threads, gst[sidx])
+              : launch_newton_group(g.bs, g.fp32, h_desc, g.list, g.smem, g.cluster, gst[sidx]);
       for (int q = 0; q < g.list.n; ++q) {
         if (e == cudaSuccess) jobs[g.list.job[q]].stream = sidx;
         else failed.push_back({g.list.job[q], PF_ERR_CUDA});

@@ -110,13 +110,12 @@ void launch_shape(pf_case c, const pf_opts& o, int B, bool fp32, int* grid, int*
   }
 }
 
-// The resident plan a solve runs on, or null: single-phase Newton-Raphson
-// whose factor fits the shared memory of a cluster, with no explicit shape of
-// the other kernels asked for.
+// The resident plan a solve runs on, or null: Newton-Raphson on a grid (or a
+// radial feeder) whose factor fits the shared memory of a cluster, with no
+// explicit shape of the other kernels asked for.
 int resident_plan(pf_case c, const pf_opts& o, int B, RunMode mode, const ResidentPlan** out) {
   *out = nullptr;
-  if (mode != RunMode::Solve || o.method != PF_NR || c->data.kind != PF_SINGLE_PHASE ||
-      o.block_threads || o.scen_per_cta)
+  if (mode != RunMode::Solve || o.method != PF_NR || o.block_threads || o.scen_per_cta)
     return PF_OK;
   const bool fp32 = o.precision == PF_MIXED;
   if (B > 1) {
@@ -128,7 +127,7 @@ int resident_plan(pf_case c, const pf_opts& o, int B, RunMode mode, const Reside
     *out = c->nr.res_single[fp32 ? 1 : 0];
     return PF_OK;
   }
-  const int P = o.cluster_size ? o.cluster_size : resident_batch(c->nr.sym, fp32, B, c->ctx->num_sms);
+  const int P = o.cluster_size ? o.cluster_size : resident_batch(c->nr.sym, fp32, c->bs == 6, B, c->ctx->num_sms);
   return P ? c->nr.resident_for(c->y, fp32, P, out) : PF_OK;
 }
 
@@ -207,7 +206,8 @@ int run_solve(pf_case c, const pf_opts& o, int B, const double* d_p_load, const 
   d.krylov = o.krylov;
   if (plan) {
     const cudaError_t e =
-        launch_resident(fp32, sys, w, d, plan->dev, plan->smem, B, B > 1 ? 1 : 0, st);
+        bs == 2 ? launch_resident(fp32, sys, w, d, plan->dev, plan->smem, B, B > 1 ? 1 : 0, st)
+                : launch_feeder(fp32, sys, w, d, plan->feed, plan->smem, B, B > 1 ? 1 : 0, st);
     if (e != cudaSuccess) return cuda_error(e, "launching the resident Newton kernel");
     return PF_OK;
   }
@@ -492,7 +492,8 @@ int solve_noalloc(pf_case c, const pf_opts& o, const double* d_p_load, const dou
   d.y_in_smem = ((size_t)n * bs * tf <= 200 * 1024) ? 1 : 0;
   if (plan) {
     w.by_scen = 1;
-    e = launch_resident(fp32, sys, w, d, plan->dev, plan->smem, 1, 0, st);
+    e = bs == 2 ? launch_resident(fp32, sys, w, d, plan->dev, plan->smem, 1, 0, st)
+                : launch_feeder(fp32, sys, w, d, plan->feed, plan->smem, 1, 0, st);
   } else {
     e = launch_newton(bs, fp32, false, sys, w, d, cluster, cluster, threads, st);
   }
@@ -586,9 +587,8 @@ int autotune(pf_case c, int B, pf_opts* io) {
   pf_opts t = o;
   t.scen_per_cta = t.block_threads = 0;
   const ResidentPlan* plan = nullptr;
-  const int P = nr && c->data.kind == PF_SINGLE_PHASE
-                    ? resident_batch(c->nr.sym, o.precision == PF_MIXED, B, c->ctx->num_sms)
-                    : 0;
+  const int P =
+      nr ? resident_batch(c->nr.sym, o.precision == PF_MIXED, c->bs == 6, B, c->ctx->num_sms) : 0;
   if (P) rc = c->nr.resident_for(c->y, o.precision == PF_MIXED, P, &plan);
   if (rc != PF_OK || !plan) return rc;
   float ms[2] = {1e30f, 1e30f};

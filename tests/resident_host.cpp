@@ -10,6 +10,7 @@
 #include <random>
 #include <vector>
 
+#include "../paper_1711_10579_gb300/csrc/feeder.h"
 #include "../paper_1711_10579_gb300/csrc/resident.h"
 
 using namespace pf;
@@ -229,6 +230,156 @@ extern "C" int resident_check(int n, int m, const int* f, const int* t, int P, i
       for (double d : r)
         if (!(std::fabs(d) <= *err)) *err = std::isnan(d) ? INFINITY : std::fabs(d);
     }
+  }
+  return 0;
+}
+
+// The same for a feeder plan (csrc/feeder.cpp): a tree of n nodes with random
+// diagonally dominant scalar blocks (the order of the operations is what the
+// plan decides).  kinds[n]: bus types as the library packs them.
+extern "C" int feeder_check(int n, const int* f, const int* t, const int8_t* kinds, int P, int G,
+                            double* err, int* levels) {
+  Ybus y;
+  y.n = n;
+  std::vector<std::vector<int>> adj(n);
+  for (int i = 0; i < n; ++i) adj[i].push_back(i);
+  for (int e = 0; e < n - 1; ++e) {
+    adj[f[e]].push_back(t[e]);
+    adj[t[e]].push_back(f[e]);
+  }
+  y.rowptr.push_back(0);
+  for (auto& a : adj) {
+    std::sort(a.begin(), a.end());
+    for (int j : a) y.col.push_back(j);
+    y.rowptr.push_back((int)y.col.size());
+  }
+  y.ybs = 3;
+  y.val.assign(18 * y.col.size(), 1.0);
+  Symbolic s;
+  analyze(y, Ordering::MinDegree, true, s);
+  std::vector<int8_t> bt(n);
+  for (int i = 0; i < n; ++i) bt[i] = kinds[s.perm[i]];
+  FeedPlanHost p;
+  if (!feed_plan(s, bt, P, G, p)) return 100;
+  std::mt19937 g(5);
+  std::normal_distribution<double> N;
+  std::vector<double> D(n), br(n, 0.0), b(n);
+  std::vector<int> parent(n, -1), cta(n, -1), slot(n, -1);
+  for (int i = 0; i < n; ++i) {
+    D[i] = 4.0 + 0.3 * N(g);
+    b[i] = N(g);
+    if (p.branch[i] >= 0) {
+      parent[i] = s.y_col[p.branch[i]];
+      br[i] = 0.5 * N(g);
+    }
+  }
+  const double poison = NAN;
+  std::vector<std::vector<double>> H(P, std::vector<double>(p.max_slots, poison)), W = H;
+  std::vector<std::vector<int>> who(P, std::vector<int>(p.max_slots, -1));
+  std::vector<int> phases(n, 0);
+  for (int c = 0; c < P; ++c) {
+    const FeedCta& C = p.cta[c];
+    for (int k = C.own; k < C.own + C.nown; ++k) {
+      const int i = p.node[2 * k], at = p.node[2 * k + 1];
+      if (cta[i] >= 0 || at >= p.max_slots || who[c][at] >= 0) return 1;
+      cta[i] = c;
+      slot[i] = at;
+      who[c][at] = i;
+      H[c][at] = D[i];
+      W[c][at] = b[i];
+    }
+    for (int q = 0; q < 32 * C.ngrp; ++q) {
+      const int id = p.item[2 * (size_t)(32 * C.grp + q)];
+      if (id < 0) continue;
+      const int i = id & (kFeedMaxNodes - 1), a = (id >> 28) & 3;
+      const bool fr = ((bt[i] >> a) & 1) && !(bt[i] & 8);
+      if (cta[i] != c || p.item[2 * (size_t)(32 * C.grp + q) + 1] != slot[i] || fr != ((id >> 30) == 1)) return 2;
+      ++phases[i];
+      const FeedGroup& gr = p.grp[C.grp + q / 32];
+      int seen = 0;
+      for (int e = 0; e < gr.width; ++e) {
+        const int ye = p.ell_y[gr.ell + 32 * e + q % 32];
+        if (ye < 0) continue;
+        if (ye != s.y_rowptr[i] + e || p.ell_col[gr.ell + 32 * e + q % 32] != s.y_col[ye]) return 3;
+        ++seen;
+      }
+      if (fr && seen != s.y_rowptr[i + 1] - s.y_rowptr[i]) return 4;
+    }
+  }
+  for (int i = 0; i < n; ++i)
+    if (cta[i] < 0 || phases[i] != 3) return 5;
+  *levels = 0;
+  std::vector<int> done(n, 0);  // 1 eliminated, 2 substituted
+  auto run = [&](int c, const FeedPart& R, bool backward) {
+    const int r0 = backward ? R.rb : R.rf, nr = backward ? R.nrb : R.nrf;
+    for (int r = r0; r < r0 + nr;) {
+      int e = r;
+      while (p.rnd[2 * e + 1] >= 0) ++e;
+      if (e >= r0 + nr) return 10;
+      ++*levels;
+      std::vector<int> now;  // what this level finishes is not read by it
+      std::vector<double> acc(G, poison), rhs = acc;
+      std::vector<int> on(G, -1);
+      for (int rr = r; rr <= e; ++rr) {
+        const int off = p.rnd[2 * rr], cnt = p.rnd[2 * rr + 1] & 0xffff;
+        if (cnt > G) return 11;
+        for (int q = 0; q < cnt; ++q) {
+          const uint32_t x = p.rec[2 * (size_t)(off + q)], yv = p.rec[2 * (size_t)(off + q) + 1];
+          if (x == kFeedNone) continue;
+          const int at = x & 0xffff, other = x >> 16, rank = (yv >> kFeedRankShift) & 15;
+          const int k = who[c][at], id = yv & (kFeedMaxNodes - 1);
+          if (k < 0) return 12;
+          if (backward) {
+            const int pk = who[rank][other];
+            if (pk != parent[k] || id != k || done[pk] != 2 || done[k] != 1) return 13;
+            W[c][at] -= H[c][at] * W[rank][other];
+            now.push_back(k);
+            continue;
+          }
+          if (yv & kFeedFirst) {
+            acc[q] = H[c][at];
+            rhs[q] = W[c][at];
+            on[q] = k;
+          }
+          if (on[q] != k) return 14;
+          if (!(yv & kFeedFactor)) {
+            const int ch = who[rank][other];
+            if (ch != id || parent[ch] != k || done[ch] != 1) return 15;
+            acc[q] -= br[ch] * H[rank][other];
+            rhs[q] -= br[ch] * W[rank][other];
+          } else {
+            if (id != k || ((yv & kFeedRoot) != 0) != (parent[k] < 0)) return 16;
+            H[c][at] = br[k] / acc[q];
+            W[c][at] = rhs[q] / acc[q];
+            now.push_back(k);
+          }
+        }
+      }
+      for (int k : now) done[k] = backward ? 2 : 1;
+      r = e + 1;
+    }
+    return 0;
+  };
+  for (int c = 0; c < P; ++c)
+    if (int rc = run(c, p.part[c], false)) return rc;
+  if (P > 1)
+    if (int rc = run(0, p.part[P], false)) return 20 + rc;
+  for (int i = 0; i < n; ++i) {
+    if (done[i] != 1) return 30;
+    if (parent[i] < 0) done[i] = 2;
+  }
+  if (P > 1)
+    if (int rc = run(0, p.part[P], true)) return 40 + rc;
+  for (int c = 0; c < P; ++c)
+    if (int rc = run(c, p.part[c], true)) return 60 + rc;
+  *err = 0.0;
+  for (int i = 0; i < n; ++i) {
+    double r = b[i] - D[i] * W[cta[i]][slot[i]];
+    if (done[i] != 2) return 31;
+    if (parent[i] >= 0) r -= br[i] * W[cta[parent[i]]][slot[parent[i]]];
+    for (int k = 0; k < n; ++k)
+      if (parent[k] == i) r -= br[k] * W[cta[k]][slot[k]];
+    if (!(std::fabs(r) <= *err)) *err = std::isnan(r) ? INFINITY : std::fabs(r);
   }
   return 0;
 }

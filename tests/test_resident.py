@@ -1,5 +1,5 @@
-"""Resident solves (csrc/resident.cpp, csrc/resident.cu): the host schedule
-executed on the CPU, and the kernels against the FP64 oracle at the sizes
+"""Resident solves (csrc/resident.cpp, csrc/resident.cu; feeders csrc/feeder.cpp,
+csrc/feeder.cu): the host schedules executed on the CPU, and the kernels against the FP64 oracle at the sizes
 where the cut into CTAs, the groups of 32 rows and the rounds have edges."""
 import ctypes as C
 import dataclasses
@@ -40,7 +40,8 @@ def host():
     subprocess.check_call(["g++", "-O2", "-std=c++17", "-shared", "-fPIC",
                            "-I", os.path.join(build._cuda_home(), "include"), "-o", so,
                            os.path.join(HERE, "resident_host.cpp"),
-                           os.path.join(CSRC, "resident.cpp"), os.path.join(CSRC, "symbolic.cpp")])
+                           *[os.path.join(CSRC, f) for f in
+                             ("resident.cpp", "feeder.cpp", "symbolic.cpp")]])
     return C.CDLL(so)
 
 
@@ -71,6 +72,36 @@ def test_schedule_of_a_tree_and_of_a_star(host):
                                        t.ctypes.data_as(C.c_void_p), P, 128, C.byref(err),
                                        C.byref(parts)) == 0
             assert 0.0 <= err.value <= 1e-13
+
+
+@pytest.mark.parametrize("P,groups", [(1, 4), (1, 32), (2, 8), (4, 16), (16, 32)])
+@pytest.mark.parametrize("n", [1, 2, 40, 700, 3000])
+def test_feeder_schedule_solves_the_system(host, n, P, groups):
+    """Scalar stand-ins for the 6x6 blocks; a feeder too small for P parts has
+    no plan (the other kernels solve it)."""
+    g = cases.feeder_case(n, 4) if n > 1 else None
+    f, t = ((np.ascontiguousarray(a, np.int32) for a in (g.br_from, g.br_to)) if g is not None
+            else (np.zeros(0, np.int32),) * 2)
+    kinds = np.array([7], np.int8) if g is None else g.phases.astype(np.int8)
+    kinds[0] |= 8
+    err, levels = C.c_double(-1.0), C.c_int(0)
+    rc = host.feeder_check(n, *[a.ctypes.data_as(C.c_void_p) for a in (f, t, kinds)], P, groups,
+                           C.byref(err), C.byref(levels))
+    if P > 1 and n < 40 * P:
+        assert rc in (0, 100)
+        return
+    assert rc == 0
+    assert 0.0 <= err.value <= 1e-13
+
+
+def test_feeder_schedule_refuses_pv_nodes(host):
+    g = cases.feeder_case(40, 1)
+    f, t = (np.ascontiguousarray(a, np.int32) for a in (g.br_from, g.br_to))
+    kinds = g.phases.astype(np.int8)
+    kinds[5] |= 16
+    err, levels = C.c_double(), C.c_int()
+    args = lambda: [a.ctypes.data_as(C.c_void_p) for a in (f, t, kinds)]
+    assert host.feeder_check(40, *args(), 1, 8, C.byref(err), C.byref(levels)) == 100
 
 
 # ----------------------------------------------------------------------------
@@ -150,3 +181,40 @@ def test_resident_reports_failures(env):
     _, _, info = pf.pf_solve_batch(c, pl, ql, None, pf.make_opts(max_iter=0))
     assert np.all(info["status"] == pf.PF_ERR_MAXITER) and np.all(info["iterations"] == 0)
     pf.pf_destroy_case(c)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+@pytest.mark.parametrize("n,P", [(1, 1), (2, 1), (11, 1), (33, 1), (300, 2), (300, 4), (1000, 4),
+                                 (1000, 16)])
+def test_resident_feeder_matches_oracle(env, n, P, prec):
+    """Feeders on P CTAs, alone and in a ragged batch, with and without FP64
+    refinement: within 1e-6 of the oracle's solution (the stop test's mismatch
+    of 1e-8); a scenario alone equals the same in a batch bit for bit."""
+    pf, ctx = env
+    if n == 1:
+        z = np.zeros((1, 3))
+        case = cases.ThreePhaseCase(1, 0, np.array([7], np.uint8), z, z, np.array([[0.5, 0.3, 0.2]]),
+                                    np.zeros(0, np.int32), np.zeros(0, np.int32),
+                                    np.zeros(0, np.uint8), np.zeros((0, 3, 3), complex))
+    else:
+        case = cases.feeder_case(n, 5)
+    pl, ql = cases.feeder_scenario_loads(case, 3, seed=2)
+    refs = [O.newton_cim(case.with_loads(pl[b], ql[b]))["V"] if n > 1 else
+            O.cim_flat_start(case) for b in range(3)]
+    c = pf.pf_create_case(ctx, case)
+    try:
+        for rs in (0.1, 0.0):
+            o = pf.make_opts(precision=pf.PF_FP64 if prec == "fp64" else pf.PF_MIXED,
+                             cluster_size=P, refine_stall=rs)
+            shape = pf.pf_launch_config(c, o, 3)
+            assert shape["cluster"] == P and shape["grid"] == 3 * P
+            vm, va, info = pf.pf_solve_batch(c, pl.reshape(3, -1), ql.reshape(3, -1), None, o)
+            vm1, va1, _ = pf.pf_solve_batch(c, pl[:1].reshape(1, -1), ql[:1].reshape(1, -1), None, o)
+            assert np.all(info["status"] == 0) and np.all(info["mismatch"] <= 1e-8)
+            assert np.array_equal(vm[0], vm1[0]) and np.array_equal(va[0], va1[0])
+            for b, V in enumerate(refs):
+                V = V.reshape(-1)
+                assert np.max(np.abs(vm[b] * np.exp(1j * va[b]) - V)) <= 1e-6
+    finally:
+        pf.pf_destroy_case(c)
