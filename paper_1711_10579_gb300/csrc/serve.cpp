@@ -3,9 +3,10 @@
 // Each context owns one dispatcher thread.  Requests wait in a FIFO queue.
 // Newton-Raphson requests run as group launches: one launch takes every
 // queued request that fits (free job slots and the context's HBM budget),
-// of any cases and sizes, and each of its CTAs solves one request on its own
-// (newton.cuh: newton_group_kernel); the largest requests run in separate
-// group launches of 2-, 4- and 8-CTA clusters, one cluster per request.  A job's
+// of any cases and sizes, and each of its CTAs or clusters solves one request
+// on its own: the resident solve of the case where it has one (resident.cu,
+// feeder.cu), else newton.cuh's (newton_group_kernel), the largest on 8-CTA
+// clusters; each kernel and launch shape is a launch of its own.  A job's
 // descriptor, inputs and outputs
 // live in pinned host memory; the CTA raises the job's done flag when its
 // results are written, so every request retires as soon as its own solve
@@ -44,15 +45,11 @@ constexpr int kGroupStreams = 64;  // group launches in flight at once (each on 
 constexpr int kSlots = 8;         // per-request launches (Newton-Krylov, reactive limits)
 constexpr size_t kMaxQueue = 1 << 20;
 constexpr size_t kGroupSmemMax = 200 * 1024;  // a job's solve vector in shared memory up to this
-// Requests of at least this many rows (buses; nodes of a feeder) run on a
-// cluster of CTAs instead of one CTA: their single-CTA solve is the tail of
-// the latency (a 63,000-bus grid: 65 ms on one CTA, 37 ms on 4).  Tiers:
-// kMidCluster CTAs from kMidRows*, kBigCluster from kBigRows*, kHugeCluster
-// from kHugeRows*.
-constexpr int kMidRows1ph = 4000, kMidRows3ph = 2000, kMidCluster = 2;
-constexpr int kBigRows1ph = 16000, kBigRows3ph = 5000, kBigCluster = 4;
-constexpr int kHugeRows1ph = 40000, kHugeRows3ph = 12000, kHugeCluster = 8;
-constexpr int kTierCluster[4] = {1, kMidCluster, kBigCluster, kHugeCluster};
+// Requests without a resident plan of at least this many rows (buses; nodes of
+// a feeder) run on a cluster of kBigCluster CTAs instead of one CTA: they are
+// the tail of the latency (8,000 nodes mixed: 14.5 / 9.6 / 6.4 / 4.8 ms on 1 /
+// 2 / 4 / 8 CTAs; a 37,000-bus grid 29.5 / 22.9 / 17.5 / 15.4 ms).
+constexpr int kBigRows1ph = 4000, kBigRows3ph = 2000, kBigCluster = 8;
 
 // Coalesced batches: kBatchMin or more queued Newton-Raphson requests of one
 // case with the same solve options and their own loads run as one batched
@@ -79,13 +76,11 @@ bool grouped(const Request& r) {
          !r.o.block_threads && !r.o.scen_per_cta && !r.o.cluster_size;
 }
 
-// The cluster size of a request is kTierCluster[size_tier].
-int size_tier(const Request& r) {
-  const bool one = r.c->data.kind == PF_SINGLE_PHASE;
-  const int n = r.c->data.n;
-  if (n >= (one ? kHugeRows1ph : kHugeRows3ph)) return 3;
-  if (n >= (one ? kBigRows1ph : kBigRows3ph)) return 2;
-  return n >= (one ? kMidRows1ph : kMidRows3ph) ? 1 : 0;
+// CTAs of a request that the group kernel of newton.cuh solves.
+int group_cluster(const Request& r) {
+  return r.c->data.n >= (r.c->data.kind == PF_SINGLE_PHASE ? kBigRows1ph : kBigRows3ph)
+             ? kBigCluster
+             : 1;
 }
 
 size_t slots_of(const Request& r) {
@@ -452,7 +447,7 @@ struct Server {
       Group want;
       want.bs = r->c->bs;
       want.fp32 = r->o.precision == PF_MIXED;
-      want.cluster = plan ? plan->P : kTierCluster[size_tier(*r)];
+      want.cluster = plan ? plan->P : group_cluster(*r);
       want.threads = plan ? plan->threads : 0;
       want.list.n = 0;
       auto it = std::find_if(grp.begin(), grp.end(), [&](const Group& g) {
