@@ -1,6 +1,6 @@
 // C ABI of the power-flow library: contexts, cases, solves and inspection
 // calls.  Host code only; every numeric step runs in the CUDA kernels of
-// resident.cu (single-phase Newton-Raphson that fits shared memory),
+// resident.cu, resident_nk.cu and feeder.cu (solves that fit shared memory),
 // newton.cuh (other single solves, Newton-Krylov, served requests), batch.cu
 // (batched Newton-Raphson), flows.cu and qlim.cu.
 #include <cuda_runtime.h>
@@ -363,10 +363,6 @@ int SysBuf::resident_for(const Ybus& y, bool fp32, int P, const ResidentPlan** o
   return PF_OK;
 }
 
-// Shared memory of a resident CTA at most (with the kernels' static arrays
-// below the 227 KB of a CTA).
-constexpr size_t kResidentSmem = 224 * 1024;
-
 int SysBuf::upload_resident(const Ybus& y, bool fp32, ResidentPlan& r) {
   ResPlanHost h;
   r.threads = resident_threads(sym.n, r.P);
@@ -383,12 +379,12 @@ int SysBuf::upload_resident(const Ybus& y, bool fp32, ResidentPlan& r) {
   std::vector<double2> jy64;
   for (size_t k = 0; k < row.size(); ++k) {
     const int* s = &h.row[4 * k];
-    row[k] = make_int4(s[0], s[1], s[2], 0);
+    row[k] = make_int4(s[0], s[1], s[2], s[3]);
     if (s[0] >= 0) diag32[k] = make_float2((float)val(s[3])[0], (float)val(s[3])[1]);
   }
   for (size_t k = 0; k < jac.size(); ++k) {
     const int* s = &h.jac[4 * k];
-    jac[k] = make_int4(s[0], s[1], s[2], bus_type[s[1]] | bus_type[s[2]] << 8);
+    jac[k] = make_int4(s[0], s[1], s[2], bus_type[s[1]] | bus_type[s[2]] << 2 | s[3] << 4);
     if (fp32) jy32.push_back(make_float2((float)val(s[3])[0], (float)val(s[3])[1]));
     else jy64.push_back(make_double2(val(s[3])[0], val(s[3])[1]));
   }

@@ -30,6 +30,10 @@ struct DevBuffer {
   cudaError_t alloc(void** out, size_t nbytes);
 };
 
+// Shared memory of a resident CTA at most (with the kernels' static arrays
+// below the 227 KB of a CTA).
+constexpr size_t kResidentSmem = 224 * 1024;
+
 // A resident plan on the device (resident.h; three phase: feeder.h).
 struct ResidentPlan {
   int P = 1, threads = 0;

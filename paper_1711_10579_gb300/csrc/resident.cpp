@@ -182,7 +182,8 @@ bool res_plan(const Symbolic& s, int P, int threads, ResPlanHost& out) {
   auto find = [&](int i, int j) {
     const int* b = s.lu_col.data() + s.lu_rowptr[i];
     const int* e = s.lu_col.data() + s.lu_rowptr[i + 1];
-    return (int)(std::lower_bound(b, e, j) - s.lu_col.data());
+    const int* q = std::lower_bound(b, e, j);
+    return q != e && *q == j ? (int)(q - s.lu_col.data()) : -1;
   };
   // home part of an entry: that of its pivot, the smaller of row and column
   auto home = [&](int e) { return part[std::min(rowof[e], s.lu_col[e])]; };
@@ -239,6 +240,7 @@ bool res_plan(const Symbolic& s, int P, int threads, ResPlanHost& out) {
           const int i = s.lu_col[pi], eik = find(i, k);
           for (int pj = s.lu_diag[k] + 1; pj < s.lu_rowptr[k + 1]; ++pj) {
             const int j = s.lu_col[pj], e = find(i, j);
+            if (e < 0) continue;  // ILU(0): outside the pattern
             int t;
             if (home(e) == q) {
               t = pos[e];

@@ -7,220 +7,11 @@
 // three dependent L2 round trips, 1.4 us of factorisation and 2 x 1.4 us of
 // sweeps; here it is one round of shared-memory reads, a few FMAs and a block
 // barrier.
-#include "resident.cuh"
-#include "resident.h"
+#include "resident_blocks.cuh"
 
 namespace pf {
 
 namespace {
-
-// 8-byte asynchronous copy global -> shared.
-__device__ __forceinline__ void cp8(void* smem, const void* gmem) {
-  const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(s), "l"(gmem) : "memory");
-}
-
-template <typename TF>
-struct Blk {
-  TF a, b, c, d;  // [a b; c d]
-};
-template <typename TF>
-struct Vec2;
-template <>
-struct Vec2<float> {
-  using T = float2;
-};
-template <>
-struct Vec2<double> {
-  using T = double2;
-};
-
-__device__ __forceinline__ Blk<float> ld_blk(const float* p) {
-  const float4 v = *reinterpret_cast<const float4*>(p);
-  return {v.x, v.y, v.z, v.w};
-}
-__device__ __forceinline__ Blk<double> ld_blk(const double* p) {
-  const double2 v = reinterpret_cast<const double2*>(p)[0], u = reinterpret_cast<const double2*>(p)[1];
-  return {v.x, v.y, u.x, u.y};
-}
-__device__ __forceinline__ void st_blk(float* p, const Blk<float>& v) {
-  *reinterpret_cast<float4*>(p) = make_float4(v.a, v.b, v.c, v.d);
-}
-__device__ __forceinline__ void st_blk(double* p, const Blk<double>& v) {
-  reinterpret_cast<double2*>(p)[0] = make_double2(v.a, v.b);
-  reinterpret_cast<double2*>(p)[1] = make_double2(v.c, v.d);
-}
-__device__ __forceinline__ float2 mk2(float x, float y) { return make_float2(x, y); }
-__device__ __forceinline__ double2 mk2(double x, double y) { return make_double2(x, y); }
-
-// Inverse in closed form; false for a zero or non-finite determinant or
-// inverse (the rule of the batched factorisation).
-template <typename TF>
-__device__ __forceinline__ bool inv2(Blk<TF>& m) {
-  const TF det = dot2(m.a, m.d, -m.b, m.c);
-  const TF r = TF(1) / det;
-  const Blk<TF> v{m.d * r, -m.b * r, -m.c * r, m.a * r};
-  m = v;
-  return det != TF(0) && isfinite(v.a) && isfinite(v.b) && isfinite(v.c) && isfinite(v.d);
-}
-
-enum { kFactor = 0, kForward = 1, kBackward = 2 };
-
-// The rounds tab[0 .. nr) of one part (blocks A, vector y).  A thread's items
-// of the next kResRing rounds are in flight by cp.async, so a round waits
-// for no global load.  Ends with a block barrier (nr > 0).
-template <int MODE, typename TF>
-__device__ __noinline__ void run_rounds(const int2* tab, int nr, const uint2* __restrict__ rec, TF* A,
-                                        TF* y, uint2* ring, int* flag) {
-  using V2 = typename Vec2<TF>::T;
-  constexpr int D = kResRing;
-  const int t = threadIdx.x, T = blockDim.x;
-  V2* yv = reinterpret_cast<V2*>(y);
-#pragma unroll
-  for (int d = 0; d < D; ++d) {
-    if (d < nr) {
-      const int2 q = tab[d];
-      if (t < (q.y & 0xffff)) cp8(ring + d * T + t, rec + q.x + t);
-    }
-    cp_commit();
-  }
-  for (int r = 0; r < nr; ++r) {
-    const int2 q = tab[r];
-    cp_wait<D - 1>();
-    uint2* mine = ring + (r & (D - 1)) * T + t;
-    if (t < (q.y & 0xffff)) {
-      const uint2 it = *mine;
-      const int x = it.x & 0xffff;
-      if (x != kResNone) {
-        const int b = it.x >> 16, c = it.y & 0xffff, k = (it.y >> 16) & (kResMaxRows - 1);
-        if constexpr (MODE == kBackward) {
-          V2 v = yv[x];
-          if (b != kResNone) {
-            const Blk<TF> B = ld_blk(A + 4 * b);
-            const V2 u = yv[c];
-            v.x = nmac2(v.x, B.a, u.x, B.b, u.y);
-            v.y = nmac2(v.y, B.c, u.x, B.d, u.y);
-          }
-          if (it.y & kResFinal) {
-            const Blk<TF> Di = ld_blk(A + 4 * x);
-            v = mk2(dot2(Di.a, v.x, Di.b, v.y), dot2(Di.c, v.x, Di.d, v.y));
-          }
-          yv[x] = v;
-        } else {
-          const Blk<TF> B = ld_blk(A + 4 * b), Di = ld_blk(A + 4 * k);
-          if (MODE == kForward || (it.y & kResVec)) {
-            const V2 u = yv[k];
-            V2 v = yv[x];
-            const TF m0 = dot2(Di.a, u.x, Di.b, u.y), m1 = dot2(Di.c, u.x, Di.d, u.y);
-            v.x = nmac2(v.x, B.a, m0, B.b, m1);
-            v.y = nmac2(v.y, B.c, m0, B.d, m1);
-            yv[x] = v;
-          } else {
-            const Blk<TF> U = ld_blk(A + 4 * c);
-            Blk<TF> v = ld_blk(A + 4 * x);
-            const Blk<TF> m{dot2(Di.a, U.a, Di.b, U.c), dot2(Di.a, U.b, Di.b, U.d),
-                            dot2(Di.c, U.a, Di.d, U.c), dot2(Di.c, U.b, Di.d, U.d)};
-            v.a = nmac2(v.a, B.a, m.a, B.b, m.c);
-            v.b = nmac2(v.b, B.a, m.b, B.b, m.d);
-            v.c = nmac2(v.c, B.c, m.a, B.d, m.c);
-            v.d = nmac2(v.d, B.c, m.b, B.d, m.d);
-            if (it.y & kResFinal) {
-              if (!inv2(v)) *flag = 1;
-            }
-            st_blk(A + 4 * x, v);
-          }
-        }
-      }
-    }
-    if (r + D < nr) {
-      const int2 f = tab[r + D];
-      if (t < (f.y & 0xffff)) cp8(mine, rec + f.x + t);
-    }
-    cp_commit();
-    if (q.y < 0) __syncthreads();
-  }
-}
-
-// Off-diagonal Jacobian block (Eq. 10) of entry (i, j) of types ti, tj.
-template <bool CL>
-__device__ __forceinline__ Blk<float> jac_block(const DevWork& w, int i, int j, int ti, int tj,
-                                                float2 y) {
-  const double2 Vi = ld_state<CL>(w.V + i), Vj = ld_state<CL>(w.V + j);
-  Blk<float> o{0.f, 0.f, 0.f, 0.f};
-  if (ti == PF_SLACK || tj == PF_SLACK) return o;
-  const float vix = to_f32_trunc(Vi.x), viy = to_f32_trunc(Vi.y);
-  const float vjx = to_f32_trunc(Vj.x), vjy = to_f32_trunc(Vj.y);
-  const float yvx = dot2(y.x, vjx, -y.y, vjy), yvy = dot2(y.x, vjy, y.y, vjx);
-  const float cx = dot2(vix, yvx, viy, yvy), cy = dot2(viy, yvx, -vix, yvy);
-  o.a = cy;
-  o.c = -cx;
-  if (tj >= PF_PQ) {
-    const float rv = rsqrtf(dot2(vjx, vjx, vjy, vjy));
-    o.b = cx * rv;
-    o.d = cy * rv;
-  }
-  if (ti == PF_PV) o.c = o.d = 0.f;
-  return o;
-}
-template <bool CL>
-__device__ __forceinline__ Blk<double> jac_block(const DevWork& w, int i, int j, int ti, int tj,
-                                                 double2 y) {
-  const double2 Vi = ld_state<CL>(w.V + i), Uj = ld_state<CL>(w.U + j);
-  const double vmj = ld_state<CL>(w.vm + j);
-  Blk<double> o{0.0, 0.0, 0.0, 0.0};
-  if (ti == PF_SLACK || tj == PF_SLACK) return o;
-  const double yux = dot2(y.x, Uj.x, -y.y, Uj.y), yuy = dot2(y.x, Uj.y, y.y, Uj.x);
-  const double cx = dot2(Vi.x, yux, Vi.y, yuy), cy = dot2(Vi.y, yux, -Vi.x, yuy);
-  o.a = vmj * cy;
-  o.c = -vmj * cx;
-  if (tj >= PF_PQ) {
-    o.b = cx;
-    o.d = cy;
-  }
-  if (ti == PF_PV) o.c = o.d = 0.0;
-  return o;
-}
-
-// Diagonal Jacobian block of row i: V, I of the row, its mismatch power S and
-// loads, the Ybus diagonal.
-__device__ __forceinline__ Blk<float> diag_block(const DevSys& S, int i, int t, double2 Vi, double2,
-                                                 double vm, double2 I, double2, double pl, double ql,
-                                                 float2 y) {
-  if (t == PF_SLACK) return {1.f, 0.f, 0.f, 1.f};
-  const float vix = to_f32_trunc(Vi.x), viy = to_f32_trunc(Vi.y);
-  const float Ix = to_f32_trunc(I.x), Iy = to_f32_trunc(I.y);
-  const float rvi = rsqrtf(dot2(vix, vix, viy, viy));
-  const float uix = vix * rvi, uiy = viy * rvi;
-  const float yvx = dot2(y.x, vix, -y.y, viy), yvy = dot2(y.x, viy, y.y, vix);
-  const float scx = dot2(vix, Ix, viy, Iy), scy = dot2(viy, Ix, -vix, Iy);
-  const float dx = dot2(vix, yvx, viy, yvy), dy = dot2(viy, yvx, -vix, yvy);
-  const float ax = Ix + yvx, ay = Iy + yvy;
-  const float ex = dot2(uix, ax, uiy, ay), ey = dot2(uiy, ax, -uix, ay);
-  const float dshape = fmaf(2.f * S.zip32[3 * i + 2], to_f32_trunc(vm), S.zip32[3 * i + 1]);
-  Blk<float> o{-(scy - dy), fmaf(to_f32_trunc(pl), dshape, ex), scx - dx,
-               fmaf(to_f32_trunc(ql), dshape, ey)};
-  if (t == PF_PV) {
-    o.b = o.c = 0.f;
-    o.d = 1.f;
-  }
-  return o;
-}
-__device__ __forceinline__ Blk<double> diag_block(const DevSys& S, int i, int t, double2 Vi,
-                                                  double2 Ui, double vm, double2 I, double2 Sc,
-                                                  double pl, double ql, double2 y) {
-  if (t == PF_SLACK) return {1.0, 0.0, 0.0, 1.0};
-  const double dshape = fma(2.0 * S.zip[3 * i + 2], vm, S.zip[3 * i + 1]);
-  const double yvx = dot2(y.x, Vi.x, -y.y, Vi.y), yvy = dot2(y.x, Vi.y, y.y, Vi.x);
-  const double dx = dot2(Vi.x, yvx, Vi.y, yvy), dy = dot2(Vi.y, yvx, -Vi.x, yvy);
-  const double ax = I.x + yvx, ay = I.y + yvy;
-  const double ex = dot2(Ui.x, ax, Ui.y, ay), ey = dot2(Ui.y, ax, -Ui.x, ay);
-  Blk<double> o{-(Sc.y - dy), fma(pl, dshape, ex), Sc.x - dx, fma(ql, dshape, ey)};
-  if (t == PF_PV) {
-    o.b = o.c = 0.0;
-    o.d = 1.0;
-  }
-  return o;
-}
 
 // One scenario on the CTAs of a cluster (CL) or one CTA.  w: the scenario's
 // own state (B = 1).
@@ -289,63 +80,15 @@ __device__ __forceinline__ void resident_solve(const DevSys& S, const DevWork& w
   double prev = 0.0;
   for (int it = 0;; ++it) {
     // ---- mismatch (Eq. 8-9), right-hand side and Jacobian (Eq. 10) ----
+    bool bad = false;  // a singular first-level pivot
     for (int k = part.z0 + tid; k < part.nblk; k += T) st_blk(Ap + 4 * k, Blk<TF>{0, 0, 0, 0});
     for (int k = part.np + tid; k < part.np + part.nb; k += T)
       reinterpret_cast<V2*>(yp)[k] = mk2(TF(0), TF(0));
     if (has_top)
       for (int k = top.z0 + tid; k < top.nblk; k += T) st_blk(At + 4 * k, Blk<TF>{0, 0, 0, 0});
-    for (int e = tid; e < sc.njac; e += T) {
-      const int4 r = __ldg(R.jac + sc.jac + e);
-      const V2 yv = __ldg(reinterpret_cast<const V2*>(R.jac_y) + sc.jac + e);
-      const int ti = w.bt ? w.bt[r.y] : (r.w & 0xff), tj = w.bt ? w.bt[r.z] : (r.w >> 8);
-      st_blk(A + 4 * r.x, jac_block<CL>(w, r.y, r.z, ti, tj, yv));
-    }
-    unsigned long long m = 0ull;
-    for (int g = warp; g < sc.ngrp; g += nwarp) {
-      const ResGroup G = R.grp[sc.grp + g];
-      const size_t rl = (size_t)(sc.grp + g) * 32 + lane;
-      const int4 r = __ldg(R.row + rl);
-      const bool on = r.x >= 0;
-      const int i = on ? (r.x & ~kResRowLevel0) : 0;
-      const double2 Vi = ld_state<CL>(w.V + i);
-      const double vmi = ld_state<CL>(w.vm + i);
-      const double pl = w.spec[3 * (size_t)i], ql = w.spec[3 * (size_t)i + 1],
-                   pg = w.spec[3 * (size_t)i + 2];
-      const double zp = S.zip[3 * i], zi = S.zip[3 * i + 1], zz = S.zip[3 * i + 2];
-      const int t = w.bt ? w.bt[i] : S.btype[i];
-      double2 I = make_double2(0.0, 0.0), yd = make_double2(0.0, 0.0);
-#pragma unroll 4
-      for (int e = 0; e < G.width; ++e) {
-        const size_t q = (size_t)G.ell + 32 * e + lane;
-        const int j = __ldg(R.ell_col + q);
-        const double2 yv = __ldg(R.ell_y + q), v = ld_state<CL>(w.V + j);
-        if (sizeof(TF) == 8 && e == 0) yd = yv;
-        I.x = fma(yv.x, v.x, I.x);
-        I.x = fma(-yv.y, v.y, I.x);
-        I.y = fma(yv.x, v.y, I.y);
-        I.y = fma(yv.y, v.x, I.y);
-      }
-      if (!on) continue;
-      const double2 Sc = make_double2(dot2(Vi.x, I.x, Vi.y, I.y), dot2(Vi.y, I.x, -Vi.x, I.y));
-      const double shape = fma(fma(zz, vmi, zi), vmi, zp);
-      const double f0 = (t != PF_SLACK) ? fma(-pl, shape, pg) - Sc.x : 0.0;
-      const double qgen = (t == kPQLimit) ? w.qsw[i] : S.q_gen[i];
-      const double f1 = (t >= PF_PQ) ? fma(-ql, shape, qgen) - Sc.y : 0.0;
-      if (o.refine > 0) reinterpret_cast<double2*>(w.F)[i] = make_double2(f0, f1);
-      reinterpret_cast<V2*>(y)[r.z] = mk2((TF)f0, (TF)f1);
-      m = max(m, max(abs_bits(f0), abs_bits(f1)));
-      Blk<TF> D;
-      if constexpr (sizeof(TF) == 4) {
-        D = diag_block(S, i, t, Vi, Vi, vmi, I, Sc, pl, ql, __ldg(R.diag32 + rl));
-      } else {
-        D = diag_block(S, i, t, Vi, ld_state<CL>(w.U + i), vmi, I, Sc, pl, ql, yd);
-      }
-      bool ok = true;
-      if (r.x & kResRowLevel0) ok = inv2(D);
-      if (!ok)
-        for (int q = 0; q < P; ++q) *remote_smem<CL>(&sh_flag, q) = 1;
-      st_blk(A + 4 * r.y, D);
-    }
+    const unsigned long long m = assemble<TF, CL>(S, w, R, sc, A, y, o.refine > 0, (TF*)nullptr, &bad);
+    if (bad)
+      for (int q = 0; q < P; ++q) *remote_smem<CL>(&sh_flag, q) = 1;
     spread<CL>(m, sh_red, sh_norm, P, crank);
     csync<CL>();
     tick(kProfMismatch);
@@ -484,34 +227,6 @@ __device__ __forceinline__ void resident_solve(const DevSys& S, const DevWork& w
     __syncthreads();
     if (tid == 0 && w.out_info) w.out_info->solve_us = (double)(global_ns() - t_begin) * 1e-3;
   }
-}
-
-// Scenario gs of a state laid out [scenario][row].
-__device__ __forceinline__ DevWork scenario_of(DevWork w, int n, int gs) {
-  const size_t r = (size_t)gs * n;
-  w.B = 1;
-  if (w.in_p_load) w.in_p_load += r;
-  if (w.in_q_load) w.in_q_load += r;
-  if (w.in_p_gen) w.in_p_gen += r;
-  if (w.in_vm) w.in_vm += r;
-  if (w.in_va) w.in_va += r;
-  if (w.out_vm) w.out_vm += r;
-  if (w.out_va) w.out_va += r;
-  if (w.out_info) w.out_info += gs;
-  w.spec += 3 * r;
-  w.vm += r;
-  w.va += r;
-  w.V += r;
-  if (w.U) w.U += r;
-  w.dV += r;
-  w.F += 2 * r;
-  w.dx += 2 * r;
-  w.r += 2 * r;
-  if (w.bt) {
-    w.bt += r;
-    w.qsw += r;
-  }
-  return w;
 }
 
 template <typename TF, bool CL>

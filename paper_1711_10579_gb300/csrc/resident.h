@@ -97,11 +97,11 @@ struct ResDev {
   const ResPart* part;
   const ResCta* cta;
   const ResGroup* grp;
-  const int4* row;        // row | level-0 flag, block, slot, 0
+  const int4* row;        // row | level-0 flag, block, slot, Ybus diagonal
   const float2* diag32;   // FP32: a row's Ybus diagonal
   const int* ell_col;
   const double2* ell_y;
-  const int4* jac;        // block, row, column, bus types (row | column << 8)
+  const int4* jac;        // block, row, column, bus types and Ybus entry (row's | column's << 2 | entry << 4)
   const void* jac_y;      // Ybus value, float2 or double2
   const int2* rnd;
   const uint2* rec;
@@ -118,8 +118,9 @@ inline size_t res_smem(const ResPlanHost& p, size_t tf) {
          (size_t)kResRing * p.threads * 8 + (size_t)p.max_tab * 8;
 }
 
-// The plan of P CTAs of `threads` threads for an analysed case (2x2 blocks,
-// exact factor); false if a part exceeds the items' index ranges.
+// The plan of P CTAs of `threads` threads for an analysed case (2x2 blocks; an
+// exact factor, or with P = 1 an ILU(0) pattern); false if a part exceeds the
+// items' index ranges.
 bool res_plan(const Symbolic& s, int P, int threads, ResPlanHost& out);
 
 // Launch of B scenarios on clusters of R.P CTAs (resident.cu); w holds the
@@ -127,6 +128,11 @@ bool res_plan(const Symbolic& s, int P, int threads, ResPlanHost& out);
 // counts the triangular passes.
 cudaError_t launch_resident(bool fp32, const DevSys& S, const DevWork& w, const DevOpts& o,
                             const ResDev& R, size_t smem, int B, int lin, cudaStream_t st);
+// Newton-Krylov (GMRES(m), right ILU(0)) on one CTA per scenario with the ILU(0)
+// factor in shared memory (resident_nk.cu), smem from resident_nk_smem.
+cudaError_t launch_resident_nk(bool fp32, const DevSys& S, const DevWork& w, const DevOpts& o,
+                               const ResDev& R, size_t smem, int B, cudaStream_t st);
+size_t resident_nk_smem(size_t plan_smem, size_t tf, int n, int m);
 // Several requests in one launch, one cluster each (plans of the same P and threads).
 cudaError_t launch_resident_group(bool fp32, const GroupJob* desc, const GroupList& list, size_t smem,
                                   int P, int threads, cudaStream_t st);

@@ -111,12 +111,23 @@ void launch_shape(pf_case c, const pf_opts& o, int B, bool fp32, int* grid, int*
 }
 
 // The resident plan a solve runs on, or null: Newton-Raphson on a grid (or a
-// radial feeder) whose factor fits the shared memory of a cluster, with no
-// explicit shape of the other kernels asked for.
+// radial feeder) whose factor fits the shared memory of a cluster, GMRES on a
+// grid whose ILU(0) factor fits one CTA's, with no explicit shape of the other
+// kernels asked for.
 int resident_plan(pf_case c, const pf_opts& o, int B, RunMode mode, const ResidentPlan** out) {
   *out = nullptr;
-  if (mode != RunMode::Solve || o.method != PF_NR || o.block_threads || o.scen_per_cta)
-    return PF_OK;
+  if (mode != RunMode::Solve || o.block_threads || o.scen_per_cta) return PF_OK;
+  if (o.method == PF_NK) {
+    if (c->bs != 2 || o.krylov != 0 || o.cluster_size) return PF_OK;
+    const bool f = o.precision == PF_MIXED;
+    const int n = c->data.n;
+    const size_t tf = f ? 4 : 8;
+    if (((size_t)c->nk.sym.nnz_lu() * 4 + 2 * (size_t)n) * tf > kResidentSmem) return PF_OK;
+    const ResidentPlan* plan = nullptr;
+    const int rc = c->nk.resident_for(c->y, f, 1, &plan);
+    if (plan && resident_nk_smem(plan->smem, tf, n, o.gmres_restart) <= kResidentSmem) *out = plan;
+    return rc;
+  }
   const bool fp32 = o.precision == PF_MIXED;
   if (B > 1) {
     std::lock_guard<std::mutex> lk(c->tuned_mu);
@@ -204,6 +215,12 @@ int run_solve(pf_case c, const pf_opts& o, int B, const double* d_p_load, const 
   d.max_lin = o.gmres_max_iter;
   d.rtol = o.gmres_rtol;
   d.krylov = o.krylov;
+  if (plan && nk) {
+    const size_t smem = resident_nk_smem(plan->smem, fp32 ? 4 : 8, n, o.gmres_restart);
+    const cudaError_t e = launch_resident_nk(fp32, sys, w, d, plan->dev, smem, B, st);
+    if (e != cudaSuccess) return cuda_error(e, "launching the resident Newton-Krylov kernel");
+    return PF_OK;
+  }
   if (plan) {
     const cudaError_t e =
         bs == 2 ? launch_resident(fp32, sys, w, d, plan->dev, plan->smem, B, B > 1 ? 1 : 0, st)

@@ -96,8 +96,10 @@ struct Run {
 // A grid of n buses and m branches, P CTAs of T threads: solves J x = b twice
 // (the factorisation with its forward sweep, then the forward sweep alone) on
 // random blocks.  Returns 0 and the largest residual, or the rule broken.
-extern "C" int resident_check(int n, int m, const int* f, const int* t, int P, int T, double* err,
-                              int* parts) {
+// ilu: an ILU(0) pattern instead (P = 1), and err its defining property (the
+// product of the factors equals the matrix on the pattern).
+extern "C" int resident_check(int n, int m, const int* f, const int* t, int P, int T, int ilu,
+                              double* err, int* parts) {
   Ybus y;
   y.n = n;
   std::vector<std::vector<int>> adj(n);
@@ -115,7 +117,8 @@ extern "C" int resident_check(int n, int m, const int* f, const int* t, int P, i
   }
   y.val.assign(2 * y.col.size(), 1.0);
   Symbolic s;
-  analyze(y, Ordering::MinDegree, true, s);
+  if (ilu) analyze(y, Ordering::RCM, false, s);
+  else analyze(y, Ordering::MinDegree, true, s);
   ResPlanHost p;
   if (!res_plan(s, P, T, p)) return 100;
   *parts = 0;
@@ -217,6 +220,36 @@ extern "C" int resident_check(int n, int m, const int* f, const int* t, int P, i
     for (int c = 0; c < P; ++c) {
       const int rc = run.rounds(c, p.part[c], p.part[c].rb, p.part[c].nrb, true);
       if (rc) return 60 + rc;
+    }
+    if (ilu) {
+      // sum_k A_ik D_k^-1 A_kj + A_ij (D_i) = the matrix, (i, j) in the pattern
+      std::vector<int> at(s.nnz_lu(), -1);
+      for (int e = 0; e < p.cta[0].njac; ++e) at[entry[p.jac[4 * (size_t)e + 3]]] = p.jac[4 * (size_t)e];
+      for (int k = 0; k < 32 * p.cta[0].ngrp; ++k)
+        if (p.row[4 * (size_t)k] >= 0) at[entry[p.row[4 * (size_t)k + 3]]] = p.row[4 * (size_t)k + 1];
+      auto mul = [](const B4& a, const B4& b) {
+        return B4{a[0] * b[0] + a[1] * b[2], a[0] * b[1] + a[1] * b[3], a[2] * b[0] + a[3] * b[2],
+                  a[2] * b[1] + a[3] * b[3]};
+      };
+      auto entry_of = [&](int i, int j) {
+        for (int q = s.lu_rowptr[i]; q < s.lu_rowptr[i + 1]; ++q)
+          if (s.lu_col[q] == j) return q;
+        return -1;
+      };
+      for (int i = 0; i < n; ++i)
+        for (int q = s.lu_rowptr[i]; q < s.lu_rowptr[i + 1]; ++q) {
+          const int j = s.lu_col[q];
+          B4 sum = M[0][at[q]];
+          if (i == j) invert(sum);
+          for (int k = 0; k < std::min(i, j); ++k) {
+            const int a = entry_of(i, k), c = a < 0 ? -1 : entry_of(k, j);
+            if (c < 0) continue;
+            const B4 t = mul(M[0][at[a]], mul(M[0][at[s.lu_diag[k]]], M[0][at[c]]));
+            for (int d = 0; d < 4; ++d) sum[d] += t[d];
+          }
+          for (int d = 0; d < 4; ++d) *err = std::max(*err, std::fabs(sum[d] - A[q][d]));
+        }
+      return 0;
     }
     for (int i = 0; i < n; ++i) {
       B2 r = b[i];

@@ -54,7 +54,7 @@ def test_schedule_solves_the_system(host, n, P, threads):
     f, t = (np.ascontiguousarray(a, np.int32) for a in (g.br_from, g.br_to))
     err, parts = C.c_double(-1.0), C.c_int(0)
     rc = host.resident_check(n, len(f), f.ctypes.data_as(C.c_void_p), t.ctypes.data_as(C.c_void_p),
-                             P, threads, C.byref(err), C.byref(parts))
+                             P, threads, 0, C.byref(err), C.byref(parts))
     assert rc == 0
     assert 0.0 <= err.value <= 1e-13
     if n == 2000 and P > 1:
@@ -69,9 +69,19 @@ def test_schedule_of_a_tree_and_of_a_star(host):
         for P in (1, 4):
             err, parts = C.c_double(-1.0), C.c_int(0)
             assert host.resident_check(n, len(f), f.ctypes.data_as(C.c_void_p),
-                                       t.ctypes.data_as(C.c_void_p), P, 128, C.byref(err),
+                                       t.ctypes.data_as(C.c_void_p), P, 128, 0, C.byref(err),
                                        C.byref(parts)) == 0
             assert 0.0 <= err.value <= 1e-13
+
+
+@pytest.mark.parametrize("n", [1, 2, 14, 33, 300])
+def test_schedule_of_an_incomplete_factor(host, n):
+    g = mesh(n)
+    f, t = (np.ascontiguousarray(a, np.int32) for a in (g.br_from, g.br_to))
+    err, parts = C.c_double(-1.0), C.c_int(0)
+    assert host.resident_check(n, len(f), f.ctypes.data_as(C.c_void_p), t.ctypes.data_as(C.c_void_p),
+                               1, 64, 1, C.byref(err), C.byref(parts)) == 0
+    assert 0.0 <= err.value <= 1e-14
 
 
 @pytest.mark.parametrize("P,groups", [(1, 4), (1, 32), (2, 8), (4, 16), (16, 32)])
@@ -216,5 +226,31 @@ def test_resident_feeder_matches_oracle(env, n, P, prec):
             for b, V in enumerate(refs):
                 V = V.reshape(-1)
                 assert np.max(np.abs(vm[b] * np.exp(1j * va[b]) - V)) <= 1e-6
+    finally:
+        pf.pf_destroy_case(c)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+@pytest.mark.parametrize("n,m", [(2, 30), (14, 30), (33, 7), (300, 30), (1000, 5), (1000, 40)])
+def test_resident_krylov_matches_oracle(env, n, m, prec):
+    """GMRES(m) with ILU(0), restarted and not, alone and in a ragged batch."""
+    pf, ctx = env
+    case = mesh(n)
+    pl, ql, pg = _loads(case, 3, seed=9)
+    c = pf.pf_create_case(ctx, case)
+    try:
+        o = pf.make_opts(method=pf.PF_NK, precision=pf.PF_FP64 if prec == "fp64" else pf.PF_MIXED,
+                         gmres_restart=m, nk_fallback=0, gmres_max_iter=2000)
+        assert pf.pf_launch_config(c, o, 3)["grid"] == 3
+        vm, va, info = pf.pf_solve_batch(c, pl, ql, pg, o)
+        vm1, va1, info1 = pf.pf_solve_batch(c, pl[:1], ql[:1], pg[:1], o)
+        assert np.all(info["status"] == 0) and np.all(info["mismatch"] <= 1e-8)
+        assert np.all(info["linear_iterations"] >= info["iterations"])
+        assert np.array_equal(vm[0], vm1[0]) and np.array_equal(va[0], va1[0])
+        for b in range(3):
+            r = O.newton_polar(case.with_loads(pl[b], ql[b], pg[b]))
+            assert np.max(np.abs(vm[b] - r["vm"])) <= 1e-6
+            assert np.max(np.abs(va[b] - r["va"])) <= 1e-6
     finally:
         pf.pf_destroy_case(c)
