@@ -15,11 +15,11 @@ struct Item {
   bool vec, fin;
 };
 
-// Rounds of one level: the items of a target form a chain on one thread.
-// Chains go to the thread with the fewest items, long ones first.
+// Rounds of one level: the items of a target form a chain on one slot.
+// Chains go to the slot with the fewest items, long ones first.
 class RoundPacker {
  public:
-  RoundPacker(int threads, ResPlanHost& out) : T_(threads), out_(out) {}
+  RoundPacker(int slots, ResPlanHost& out) : T_(slots), out_(out) {}
 
   void level(std::vector<std::vector<Item>>& chains) {
     if (chains.empty()) return;
@@ -162,11 +162,11 @@ void cut_tree(const Symbolic& s, int P, std::vector<int>& part) {
 
 }  // namespace
 
-bool res_plan(const Symbolic& s, int P, int threads, ResPlanHost& out) {
+bool res_plan(const Symbolic& s, int P, int slots, ResPlanHost& out) {
   const int n = s.n, nnz = s.nnz_lu();
   out = ResPlanHost();
   out.P = P;
-  out.threads = threads;
+  out.slots = slots;
   std::vector<int> part;
   cut_tree(s, P, part);
   const int Q = P > 1 ? P + 1 : 1;  // parts and the top
@@ -212,7 +212,7 @@ bool res_plan(const Symbolic& s, int P, int threads, ResPlanHost& out) {
   }
   auto slot = [&](int q, int i) { return part[i] == q ? lidx[i] : bl[q].at(i); };
 
-  RoundPacker pack(threads, out);
+  RoundPacker pack(slots, out);
   out.part.resize(Q);
   std::vector<int> lev(n, 0);
   for (int q = 0; q < Q; ++q) {

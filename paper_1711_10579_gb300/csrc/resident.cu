@@ -109,7 +109,7 @@ __device__ __forceinline__ void resident_solve(const DevSys& S, const DevWork& w
     bool singular = false;
     for (int pass = 0; pass <= npass; ++pass) {
       if (pass == 0) {
-        run_rounds<kFactor, TF>(tab, part.nrf, R.rec, Ap, yp, ring, &sh_flag);
+        run_rounds<kFactor>(tab, part.nrf, R.rec, Ap, yp, ring, &sh_flag);
       } else {
         // FP64 residual of the step so far (matrix-free), then another solve
         rows([&](int i, const int4&) { dv_row<false>(S, w, i, 0); });
@@ -122,7 +122,7 @@ __device__ __forceinline__ void resident_solve(const DevSys& S, const DevWork& w
           reinterpret_cast<V2*>(yp)[k] = mk2(TF(0), TF(0));
         __syncthreads();
         tick(kProfResidual);
-        run_rounds<kForward, TF>(tab + (part.rw - part.rf), part.nrw, R.rec, Ap, yp, ring, &sh_flag);
+        run_rounds<kForward>(tab + (part.rw - part.rf), part.nrw, R.rec, Ap, yp, ring, &sh_flag);
       }
       if constexpr (CL) {
         csync<CL>();
@@ -158,11 +158,11 @@ __device__ __forceinline__ void resident_solve(const DevSys& S, const DevWork& w
           __syncthreads();
           const int2* tt = tab + sc.ntab;
           if (pass == 0)
-            run_rounds<kFactor, TF>(tt, top.nrf, R.rec, At, yt, ring, &sh_flag);
+            run_rounds<kFactor>(tt, top.nrf, R.rec, At, yt, ring, &sh_flag);
           else
-            run_rounds<kForward, TF>(tt + (top.rw - top.rf), top.nrw, R.rec, At, yt, ring, &sh_flag);
+            run_rounds<kForward>(tt + (top.rw - top.rf), top.nrw, R.rec, At, yt, ring, &sh_flag);
           if (pass == 0) tick(kProfFactor);
-          run_rounds<kBackward, TF>(tt + (top.rb - top.rf), top.nrb, R.rec, At, yt, ring, &sh_flag);
+          run_rounds<kBackward>(tt + (top.rb - top.rf), top.nrb, R.rec, At, yt, ring, &sh_flag);
         }
         csync<CL>();
         if (pass == 0) singular = *remote_smem<CL>(&sh_flag, 0) != 0;
@@ -173,7 +173,7 @@ __device__ __forceinline__ void resident_solve(const DevSys& S, const DevWork& w
       } else {
         if (pass == 0) tick(kProfFactor);
       }
-      run_rounds<kBackward, TF>(tab + (part.rb - part.rf), part.nrb, R.rec, Ap, yp, ring, &sh_flag);
+      run_rounds<kBackward>(tab + (part.rb - part.rf), part.nrb, R.rec, Ap, yp, ring, &sh_flag);
       if (!CL && pass == 0) singular = sh_flag != 0;
       ++passes;
       if (npass > 0)
@@ -230,7 +230,7 @@ __device__ __forceinline__ void resident_solve(const DevSys& S, const DevWork& w
 }
 
 template <typename TF, bool CL>
-__global__ void __launch_bounds__(512)
+__global__ void __launch_bounds__(512, 1)
     k_resident(DevSys S, DevWork w, DevOpts o, ResDev R, int lin) {
   const int gs = CL ? blockIdx.x / (int)cg::this_cluster().num_blocks() : blockIdx.x;
   resident_solve<TF, CL>(S, scenario_of(w, S.n, gs), o, R, lin);
@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(512)
 // Several requests of any cases in one launch: cluster b solves desc[list.job[b]]
 // and raises its done flag (as newton_group_kernel).
 template <typename TF, bool CL>
-__global__ void __launch_bounds__(512) k_resident_group(const GroupJob* desc, GroupList list) {
+__global__ void __launch_bounds__(512, 1) k_resident_group(const GroupJob* desc, GroupList list) {
   const int csize = CL ? (int)cg::this_cluster().num_blocks() : 1;
   const int crank = CL ? (int)cg::this_cluster().block_rank() : 0;
   __shared__ GroupJob job;

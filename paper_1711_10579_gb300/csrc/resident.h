@@ -10,14 +10,15 @@
 // and the parts substitute back.  So a Newton step costs four cluster
 // barriers instead of two per level of the tree.
 //
-// The work of a part is a list of rounds.  In a round a thread executes at
-// most one item of 8 bytes:
+// The work of a part is a list of rounds.  In a round a slot (a thread; FP64: a
+// pair of threads, a row of the 2x2 block each) executes at most one item of 8
+// bytes:
 //   block    A_t -= A_b (A_k^-1 A_c)   (t: target, b = (i, k), c = (k, j))
 //   vector   y_t -= A_b (A_k^-1 y_k)   the right-hand side in the same pass
 //   backward y_t -= A_b y_c, and y_t = A_t^-1 y_t after the row's last entry
 // and the last update of a pivot's diagonal block inverts it in place.  The
 // items of one level read only what earlier levels finished, updates of one
-// target within a level are successive items of one thread, and a barrier
+// target within a level are successive items of one slot, and a barrier
 // ends each level's last round; so a level takes one barrier (not one for
 // the column and one for the updates) and the result does not depend on
 // timing.
@@ -39,7 +40,7 @@ constexpr uint32_t kResFinal = 1u << 31;  // invert / finish the target
 constexpr uint32_t kResVec = 1u << 30;    // a vector item among block items
 constexpr int kResMaxRows = 1 << 14;      // rows of a part (14 bits of k)
 constexpr int kResNone = 0xffff;
-// A round: records [x, x + (y & 0xffff)), one per thread; negative y: a block
+// A round: records [x, x + (y & 0xffff)), one per slot; negative y: a block
 // barrier follows.
 constexpr int kResSync = (int)0x80000000;
 
@@ -70,7 +71,7 @@ struct ResGroup {
 };
 
 struct ResPlanHost {
-  int P = 1, threads = 512;
+  int P = 1, slots = 512;
   std::vector<ResPart> part;    // P parts, then the top (P > 1)
   std::vector<ResCta> cta;
   std::vector<ResGroup> grp;
@@ -112,16 +113,20 @@ struct ResDev {
   int max_blk, max_vec;
 };
 
+// Threads of a slot.
+constexpr int res_lanes(bool fp32) { return fp32 ? 1 : 2; }
+
 // Shared memory of one CTA.
-inline size_t res_smem(const ResPlanHost& p, size_t tf) {
+inline size_t res_smem(const ResPlanHost& p, bool fp32) {
+  const size_t tf = fp32 ? 4 : 8;
   return (size_t)p.max_blk * 4 * tf + (size_t)p.max_vec * 2 * tf + 16 +
-         (size_t)kResRing * p.threads * 8 + (size_t)p.max_tab * 8;
+         (size_t)kResRing * p.slots * res_lanes(fp32) * 8 + (size_t)p.max_tab * 8;
 }
 
-// The plan of P CTAs of `threads` threads for an analysed case (2x2 blocks; an
+// The plan of P CTAs of `slots` slots for an analysed case (2x2 blocks; an
 // exact factor, or with P = 1 an ILU(0) pattern); false if a part exceeds the
 // items' index ranges.
-bool res_plan(const Symbolic& s, int P, int threads, ResPlanHost& out);
+bool res_plan(const Symbolic& s, int P, int slots, ResPlanHost& out);
 
 // Launch of B scenarios on clusters of R.P CTAs (resident.cu); w holds the
 // state [scenario][row], and lin is set for batches: info.linear_iterations

@@ -46,12 +46,24 @@ __device__ __forceinline__ void st_blk(double* p, const Blk<double>& v) {
 __device__ __forceinline__ float2 mk2(float x, float y) { return make_float2(x, y); }
 __device__ __forceinline__ double2 mk2(double x, double y) { return make_double2(x, y); }
 
+// 1 / x.  FP64: the third-order iteration r (1 + e + e^2), e = 1 - x r, from an
+// FP32 reciprocal (e = 2^-23, so e^3 is below the rounding): 3 FP64 operations
+// where the division takes about 7.  Outside the FP32 range: the division.
+__device__ __forceinline__ float recip(float x) { return 1.0f / x; }
+__device__ __forceinline__ double recip(double x) {
+  const int ex = (__double2hiint(x) & 0x7fffffff) >> 20;
+  if (ex < 1023 - 100 || ex > 1023 + 100) return 1.0 / x;
+  const double r = (double)__frcp_rn(to_f32_trunc(x));
+  const double e = __fma_rn(-x, r, 1.0);
+  return __fma_rn(r, __fma_rn(e, e, e), r);
+}
+
 // Inverse in closed form; false for a zero or non-finite determinant or
 // inverse (the rule of the batched factorisation).
 template <typename TF>
 __device__ __forceinline__ bool inv2(Blk<TF>& m) {
   const TF det = dot2(m.a, m.d, -m.b, m.c);
-  const TF r = TF(1) / det;
+  const TF r = recip(det);
   const Blk<TF> v{m.d * r, -m.b * r, -m.c * r, m.a * r};
   m = v;
   return det != TF(0) && isfinite(v.a) && isfinite(v.b) && isfinite(v.c) && isfinite(v.d);
@@ -62,10 +74,11 @@ enum { kFactor = 0, kForward = 1, kBackward = 2 };
 // The rounds tab[0 .. nr) of one part (blocks A, vector y).  A thread's items
 // of the next kResRing rounds are in flight by cp.async, so a round waits
 // for no global load.  Ends with a block barrier (nr > 0).
-template <int MODE, typename TF>
-__device__ __noinline__ void run_rounds(const int2* tab, int nr, const uint2* __restrict__ rec, TF* A,
-                                        TF* y, uint2* ring, int* flag) {
-  using V2 = typename Vec2<TF>::T;
+template <int MODE>
+__device__ __noinline__ void run_rounds(const int2* tab, int nr, const uint2* __restrict__ rec,
+                                        float* A, float* y, uint2* ring, int* flag) {
+  using TF = float;
+  using V2 = float2;
   constexpr int D = kResRing;
   const int t = threadIdx.x, T = blockDim.x;
   V2* yv = reinterpret_cast<V2*>(y);
@@ -130,6 +143,82 @@ __device__ __noinline__ void run_rounds(const int2* tab, int nr, const uint2* __
       if (t < (f.y & 0xffff)) cp8(mine, rec + f.x + t);
     }
     cp_commit();
+    if (q.y < 0) __syncthreads();
+  }
+}
+
+// FP64: two threads an item, a row each.  A warp's FP64 instruction takes 64
+// cycles of its sub-partition whether one lane is active or all, so a level of
+// few items waits for the instructions of one lane: 8 instead of 16 for an
+// update (2,749 buses: factorisations 402 -> 323 us, the solve 590 -> 509 us).
+template <int MODE>
+__device__ __noinline__ void run_rounds(const int2* tab, int nr, const uint2* __restrict__ rec,
+                                        double* A, double* y, uint2* ring, int* flag) {
+  constexpr int D = kResRing;
+  const int t = threadIdx.x, T = blockDim.x, slot = t >> 1, h = t & 1;  // h: the row of the block
+  auto fetch = [&](int r) {
+    if (r < nr) {
+      const int2 q = tab[r];
+      if (slot < (q.y & 0xffff)) cp8(ring + (r & (D - 1)) * T + t, rec + q.x + slot);
+    }
+    cp_commit();
+  };
+  auto row = [&](int blk, int r) { return reinterpret_cast<const double2*>(A)[2 * blk + r]; };
+  for (int r = 0; r < D; ++r) fetch(r);
+  for (int r = 0; r < nr; ++r) {
+    const int2 q = tab[r];
+    cp_wait<D - 1>();
+    const uint2 it = slot < (q.y & 0xffff) ? ring[(r & (D - 1)) * T + t] : make_uint2(kResNone, 0);
+    const int x = it.x & 0xffff, b = it.x >> 16, c = it.y & 0xffff, k = (it.y >> 16) & (kResMaxRows - 1);
+    const bool on = x != kResNone;
+    if constexpr (MODE == kBackward) {
+      double v = 0.0;
+      if (on) {
+        v = y[2 * x + h];
+        if (b != kResNone) {
+          const double2 B = row(b, h);
+          v = nmac2(v, B.x, y[2 * c], B.y, y[2 * c + 1]);
+        }
+      }
+      const double w = __shfl_xor_sync(0xffffffffu, v, 1);  // the pair's other row
+      if (on) {
+        if (it.y & kResFinal) {
+          const double2 Q = row(x, h);
+          v = dot2(Q.x, h ? w : v, Q.y, h ? v : w);
+        }
+        y[2 * x + h] = v;
+      }
+    } else {
+      double2 v = make_double2(0, 0);
+      const bool vec = MODE == kForward || (it.y & kResVec);
+      if (on) {
+        const double2 B = row(b, h), k0 = row(k, 0), k1 = row(k, 1);
+        // the row of A_b A_k^-1
+        const double m0 = dot2(B.x, k0.x, B.y, k1.x), m1 = dot2(B.x, k0.y, B.y, k1.y);
+        if (vec) {
+          y[2 * x + h] = nmac2(y[2 * x + h], m0, y[2 * k], m1, y[2 * k + 1]);
+        } else {
+          const double2 u0 = row(c, 0), u1 = row(c, 1);
+          v = row(x, h);
+          v.x = nmac2(v.x, m0, u0.x, m1, u1.x);
+          v.y = nmac2(v.y, m0, u0.y, m1, u1.y);
+        }
+      }
+      if constexpr (MODE == kFactor) {
+        const double2 w = make_double2(__shfl_xor_sync(0xffffffffu, v.x, 1),
+                                       __shfl_xor_sync(0xffffffffu, v.y, 1));
+        if (on && !vec) {
+          if (it.y & kResFinal) {
+            const double2 r0 = h ? w : v, r1 = h ? v : w;  // [a b], [c d]
+            const double det = dot2(r0.x, r1.y, -r0.y, r1.x), rd = recip(det);
+            v = h ? make_double2(-r1.x * rd, r0.x * rd) : make_double2(r1.y * rd, -r0.y * rd);
+            if (det == 0.0 || !isfinite(v.x) || !isfinite(v.y)) *flag = 1;
+          }
+          reinterpret_cast<double2*>(A)[2 * x + h] = v;
+        }
+      }
+    }
+    fetch(r + D);
     if (q.y < 0) __syncthreads();
   }
 }

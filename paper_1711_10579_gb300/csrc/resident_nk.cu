@@ -90,8 +90,8 @@ __global__ void __launch_bounds__(512, 1) k_resident_nk(DevSys S, DevWork w0, De
   // y <- M^-1 y by the ILU(0) sweeps
   auto precond = [&] {
     __syncthreads();
-    run_rounds<kForward, TF>(tab + (part.rw - part.rf), part.nrw, R.rec, A, yraw, ring, &sh_flag);
-    run_rounds<kBackward, TF>(tab + (part.rb - part.rf), part.nrb, R.rec, A, yraw, ring, &sh_flag);
+    run_rounds<kForward>(tab + (part.rw - part.rf), part.nrw, R.rec, A, yraw, ring, &sh_flag);
+    run_rounds<kBackward>(tab + (part.rb - part.rf), part.nrb, R.rec, A, yraw, ring, &sh_flag);
   };
   // h_j = (V_j, W) for j <= k, a warp each, and W -= sum_j h_j V_j
   auto dots = [&](TF* h, int k) {
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(512, 1) k_resident_nk(DevSys S, DevWork w0, De
     }
     tick(kProfStop);
     // ILU(0); the vector items of the same rounds work on y, which is free here
-    run_rounds<kFactor, TF>(tab, part.nrf, R.rec, A, yraw, ring, &sh_flag);
+    run_rounds<kFactor>(tab, part.nrf, R.rec, A, yraw, ring, &sh_flag);
     __syncthreads();
     tick(kProfFactor);
     if (sh_flag) {

@@ -41,7 +41,7 @@ struct Run {
       for (int pass = 0; pass < 2; ++pass)
         for (int rr = r; rr <= e; ++rr) {
           const int off = p.rnd[2 * rr], cnt = p.rnd[2 * rr + 1] & 0xffff;
-          if (cnt > p.threads) return 2;
+          if (cnt > p.slots) return 2;
           for (int th = 0; th < cnt; ++th) {
             const uint32_t x = p.rec[2 * (size_t)(off + th)], y = p.rec[2 * (size_t)(off + th) + 1];
             const int t = x & 0xffff, b = x >> 16, k = (y >> 16) & (kResMaxRows - 1), u = y & 0xffff;
