@@ -327,35 +327,67 @@ int resident_single(const Symbolic& s, bool fp32, bool three) {
   return P;
 }
 
-// Batches: the fewest CTAs per scenario, as long as the clusters make at most
-// this many waves over the SMs; beyond, the phase kernels' 32 scenarios per
-// warp win.  Measured (ms, resident against phase kernels in their best
-// shape): 2,000 buses mixed x 256 0.69 / 1.94, x 1,000 2.40 / 3.47, x 3,000
-// 6.83 / 6.99; 5,000 mixed x 256 3.4 / 4.7, x 1,000 11.9 / 8.3; 500 FP64 x
-// 256 0.89 / 1.55, x 1,000 3.1 / 2.3; 100 FP64 x 1,000 0.48 / 0.81.
-int resident_batch(const Symbolic& s, bool fp32, bool three, int B, int num_sms) {
-  int P = three ? feeder_least(s.n, fp32) : resident_least(s, fp32);
+// Batches: the fewest CTAs per scenario, and of fewer threads the more of them
+// an SM is to hold (at 128 registers a thread 512 threads fill it): narrow
+// levels leave most of a CTA idle, and other scenarios fill that.  Measured
+// (us, 64 / 128 / 256 / 512 threads): 100 buses mixed x 1,000 107 / 154 / - /
+// -; 200 x 1,000 221 / 270 / 381 / -; 500 x 1,000 706 / 504 / 691 / 933; 500
+// FP64 x 255 685 / 482 / 439 / 636; 2,000 mixed x 512 (one CTA an SM) 4,558 /
+// 2,471 / 1,584 / 1,322.
+//
+// Resident up to 8 clusters per resident CTA of the GPU, whatever the batch
+// where 8 fit an SM; beyond, the phase kernels' 32 scenarios per warp win.
+// Measured (ms, resident against phase kernels in their best shape): mixed, 14
+// buses x 9,728 0.26 / 0.43, 200 x 9,728 1.76 / 2.01, 500 x 2,000 0.96 / 1.79
+// and x 9,728 4.7 / 4.0, 1,000 x 2,400 2.17 / 3.10, 2,000 x 1,000 2.40 / 3.47
+// and x 3,000 6.8 / 7.0, 5,000 (4 CTAs) x 256 3.4 / 4.7 and x 1,000 11.9 / 8.3;
+// FP64, 60 x 9,728 1.40 / 1.46, 200 x 3,000 1.70 / 2.15 and x 9,728 5.4 / 4.7,
+// 500 x 2,000 2.98 / 3.80, 1,000 x 1,200 3.9 / 4.3 and x 2,400 7.9 / 7.1, 2,000
+// (2 CTAs) x 256 3.2 / 4.2 and x 1,000 11.0 / 7.7.
+ResidentShape resident_batch(const Symbolic& s, bool fp32, bool three, int B, int num_sms, int P) {
+  const bool asked = P > 0;  // CTAs per scenario given by the caller
   if (three) {
     // feeders: CTAs of at most 256 nodes, so that two fit an SM.  Measured (ms,
     // resident against phase kernels): 1,000 nodes mixed x 500 3.6 / 4.7, FP64
     // x 250 5.0 / 5.8; 8,000 nodes FP64 x 16 5.4 / 16.3, x 61 16.3 / 16.8
-    while (P > 0 && P < 16 && s.n > 256 * P) P <<= 1;
-    return P > 0 && (double)B * P <= (s.n > 280 * P ? 4.0 : 13.0) * num_sms ? P : 0;
+    if (!asked) {
+      P = feeder_least(s.n, fp32);
+      while (P > 0 && P < 16 && s.n > 256 * P) P <<= 1;
+      if ((double)B * P > (s.n > 280 * P ? 4.0 : 13.0) * num_sms) P = 0;
+    }
+    return {P, 0};
   }
-  const double waves = fp32 || s.n <= 128 ? 8.0 : 3.5;
-  return P > 0 && (double)B * P <= waves * num_sms ? P : 0;
+  if (!asked) P = resident_least(s, fp32);
+  if (P == 0) return {0, 0};
+  int threads = resident_threads(s.n, P), per_sm = 1;
+  const double blocks =
+      (P > 1 ? 1.15 : 1.0) * ((double)s.nnz_lu() * 4 + 2.0 * s.n) * (fp32 ? 4 : 8) / P + 4096;
+  while (per_sm < 8 && (double)B * P > (double)per_sm * num_sms &&
+         2 * per_sm * (blocks + 64.0 * std::min(threads, 256 / per_sm)) <= 224 * 1024) {
+    per_sm <<= 1;
+    threads = std::min(threads, 512 / per_sm);
+  }
+  const double most = per_sm >= 8 ? 1e30 : (P > 1 && !fp32 ? 5.0 : 8.0) * per_sm;
+  if (!asked && (double)B * P > most * num_sms) P = 0;
+  return {P, threads};
 }
 
-int SysBuf::resident_for(const Ybus& y, bool fp32, int P, const ResidentPlan** out) {
+int SysBuf::resident_for(const Ybus& y, bool fp32, ResidentShape shape, const ResidentPlan** out) {
   std::lock_guard<std::mutex> lk(g_mu);
   *out = nullptr;
-  auto& slot = res_cache[2 * P + (fp32 ? 1 : 0)];
+  if (shape.P == 0) return PF_OK;
+  if (shape.threads == 0)
+    shape.threads = y.ybs == 1 ? resident_threads(sym.n, shape.P)
+                               : feeder_groups(sym.n, shape.P) * kFeedLanes;
+  const std::array<int, 3> key = {shape.P, shape.threads, fp32 ? 1 : 0};
+  auto& slot = res_cache[key];
   if (!slot) {
     slot = std::make_unique<ResidentPlan>();
-    slot->P = P;
+    slot->P = shape.P;
+    slot->threads = shape.threads;
     const int rc = y.ybs == 1 ? upload_resident(y, fp32, *slot) : upload_feeder(y, fp32, *slot);
     if (rc != PF_OK) {
-      res_cache.erase(2 * P + (fp32 ? 1 : 0));
+      res_cache.erase(key);
       return rc;
     }
   }
@@ -365,7 +397,6 @@ int SysBuf::resident_for(const Ybus& y, bool fp32, int P, const ResidentPlan** o
 
 int SysBuf::upload_resident(const Ybus& y, bool fp32, ResidentPlan& r) {
   ResPlanHost h;
-  r.threads = resident_threads(sym.n, r.P);
   if (!res_plan(sym, r.P, r.threads / res_lanes(fp32), h)) return PF_OK;
   r.smem = res_smem(h, fp32);
   if (r.smem > kResidentSmem || resident_clusters(fp32, r.P, r.threads, r.smem) < 1) return PF_OK;
@@ -437,9 +468,7 @@ constexpr int kFeederMixedMax = 2000;
 int SysBuf::upload_feeder(const Ybus& y, bool fp32, ResidentPlan& r) {
   FeedPlanHost h;
   if (fp32 && sym.n > kFeederMixedMax) return PF_OK;
-  const int groups = feeder_groups(sym.n, r.P);
-  r.threads = groups * kFeedLanes;
-  if (!feed_plan(sym, bus_type, r.P, groups, h)) return PF_OK;
+  if (!feed_plan(sym, bus_type, r.P, r.threads / kFeedLanes, h)) return PF_OK;
   r.smem = feed_smem(h, fp32);
   if (r.smem > kResidentSmem || feeder_clusters(fp32, r.P, r.threads, r.smem) < 1) return PF_OK;
   const int n = sym.n;
@@ -770,7 +799,7 @@ int pf_create_case(pf_ctx ctx, const pf_case_desc* desc, pf_case* out) {
     for (int fp32 = 0; fp32 < 2; ++fp32) {
       const ResidentPlan* plan = nullptr;
       for (int P = resident_single(c->nr.sym, fp32 != 0, c->bs == 6); P > 0 && P <= 16 && !plan; P <<= 1) {
-        rc = c->nr.resident_for(c->y, fp32 != 0, P, &plan);
+        rc = c->nr.resident_for(c->y, fp32 != 0, {P, 0}, &plan);
         if (rc != PF_OK) return rc;
       }
       c->nr.res_single[fp32] = plan;

@@ -34,6 +34,12 @@ struct DevBuffer {
 // below the 227 KB of a CTA).
 constexpr size_t kResidentSmem = 224 * 1024;
 
+// CTAs per scenario (0: not resident) and threads of one (0: by their share of
+// the rows).
+struct ResidentShape {
+  int P, threads;
+};
+
 // A resident plan on the device (resident.h; three phase: feeder.h).
 struct ResidentPlan {
   int P = 1, threads = 0;
@@ -57,16 +63,16 @@ struct SysBuf {
   // and cached); lanes_cached only looks them up and fails if absent.
   int lanes_for(int threads, int S, DevSys& out);
   int lanes_cached(int threads, int S, DevSys& out);
-  // The resident plan of P CTAs, built and uploaded on first use; null if the
-  // case does not fit it.
-  int resident_for(const Ybus& y, bool fp32, int P, const ResidentPlan** out);
+  // The resident plan of a shape, built and uploaded on first use; null if the
+  // case does not fit it (or shape.P is 0).
+  int resident_for(const Ybus& y, bool fp32, ResidentShape shape, const ResidentPlan** out);
   // The plan of single solves (FP64, FP32), built with the case, or null.
   const ResidentPlan* res_single[2] = {nullptr, nullptr};
 
  private:
   int upload_resident(const Ybus& y, bool fp32, ResidentPlan& r);
   int upload_feeder(const Ybus& y, bool fp32, ResidentPlan& r);
-  std::map<int, std::unique_ptr<ResidentPlan>> res_cache;  // 2 P + fp32
+  std::map<std::array<int, 3>, std::unique_ptr<ResidentPlan>> res_cache;  // P, threads, fp32
 
   void finish_view(const std::array<const int8_t*, 2>& g, int threads, DevSys& out) const;
 };
@@ -157,9 +163,10 @@ struct pf_case_s {
 
 namespace pf {
 
-// CTAs of a resident solve (of one scenario of a batch of B), 0: none.
+// CTAs of a resident single solve, and the shape of a batch of B (P > 0: on P
+// CTAs per scenario).
 int resident_single(const Symbolic& s, bool fp32, bool three);
-int resident_batch(const Symbolic& s, bool fp32, bool three, int B, int num_sms);
+ResidentShape resident_batch(const Symbolic& s, bool fp32, bool three, int B, int num_sms, int P = 0);
 
 enum class RunMode { Solve, Eval, Step };
 enum class InspectKind { Mismatch, Jacobian, Step };

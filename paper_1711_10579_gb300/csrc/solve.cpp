@@ -98,10 +98,13 @@ void launch_shape(pf_case c, const pf_opts& o, int B, bool fp32, int* grid, int*
         tth = it->second[1];
       }
     }
-    // default: about one CTA per SM, up to 8 scenarios per CTA
+    // default: about one CTA per SM, up to 8 scenarios per CTA, 32 for the
+    // phase kernels of 2x2 blocks (a warp's blocks are contiguous there; ms, 8
+    // / 16 / 32: 200 buses mixed x 9,728 3.98 / 2.89 / 2.01, FP64 8.9 / 6.6 /
+    // 4.7; 500 FP64 x 2,000 4.4 / 3.8 / 4.4; 2,000 mixed x 1,200 3.6 / 4.6 / 5.6)
+    const int most = bs == 2 && o.method == PF_NR ? 32 : 8;
     int dS = 1;
-    while (dS < 8 && (long long)B >= 2LL * dS * c->ctx->num_sms) dS <<= 1;
-    if (o.method == PF_NK) dS = std::min(dS, 8);
+    while (dS < most && (long long)B >= 2LL * dS * c->ctx->num_sms) dS <<= 1;
     *threads = o.block_threads ? std::min(o.block_threads, max_threads)
                                : (tth ? tth : max_threads);
     *cluster = 1;
@@ -124,7 +127,7 @@ int resident_plan(pf_case c, const pf_opts& o, int B, RunMode mode, const Reside
     const size_t tf = f ? 4 : 8;
     if (((size_t)c->nk.sym.nnz_lu() * 4 + 2 * (size_t)n) * tf > kResidentSmem) return PF_OK;
     const ResidentPlan* plan = nullptr;
-    const int rc = c->nk.resident_for(c->y, f, 1, &plan);
+    const int rc = c->nk.resident_for(c->y, f, {1, 0}, &plan);
     if (plan && resident_nk_smem(plan->smem, tf, n, o.gmres_restart) <= kResidentSmem) *out = plan;
     return rc;
   }
@@ -138,8 +141,10 @@ int resident_plan(pf_case c, const pf_opts& o, int B, RunMode mode, const Reside
     *out = c->nr.res_single[fp32 ? 1 : 0];
     return PF_OK;
   }
-  const int P = o.cluster_size ? o.cluster_size : resident_batch(c->nr.sym, fp32, c->bs == 6, B, c->ctx->num_sms);
-  return P ? c->nr.resident_for(c->y, fp32, P, out) : PF_OK;
+  const ResidentShape shape =
+      B == 1 ? ResidentShape{o.cluster_size, 0}
+             : resident_batch(c->nr.sym, fp32, c->bs == 6, B, c->ctx->num_sms, o.cluster_size);
+  return c->nr.resident_for(c->y, fp32, shape, out);
 }
 
 int run_solve(pf_case c, const pf_opts& o, int B, const double* d_p_load, const double* d_q_load,
@@ -604,9 +609,10 @@ int autotune(pf_case c, int B, pf_opts* io) {
   pf_opts t = o;
   t.scen_per_cta = t.block_threads = 0;
   const ResidentPlan* plan = nullptr;
-  const int P =
-      nr ? resident_batch(c->nr.sym, o.precision == PF_MIXED, c->bs == 6, B, c->ctx->num_sms) : 0;
-  if (P) rc = c->nr.resident_for(c->y, o.precision == PF_MIXED, P, &plan);
+  const bool fp32 = o.precision == PF_MIXED;
+  if (nr)
+    rc = c->nr.resident_for(
+        c->y, fp32, resident_batch(c->nr.sym, fp32, c->bs == 6, B, c->ctx->num_sms), &plan);
   if (rc != PF_OK || !plan) return rc;
   float ms[2] = {1e30f, 1e30f};
   e = cudaEventCreate(&e0);

@@ -177,6 +177,29 @@ def test_resident_matches_oracle(env, n, P, prec):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+@pytest.mark.parametrize("n,B", [(14, 153), (14, 1217), (14, 9728), (60, 305), (300, 153), (300, 609), (500, 305),
+                                 (500, 609)])
+def test_resident_batch_threads(env, n, B, prec):
+    """The threads of a CTA follow the batch: every shape of a scenario's CTA
+    gives the same bits (the order of a block's updates is the plan's)."""
+    pf, ctx = env
+    case = mesh(n)
+    pl, ql, pg = _loads(case, B, seed=9)
+    c = pf.pf_create_case(ctx, case)
+    try:
+        o = pf.make_opts(precision=pf.PF_FP64 if prec == "fp64" else pf.PF_MIXED, cluster_size=1)
+        assert pf.pf_launch_config(c, o, B)["threads"] <= pf.pf_launch_config(c, o, 3)["threads"]
+        vm, va, info = pf.pf_solve_batch(c, pl, ql, pg, o)
+        assert np.all(info["status"] == 0)
+        for k in (0, B // 2, B - 3):
+            vm3, va3, _ = pf.pf_solve_batch(c, pl[k:k + 3], ql[k:k + 3], pg[k:k + 3], o)
+            assert np.array_equal(vm[k:k + 3], vm3) and np.array_equal(va[k:k + 3], va3)
+    finally:
+        pf.pf_destroy_case(c)
+
+
+@pytest.mark.gpu
 def test_resident_reports_failures(env):
     """A scenario past the loading nose next to one that converges, and an
     iteration limit."""
