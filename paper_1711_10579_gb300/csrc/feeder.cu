@@ -39,18 +39,6 @@ struct Mag {
   static constexpr int inf = sizeof(TF) == 4 ? 0x7f800000 : 0x7ff00000;
 };
 
-// 1 / x.  FP64: the third-order iteration r (1 + e + e^2), e = 1 - x r, from an
-// FP32 reciprocal (e = 2^-23, so e^3 is below the rounding): 3 FP64 operations
-// where the division takes about 7.  Outside the FP32 range: the division.
-__device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
-__device__ __forceinline__ double recip(double x) {
-  const int ex = mag(x) >> 20;
-  if (ex < 1023 - 100 || ex > 1023 + 100) return 1.0 / x;
-  const double r = (double)__frcp_rn(to_f32_trunc(x));
-  const double e = __fma_rn(-x, r, 1.0);
-  return __fma_rn(r, __fma_rn(e, e, e), r);
-}
-
 // d += Y g for a branch admittance (complex 3x3 in the form of Eq. 21: rows
 // Im, Re of the current, columns Re, Im of the voltage).
 template <typename TF>

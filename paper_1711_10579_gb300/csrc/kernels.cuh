@@ -58,6 +58,18 @@ __device__ __forceinline__ void cp_wait() {
 // FP64 -> FP32 rounded toward zero by integer instructions (fixtrig.h).
 __device__ __forceinline__ float to_f32_trunc(double v) { return fx::to_f32_trunc(v); }
 
+// 1 / x.  FP64: the third-order iteration r (1 + e + e^2), e = 1 - x r, from an
+// FP32 reciprocal (e = 2^-23, so e^3 is below the rounding): 3 FP64 operations
+// where the division takes about 7.  Outside the FP32 range: the division.
+__device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
+__device__ __forceinline__ double recip(double x) {
+  const int ex = (__double2hiint(x) & 0x7fffffff) >> 20;
+  if (ex < 1023 - 100 || ex > 1023 + 100) return 1.0 / x;
+  const double r = (double)__frcp_rn(to_f32_trunc(x));
+  const double e = __fma_rn(-x, r, 1.0);
+  return __fma_rn(r, __fma_rn(e, e, e), r);
+}
+
 // |v| as an ordered bit pattern: non-negative doubles order like their bits,
 // and a NaN of either sign maps above +inf.  Integer work only.
 __device__ __forceinline__ unsigned long long abs_bits(double v) {
@@ -1164,6 +1176,31 @@ __device__ __noinline__ void factor_run(const FactorArgs<TF> S, const Team tm, i
   }
 }
 
+// Finite, by the exponent bits: isfinite() of a double is an FP64 instruction.
+__device__ __forceinline__ bool finite_bits(float x) {
+  return (__float_as_int(x) & 0x7f800000) != 0x7f800000;
+}
+__device__ __forceinline__ bool finite_bits(double x) {
+  return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;
+}
+
+// U_kk^-1 of a 2x2 block, adjugate over determinant; false for a zero or
+// non-finite determinant or inverse (1 / 0 leaves no entry finite).
+template <typename TF>
+__device__ __forceinline__ bool inv_2x2(const TF (&a)[4], TF (&di)[4]) {
+  const TF det = a[0] * a[3] - a[1] * a[2];
+  const TF rd = recip(det);
+  di[0] = a[3] * rd;
+  di[1] = -a[1] * rd;
+  di[2] = -a[2] * rd;
+  di[3] = a[0] * rd;
+  return finite_bits(di[0]) && finite_bits(di[1]) && finite_bits(di[2]) && finite_bits(di[3]);
+}
+
+// The pivot whose diagonal block a target record finishes (-1: none), from the
+// record's `rest` or the end mark of its list.
+__device__ __forceinline__ int finished_pivot(int mark) { return mark < -1 ? -2 - mark : -1; }
+
 // Depth of factor_pipe's per-thread ring of items (2x2 blocks).
 template <typename TF>
 struct FactorPipe {
@@ -1179,7 +1216,10 @@ struct FactorPipe {
 // cp.async while it computes the current item, so the wide levels are not
 // bound by one load latency per item.  Shared memory is laid out [piece]
 // [thread] in 16-byte units so that a warp's accesses do not conflict.  The
-// next step's first records are requested before each barrier.
+// next step's first records are requested before each barrier.  FP64 is bound
+// by its pipe (a warp instruction per 64 cycles and sub-partition), so a
+// pivot's block is inverted once, by the item that updates it last (a level
+// earlier), not for each of its L entries: @@
 template <typename TF>
 __device__ __noinline__ void factor_pipe(const FactorArgs<TF> S, const Team tm, int l0, int l1) {
   if (l0 >= l1) return;
@@ -1195,9 +1235,10 @@ __device__ __noinline__ void factor_pipe(const FactorArgs<TF> S, const Team tm, 
   auto blk_at = [&](int d, int c, int v) { return R + ((d * 3 + c) * NV + v) * T + threadIdx.x; };
   auto rec_at = [&](int m) { return R + (D * 3 * NV + m) * T + threadIdx.x; };
   auto gblk = [&](int e) { return S.lu + ((size_t)e * S.B + gs) * BB; };
-  auto fetch_blk = [&](int d, int c, int e) {
+  auto fetch_blk = [&](int d, int c, const TF* p, int e) {
+    const TF* q = p + ((size_t)e * S.B + gs) * BB;
 #pragma unroll
-    for (int v = 0; v < NV; ++v) cp16(blk_at(d, c, v), gblk(e) + v * (16 / sizeof(TF)));
+    for (int v = 0; v < NV; ++v) cp16(blk_at(d, c, v), q + v * (16 / sizeof(TF)));
   };
   auto read_blk = [&](int d, int c, TF (&a)[BB]) {
 #pragma unroll
@@ -1240,15 +1281,25 @@ __device__ __noinline__ void factor_pipe(const FactorArgs<TF> S, const Team tm, 
       cp_commit();
     }
   };
-  // step 1: r = {e, k, diag(k)}: U_kk^-1 for the diagonal, else L_ik = A_ik U_kk^-1
+  // step 1: r = {e, k, diag(k), ready}: L_ik = A_ik U_kk^-1, with U_kk^-1
+  // formed here for the pivots without updates (ready = 0)
   auto fetch1 = [&](int d, int4 r) {
-    fetch_blk(d, 0, r.z);
-    if (r.x != r.z) fetch_blk(d, 1, r.x);
+    if (!r.w) {
+      fetch_blk(d, 0, S.lu, r.z);
+    } else if (r.x != r.z) {
+      fetch_blk(d, 0, S.uinv, r.y);
+    }
+    if (r.x != r.z) fetch_blk(d, 1, S.lu, r.x);
   };
   auto work1 = [&](int d, int4 r) {
-    TF a[BB], di[BB];
-    read_blk(d, 0, a);
-    const bool ok = blk_inv<2>(a, di);
+    if (r.w && r.x == r.z) return;
+    TF di[BB];
+    read_blk(d, 0, di);
+    bool ok = true;
+    if (!r.w) {
+      const TF a[BB] = {di[0], di[1], di[2], di[3]};
+      ok = inv_2x2(a, di);
+    }
     if (r.x == r.z) {
       if (!ok) S.flag[gs] = 1;
       blk_store<2>(S.uinv + ((size_t)r.y * S.B + gs) * BB, di);
@@ -1261,9 +1312,9 @@ __device__ __noinline__ void factor_pipe(const FactorArgs<TF> S, const Team tm, 
   };
   // step 2: r = {e, L entry, U entry, rest}: A_e -= L U, then the rest
   auto fetch2 = [&](int d, int4 r) {
-    if (!(r.x & kFillFirst)) fetch_blk(d, 0, r.x);
-    fetch_blk(d, 1, r.y);
-    fetch_blk(d, 2, r.z);
+    if (!(r.x & kFillFirst)) fetch_blk(d, 0, S.lu, r.x);
+    fetch_blk(d, 1, S.lu, r.y);
+    fetch_blk(d, 2, S.lu, r.z);
   };
   auto work2 = [&](int d, int4 r) {
     TF c[BB], lv[BB], uv[BB];
@@ -1276,9 +1327,11 @@ __device__ __noinline__ void factor_pipe(const FactorArgs<TF> S, const Team tm, 
     read_blk(d, 1, lv);
     read_blk(d, 2, uv);
     blk_msub<2>(c, lv, uv);
+    int mark = r.w;
     if (r.w >= 0) {
       for (int q = r.w;; ++q) {
         const int2 cq = __ldg(S.con + q);
+        mark = cq.y;
         if (cq.x < 0) break;
         TF l2[BB], u2[BB];
         blk_load<2>(gblk(cq.x), l2);
@@ -1286,7 +1339,14 @@ __device__ __noinline__ void factor_pipe(const FactorArgs<TF> S, const Team tm, 
         blk_msub<2>(c, l2, u2);
       }
     }
-    blk_store<2>(gblk(r.x & ~kFillFirst), c);
+    const int k = finished_pivot(mark);
+    if (k < 0) {
+      blk_store<2>(gblk(r.x & ~kFillFirst), c);
+    } else {  // only its inverse is read from here on
+      TF di[BB];
+      if (!inv_2x2(c, di)) S.flag[gs] = 1;
+      blk_store<2>(S.uinv + ((size_t)k * S.B + gs) * BB, di);
+    }
   };
   fetch_recs(S.fac_rec + S.fac_ptr[l0], count(S.fac_ptr[l0 + 1] - S.fac_ptr[l0]));
   for (int l = l0; l < l1; ++l) {
@@ -1322,9 +1382,7 @@ struct FactorWarp {
 // A warp takes the items w, w + W, ... of a step (W warps); lane j loads the
 // record of the warp's item 32 b + j, and the record of any item in flight is
 // broadcast from the two batches held in registers, so the shared-memory ring
-// holds block data only and keeps D items per warp in flight.  The 2x2
-// pivot block is inverted in closed form (adjugate over the determinant); a
-// zero or non-finite determinant or inverse marks the scenario singular.
+// holds block data only and keeps D items per warp in flight.
 template <typename TF>
 __device__ __noinline__ void factor_warp(const FactorArgs<TF> S, const Team tm, int l0, int l1) {
   if (l0 >= l1) return;
@@ -1338,9 +1396,10 @@ __device__ __noinline__ void factor_warp(const FactorArgs<TF> S, const Team tm, 
   uint4* R = reinterpret_cast<uint4*>(S.ring);
   auto at = [&](int d, int c, int v) { return R + ((d * 3 + c) * NV + v) * T + threadIdx.x; };
   auto gblk = [&](int e) { return S.lu + ((size_t)e * S.B + gs) * BB; };
-  auto fetch_blk = [&](int d, int c, int e) {
+  auto fetch_blk = [&](int d, int c, const TF* p, int e) {
+    const TF* q = p + ((size_t)e * S.B + gs) * BB;
 #pragma unroll
-    for (int v = 0; v < NV; ++v) cp16(at(d, c, v), gblk(e) + v * (16 / sizeof(TF)));
+    for (int v = 0; v < NV; ++v) cp16(at(d, c, v), q + v * (16 / sizeof(TF)));
   };
   auto read_blk = [&](int d, int c, TF (&a)[BB]) {
 #pragma unroll
@@ -1399,21 +1458,27 @@ __device__ __noinline__ void factor_warp(const FactorArgs<TF> S, const Team tm, 
       }
     }
   };
-  // step 1: r = {e, k, diag(k)}: U_kk^-1 for the diagonal, else L_ik = A_ik U_kk^-1
+  // step 1: r = {e, k, diag(k), ready}: L_ik = A_ik U_kk^-1, with U_kk^-1
+  // formed here for the pivots without updates (ready = 0)
   auto fetch1 = [&](int d, int4 r) {
-    fetch_blk(d, 0, r.z);
-    if (r.x != r.z) fetch_blk(d, 1, r.x);
+    if (!r.w) {
+      fetch_blk(d, 0, S.lu, r.z);
+    } else if (r.x != r.z) {
+      fetch_blk(d, 0, S.uinv, r.y);
+    }
+    if (r.x != r.z) fetch_blk(d, 1, S.lu, r.x);
   };
   auto work1 = [&](int d, int4 r) {
-    TF a[BB];
-    read_blk(d, 0, a);
-    const TF det = a[0] * a[3] - a[1] * a[2];
-    const TF rd = TF(1) / det;
-    TF di[BB] = {a[3] * rd, -a[1] * rd, -a[2] * rd, a[0] * rd};
+    if (r.w && r.x == r.z) return;
+    TF di[BB];
+    read_blk(d, 0, di);
+    bool ok = true;
+    if (!r.w) {
+      const TF a[BB] = {di[0], di[1], di[2], di[3]};
+      ok = inv_2x2(a, di);
+    }
     if (r.x == r.z) {
-      if (!(det != TF(0)) || !isfinite(di[0]) || !isfinite(di[1]) || !isfinite(di[2]) ||
-          !isfinite(di[3]))
-        S.flag[gs] = 1;
+      if (!ok) S.flag[gs] = 1;
       blk_store<2>(S.uinv + ((size_t)r.y * S.B + gs) * BB, di);
     } else {
       TF x[BB], lk[BB];
@@ -1424,9 +1489,9 @@ __device__ __noinline__ void factor_warp(const FactorArgs<TF> S, const Team tm, 
   };
   // step 2: r = {e, L entry, U entry, rest}: A_e -= L U, then the rest
   auto fetch2 = [&](int d, int4 r) {
-    if (!(r.x & kFillFirst)) fetch_blk(d, 0, r.x);
-    fetch_blk(d, 1, r.y);
-    fetch_blk(d, 2, r.z);
+    if (!(r.x & kFillFirst)) fetch_blk(d, 0, S.lu, r.x);
+    fetch_blk(d, 1, S.lu, r.y);
+    fetch_blk(d, 2, S.lu, r.z);
   };
   auto work2 = [&](int d, int4 r) {
     TF c[BB], lv[BB], uv[BB];
@@ -1439,9 +1504,11 @@ __device__ __noinline__ void factor_warp(const FactorArgs<TF> S, const Team tm, 
     read_blk(d, 1, lv);
     read_blk(d, 2, uv);
     blk_msub<2>(c, lv, uv);
+    int mark = r.w;
     if (r.w >= 0) {
       for (int q = r.w;; ++q) {
         const int2 cq = __ldg(S.con + q);
+        mark = cq.y;
         if (cq.x < 0) break;
         TF l2[BB], u2[BB];
         blk_load<2>(gblk(cq.x), l2);
@@ -1449,7 +1516,14 @@ __device__ __noinline__ void factor_warp(const FactorArgs<TF> S, const Team tm, 
         blk_msub<2>(c, l2, u2);
       }
     }
-    blk_store<2>(gblk(r.x & ~kFillFirst), c);
+    const int k = finished_pivot(mark);
+    if (k < 0) {
+      blk_store<2>(gblk(r.x & ~kFillFirst), c);
+    } else {  // only its inverse is read from here on
+      TF di[BB];
+      if (!inv_2x2(c, di)) S.flag[gs] = 1;
+      blk_store<2>(S.uinv + ((size_t)k * S.B + gs) * BB, di);
+    }
   };
   int f0 = S.fac_ptr[l0], nf = S.fac_ptr[l0 + 1] - f0;
   nstep = nf;

@@ -46,18 +46,6 @@ __device__ __forceinline__ void st_blk(double* p, const Blk<double>& v) {
 __device__ __forceinline__ float2 mk2(float x, float y) { return make_float2(x, y); }
 __device__ __forceinline__ double2 mk2(double x, double y) { return make_double2(x, y); }
 
-// 1 / x.  FP64: the third-order iteration r (1 + e + e^2), e = 1 - x r, from an
-// FP32 reciprocal (e = 2^-23, so e^3 is below the rounding): 3 FP64 operations
-// where the division takes about 7.  Outside the FP32 range: the division.
-__device__ __forceinline__ float recip(float x) { return 1.0f / x; }
-__device__ __forceinline__ double recip(double x) {
-  const int ex = (__double2hiint(x) & 0x7fffffff) >> 20;
-  if (ex < 1023 - 100 || ex > 1023 + 100) return 1.0 / x;
-  const double r = (double)__frcp_rn(to_f32_trunc(x));
-  const double e = __fma_rn(-x, r, 1.0);
-  return __fma_rn(r, __fma_rn(e, e, e), r);
-}
-
 // Inverse in closed form; false for a zero or non-finite determinant or
 // inverse (the rule of the batched factorisation).
 template <typename TF>

@@ -1,0 +1,42 @@
+"""The phase kernels of batches (explicit shapes): factorisation and sweeps."""
+import numpy as np
+import pytest
+
+from oracle import pf_oracle as O
+from paper_1711_10579_gb300 import cases
+
+
+@pytest.fixture(scope="module")
+def env():
+    from paper_1711_10579_gb300 import pf
+
+    ctx = pf.pf_ctx_create(0)
+    yield pf, ctx
+    pf.pf_ctx_destroy(ctx)
+
+
+def mesh(n):
+    return cases.transmission_case(n, int(1.35 * n), max(n // 5, 1), 3, max_angle=0.06)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("prec", ["mixed", "fp64"])
+@pytest.mark.parametrize("S,B", [(2, 3), (4, 5), (8, 9), (16, 33), (32, 65)])
+@pytest.mark.parametrize("n", [5, 33, 300])
+def test_phase_kernels_match_oracle(env, n, S, B, prec):
+    """Ragged batches in every scenarios-per-CTA shape: within 1e-6 of the
+    oracle's solution, as every solve (the stop test's mismatch of 1e-8)."""
+    pf, ctx = env
+    case = mesh(n)
+    pl, ql, pg = cases.scenario_loads(case, B, seed=5)
+    c = pf.pf_create_case(ctx, case)
+    try:
+        o = pf.make_opts(precision=pf.PF_FP64 if prec == "fp64" else pf.PF_MIXED, scen_per_cta=S)
+        vm, va, info = pf.pf_solve_batch(c, pl, ql, pg, o)
+        assert np.all(info["status"] == 0) and np.all(info["mismatch"] <= 1e-8)
+        for b in (0, B // 2, B - 1):
+            r = O.newton_polar(case.with_loads(pl[b], ql[b], pg[b]))
+            assert np.max(np.abs(vm[b] - r["vm"])) <= 1e-6
+            assert np.max(np.abs(va[b] - r["va"])) <= 1e-6
+    finally:
+        pf.pf_destroy_case(c)
