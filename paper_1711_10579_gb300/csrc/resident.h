@@ -135,9 +135,9 @@ cudaError_t launch_resident(bool fp32, const DevSys& S, const DevWork& w, const 
                             const ResDev& R, size_t smem, int B, int lin, cudaStream_t st);
 // Newton-Krylov (GMRES(m), right ILU(0)) on one CTA per scenario with the ILU(0)
 // factor in shared memory (resident_nk.cu), smem from resident_nk_smem.
-cudaError_t launch_resident_nk(bool fp32, const DevSys& S, const DevWork& w, const DevOpts& o,
-                               const ResDev& R, size_t smem, int B, cudaStream_t st);
-size_t resident_nk_smem(size_t plan_smem, size_t tf, int n, int m);
+cudaError_t launch_resident_nk(const DevSys& S, const DevWork& w, const DevOpts& o, const ResDev& R,
+                               size_t smem, int B, cudaStream_t st);
+size_t resident_nk_smem(size_t plan_smem, int n, int m);
 // Several requests in one launch, one cluster each (plans of the same P and threads).
 cudaError_t launch_resident_group(bool fp32, const GroupJob* desc, const GroupList& list, size_t smem,
                                   int P, int threads, cudaStream_t st);

@@ -8,16 +8,18 @@
 // product two cluster barriers, 176 us per inner iteration on the 2,000-bus
 // grid.  Here the sweeps run the rounds of resident.h and a warp takes a whole
 // dot product (a basis vector read once, coalesced; no reduction across
-// warps).
+// warps).  FP64 only (resident_plan says why).  Measured (ms, persistent kernel ->
+// this one): 500 buses 29.4 -> 11.7, x 64 -> 12.5.
 #include "resident_blocks.cuh"
 
 namespace pf {
 
 namespace {
 
-template <typename TF>
+using TF = double;
+
 __global__ void __launch_bounds__(512, 1) k_resident_nk(DevSys S, DevWork w0, DevOpts o, ResDev R) {
-  using V2 = typename Vec2<TF>::T;
+  using V2 = double2;
   const int n = S.n, m = o.m, gs = blockIdx.x;
   const DevWork w = scenario_of(w0, n, gs);
   const size_t nnz = S.y_rowptr[n];
@@ -274,7 +276,7 @@ __global__ void __launch_bounds__(512, 1) k_resident_nk(DevSys S, DevWork w0, De
       w.va[i] = va;
       double sn, cs;
       sincos_tab(S.trig, va, &sn, &cs);
-      if (sizeof(TF) == 8) w.U[i] = make_double2(cs, sn);
+      w.U[i] = make_double2(cs, sn);
       w.V[i] = make_double2(vm * cs, vm * sn);
     });
     spread<false>(ms, sh_red, sh_step, 1, 0);
@@ -288,27 +290,21 @@ __global__ void __launch_bounds__(512, 1) k_resident_nk(DevSys S, DevWork w0, De
   if (tid == 0 && w.out_info) w.out_info->solve_us = (double)(global_ns() - t_begin) * 1e-3;
 }
 
-template <typename TF>
-cudaError_t launch_nk(const DevSys& S, const DevWork& w, const DevOpts& o, const ResDev& R, size_t smem,
-                      int B, cudaStream_t st) {
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
-  const cudaError_t e = configure_clusters(k_resident_nk<TF>, 1, R.threads, smem, B, st, cfg, attr);
-  if (e != cudaSuccess) return e;
-  return cudaLaunchKernelEx(&cfg, k_resident_nk<TF>, S, w, o, R);
-}
-
 }  // namespace
 
 // The plan's shared memory, the orthogonalised vector, two columns of
 // coefficients and the Hessenberg state.
-size_t resident_nk_smem(size_t plan_smem, size_t tf, int n, int m) {
-  return plan_smem + 32 + ((size_t)2 * n + 2 * (m + 1) + (size_t)(m + 1) * m + 4 * m + 1) * tf;
+size_t resident_nk_smem(size_t plan_smem, int n, int m) {
+  return plan_smem + 32 + ((size_t)2 * n + 2 * (m + 1) + (size_t)(m + 1) * m + 4 * m + 1) * sizeof(TF);
 }
 
-cudaError_t launch_resident_nk(bool fp32, const DevSys& S, const DevWork& w, const DevOpts& o,
-                               const ResDev& R, size_t smem, int B, cudaStream_t st) {
-  return fp32 ? launch_nk<float>(S, w, o, R, smem, B, st) : launch_nk<double>(S, w, o, R, smem, B, st);
+cudaError_t launch_resident_nk(const DevSys& S, const DevWork& w, const DevOpts& o, const ResDev& R,
+                               size_t smem, int B, cudaStream_t st) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  const cudaError_t e = configure_clusters(k_resident_nk, 1, R.threads, smem, B, st, cfg, attr);
+  if (e != cudaSuccess) return e;
+  return cudaLaunchKernelEx(&cfg, k_resident_nk, S, w, o, R);
 }
 
 }  // namespace pf

@@ -121,14 +121,16 @@ int resident_plan(pf_case c, const pf_opts& o, int B, RunMode mode, const Reside
   *out = nullptr;
   if (mode != RunMode::Solve || o.block_threads || o.scen_per_cta) return PF_OK;
   if (o.method == PF_NK) {
-    if (c->bs != 2 || o.krylov != 0 || o.cluster_size) return PF_OK;
-    const bool f = o.precision == PF_MIXED;
+    // Not mixed: FP32 sums in another order move the mismatch of a step by 10%,
+    // and where it lands that close to the limit (2.5% of load scenarios of the
+    // 2,000-bus grid) the solve ends a step earlier or later, its voltages 1e-7
+    // apart from the persistent kernel's.
+    if (c->bs != 2 || o.krylov != 0 || o.cluster_size || o.precision == PF_MIXED) return PF_OK;
     const int n = c->data.n;
-    const size_t tf = f ? 4 : 8;
-    if (((size_t)c->nk.sym.nnz_lu() * 4 + 2 * (size_t)n) * tf > kResidentSmem) return PF_OK;
+    if (((size_t)c->nk.sym.nnz_lu() * 4 + 2 * (size_t)n) * 8 > kResidentSmem) return PF_OK;
     const ResidentPlan* plan = nullptr;
-    const int rc = c->nk.resident_for(c->y, f, {1, 0}, &plan);
-    if (plan && resident_nk_smem(plan->smem, tf, n, o.gmres_restart) <= kResidentSmem) *out = plan;
+    const int rc = c->nk.resident_for(c->y, false, {1, 0}, &plan);
+    if (plan && resident_nk_smem(plan->smem, n, o.gmres_restart) <= kResidentSmem) *out = plan;
     return rc;
   }
   const bool fp32 = o.precision == PF_MIXED;
@@ -221,8 +223,8 @@ int run_solve(pf_case c, const pf_opts& o, int B, const double* d_p_load, const 
   d.rtol = o.gmres_rtol;
   d.krylov = o.krylov;
   if (plan && nk) {
-    const size_t smem = resident_nk_smem(plan->smem, fp32 ? 4 : 8, n, o.gmres_restart);
-    const cudaError_t e = launch_resident_nk(fp32, sys, w, d, plan->dev, smem, B, st);
+    const size_t smem = resident_nk_smem(plan->smem, n, o.gmres_restart);
+    const cudaError_t e = launch_resident_nk(sys, w, d, plan->dev, smem, B, st);
     if (e != cudaSuccess) return cuda_error(e, "launching the resident Newton-Krylov kernel");
     return PF_OK;
   }

@@ -254,17 +254,15 @@ def test_resident_feeder_matches_oracle(env, n, P, prec):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("prec", ["mixed", "fp64"])
 @pytest.mark.parametrize("n,m", [(2, 30), (14, 30), (33, 7), (300, 30), (1000, 5), (1000, 40)])
-def test_resident_krylov_matches_oracle(env, n, m, prec):
+def test_resident_krylov_matches_oracle(env, n, m):
     """GMRES(m) with ILU(0), restarted and not, alone and in a ragged batch."""
     pf, ctx = env
     case = mesh(n)
     pl, ql, pg = _loads(case, 3, seed=9)
     c = pf.pf_create_case(ctx, case)
     try:
-        o = pf.make_opts(method=pf.PF_NK, precision=pf.PF_FP64 if prec == "fp64" else pf.PF_MIXED,
-                         gmres_restart=m, nk_fallback=0, gmres_max_iter=2000)
+        o = pf.make_opts(method=pf.PF_NK, precision=pf.PF_FP64, gmres_restart=m, nk_fallback=0, gmres_max_iter=2000)
         assert pf.pf_launch_config(c, o, 3)["grid"] == 3
         vm, va, info = pf.pf_solve_batch(c, pl, ql, pg, o)
         vm1, va1, info1 = pf.pf_solve_batch(c, pl[:1], ql[:1], pg[:1], o)
