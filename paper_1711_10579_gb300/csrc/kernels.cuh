@@ -70,6 +70,16 @@ __device__ __forceinline__ double recip(double x) {
   return __fma_rn(r, __fma_rn(e, e, e), r);
 }
 
+// FP32 -> FP64 by integer instructions (the conversion is an FP64 one);
+// denormals become zeros of their sign.
+__device__ __forceinline__ double to_f64(float v) {
+  const unsigned u = (unsigned)__float_as_int(v), ex = u & 0x7f800000u, sign = u & 0x80000000u;
+  unsigned hi = ((u & 0x7fffffffu) >> 3) + (896u << 20);
+  hi = ex == 0x7f800000u ? hi | 0x7ff00000u : hi;  // infinities and NaN
+  hi = ex == 0u ? 0u : hi;
+  return __hiloint2double((int)(hi | sign), ex == 0u ? 0 : (int)(u << 29));
+}
+
 // |v| as an ordered bit pattern: non-negative doubles order like their bits,
 // and a NaN of either sign maps above +inf.  Integer work only.
 __device__ __forceinline__ unsigned long long abs_bits(double v) {
@@ -79,8 +89,19 @@ __device__ __forceinline__ unsigned long long abs_bits(double v) {
 // sin a and cos a: the table method in 64-bit fixed point on the integer
 // pipes (fixtrig.h; four FP64-free conversions and a dozen 64-bit integer
 // products), sincos() beyond |a| <= 4.
+// The library's in a function of its own: inlined, part of it is executed
+// under a false predicate, which takes the FP64 pipe all the same.
+static __device__ __noinline__ double2 sincos_lib(double a) {
+  double2 r;
+  sincos(a, &r.y, &r.x);
+  return r;
+}
 __device__ __forceinline__ void sincos_tab(const long long* tab, double a, double* s, double* c) {
-  if (!fx::sincos_q(tab, a, s, c)) sincos(a, s, c);
+  if (!fx::sincos_q(tab, a, s, c)) {
+    const double2 r = sincos_lib(a);
+    *s = r.y;
+    *c = r.x;
+  }
 }
 
 // The FP64 refinement of a mixed-precision Newton-Raphson step is taken
@@ -232,6 +253,16 @@ __device__ __forceinline__ T group_sum(T v, int G, unsigned gmask) {
 // step A: mismatch + Jacobian, single phase (polar unknowns, 2x2 blocks)
 // ---------------------------------------------------------------------------
 
+// The voltage dependence of a load other than constant power, in a function of
+// its own: a branch the other rows jump over instead of two predicated FP64
+// instructions, which take the pipe all the same.
+static __device__ __noinline__ double load_shape(double zz, double zi, double zp, double vm) {
+  return fma(fma(zz, vm, zi), vm, zp);
+}
+__device__ __forceinline__ bool nonzero(double a, double b) {
+  return ((__double_as_longlong(a) | __double_as_longlong(b)) & 0x7fffffffffffffffLL) != 0;
+}
+
 // Rows: (P, Q) equations of bus i; columns: (delta, |V|) of bus j.  The slack
 // has no unknown and PV buses no |V| unknown: their rows become identity rows
 // and their columns zero, which keeps the system of Eq. 10 unchanged.  With
@@ -259,20 +290,26 @@ __device__ void mismatch_jacobian_1ph(const DevSys& S, const DevWork& w, int i, 
     blk_store<2>(lu + ((size_t)e * B + gs) * 4, blk);
     if (jcopy) blk_store<2>(jcopy + ((size_t)e * B + gs) * 4, blk);
   };
-  // FP64 mismatch of Eq. 8-9 from the current I = sum_j Y_ij V_j (four FMAs
-  // per entry) and S = V conj(I)
+  // FP64 mismatch of Eq. 8-9 from the current I = sum_j Y_ij V_j and S = V
+  // conj(I): the operations of a row are what the batched kernel takes its time
+  // for, so only the bus type's equations are formed (the lanes of a warp share
+  // the row) and constant-power loads take no polynomial.
   double2 I = make_double2(0.0, 0.0);
   auto mismatch = [&]() {
-    const double2 Sc = cmulc(Vi, I);
-    const double shape = fma(fma(zz, vmi, zi), vmi, zp);
-    const double f0 = (t != PF_SLACK) ? fma(-pl, shape, pg) - Sc.x : 0.0;
-    const double qgen = (t == kPQLimit) ? __ldcg(w.qsw + b) : S.q_gen[i];
-    const double f1 = (t >= PF_PQ) ? fma(-ql, shape, qgen) - Sc.y : 0.0;
+    double f0 = 0.0, f1 = 0.0;
+    if (t != PF_SLACK) {
+      double shape = zp;
+      if (nonzero(zi, zz)) shape = load_shape(zz, zi, zp, vmi);
+      f0 = fma(-Vi.x, I.x, fma(-Vi.y, I.y, fma(-pl, shape, pg)));
+      if (t >= PF_PQ) {
+        const double qgen = (t == kPQLimit) ? __ldcg(w.qsw + b) : S.q_gen[i];
+        f1 = fma(-Vi.y, I.x, fma(Vi.x, I.y, fma(-ql, shape, qgen)));
+      }
+    }
     w.F[b * 2] = f0;
     w.F[b * 2 + 1] = f1;
     // max(|f0|, |f1|) on the bit patterns (NaN above +inf), no FP64 instruction
     nrm = __longlong_as_double((long long)max(abs_bits(f0), abs_bits(f1)));
-    return Sc;
   };
   if constexpr (sizeof(TF) == 4) {
 #pragma unroll 4
@@ -354,63 +391,69 @@ __device__ void mismatch_jacobian_1ph(const DevSys& S, const DevWork& w, int i, 
       put(ed, j00, j01, j10, j11);
     }
   } else {
-#pragma unroll 4
-    for (int e = S.y_rowptr[i]; e < S.y_rowptr[i + 1]; ++e) {
-      const int j = S.y_col[e];
-      const double2 y = Y[e], v = ldc(w.V + (size_t)j * B + gs);
-      I.x = fma(y.x, v.x, I.x);
-      I.x = fma(-y.y, v.y, I.x);
-      I.y = fma(y.x, v.y, I.y);
-      I.y = fma(y.y, v.x, I.y);
-    }
-    const double2 Sc = mismatch();
-    // U = V / |V| per bus (kept by the update in FP64 solves) avoids divisions
-    const double2 Ui = ldc(w.U + b);
-    const double dshape = fma(2.0 * zz, vmi, zi);
+    // One pass over the factor's row: Y_ij U_j (U = V / |V|, kept by the update
+    // in FP64 solves) gives both the current, I += |V_j| Y_ij U_j, and the
+    // off-diagonal block (12 operations an entry; two passes took 14 and read
+    // V_j as well).
+    double ydx = 0.0, ydy = 0.0;
+    int ed = -1;
 #pragma unroll 2
     for (int e = S.lu_rowptr[i]; e < S.lu_rowptr[i + 1]; ++e) {
-      const int j = S.lu_col[e];
       const int yi = S.lu2y[e];
       if (yi < 0) continue;  // fill entry: the factor starts it from zero
+      const int j = S.lu_col[e];
+      const double yx = Y[yi].x, yy = Y[yi].y;
+      if (j == i) {
+        ed = e;
+        ydx = yx;
+        ydy = yy;
+        continue;
+      }
+      const size_t bj = (size_t)j * B + gs;
+      const double2 Uj = ldc(w.U + bj);
+      const double vmj = __ldcg(w.vm + bj);
+      const double yux = fma(yx, Uj.x, -yy * Uj.y), yuy = fma(yx, Uj.y, yy * Uj.x);
+      I.x = fma(vmj, yux, I.x);
+      I.y = fma(vmj, yuy, I.y);
       double j00 = 0, j01 = 0, j10 = 0, j11 = 0;
-      {
-        const double yx = Y[yi].x, yy = Y[yi].y;
-        if (j != i) {
-          const int tj = tp[j * ts];
-          if (t != PF_SLACK && tj != PF_SLACK) {
-            const size_t bj = (size_t)j * B + gs;
-            // dS_i/d|V_j| = V_i conj(Y_ij U_j); dS_i/d delta_j = -j |V_j| dS_i/d|V_j|
-            const double2 Uj = ldc(w.U + bj);
-            const double vmj = __ldcg(w.vm + bj);
-            const double yux = yx * Uj.x - yy * Uj.y, yuy = yx * Uj.y + yy * Uj.x;
-            const double cx = Vi.x * yux + Vi.y * yuy, cy = Vi.y * yux - Vi.x * yuy;
-            j00 = vmj * cy;
-            j10 = -vmj * cx;
-            if (tj >= PF_PQ) {
-              j01 = cx;
-              j11 = cy;
-            }
-            if (t == PF_PV) j10 = j11 = 0.0;
-          }
-        } else if (t == PF_SLACK) {
-          j00 = j11 = 1.0;
-        } else {
-          const double yvx = yx * Vi.x - yy * Vi.y, yvy = yx * Vi.y + yy * Vi.x;  // Y_ii V_i
-          const double dx = Vi.x * yvx + Vi.y * yvy, dy = Vi.y * yvx - Vi.x * yvy;
-          const double ax = I.x + yvx, ay = I.y + yvy;
-          const double ex = Ui.x * ax + Ui.y * ay, ey = Ui.y * ax - Ui.x * ay;
-          j00 = -(Sc.y - dy);
-          j10 = Sc.x - dx;
-          j01 = ex + pl * dshape;
-          j11 = ey + ql * dshape;
-          if (t == PF_PV) {
-            j01 = 0.0;
-            j10 = 0.0;
-            j11 = 1.0;
-          }
+      const int tj = tp[j * ts];
+      if (t != PF_SLACK && tj != PF_SLACK) {
+        // dS_i/d|V_j| = V_i conj(Y_ij U_j); dS_i/d delta_j = -j |V_j| dS_i/d|V_j|
+        const double cx = fma(Vi.x, yux, Vi.y * yuy), cy = fma(Vi.y, yux, -Vi.x * yuy);
+        j00 = vmj * cy;
+        if (t != PF_PV) j10 = -vmj * cx;
+        if (tj >= PF_PQ) {
+          j01 = cx;
+          if (t != PF_PV) j11 = cy;
         }
       }
       put(e, (TF)j00, (TF)j01, (TF)j10, (TF)j11);
+    }
+    const double yvx = fma(ydx, Vi.x, -ydy * Vi.y), yvy = fma(ydx, Vi.y, ydy * Vi.x);  // Y_ii V_i
+    I.x = fma(ydx, Vi.x, fma(-ydy, Vi.y, I.x));
+    I.y = fma(ydx, Vi.y, fma(ydy, Vi.x, I.y));
+    mismatch();
+    if (ed >= 0) {
+      double j00 = 1.0, j01 = 0.0, j10 = 0.0, j11 = 1.0;
+      if (t != PF_SLACK) {
+        // dS_i/d delta_i = j (S_i - V_i conj(Y_ii V_i)) = j V_i conj(I_i - Y_ii V_i);
+        // dS_i/d|V_i| = U_i conj(I_i + Y_ii V_i), plus the load's slope
+        const double ox = I.x - yvx, oy = I.y - yvy;
+        j00 = fma(Vi.x, oy, -Vi.y * ox);
+        if (t != PF_PV) {
+          const double2 Ui = ldc(w.U + b);
+          const double ax = I.x + yvx, ay = I.y + yvy;
+          j10 = fma(Vi.x, ox, Vi.y * oy);
+          j01 = fma(Ui.x, ax, Ui.y * ay);
+          j11 = fma(Ui.y, ax, -Ui.x * ay);
+          if (nonzero(zi, zz)) {
+            const double dshape = fma(2.0 * zz, vmi, zi);
+            j01 = fma(pl, dshape, j01);
+            j11 = fma(ql, dshape, j11);
+          }
+        }
+      }
+      put(ed, (TF)j00, (TF)j01, (TF)j10, (TF)j11);
     }
   }
 }
@@ -2069,8 +2112,8 @@ __device__ __forceinline__ double update_row(const DevSys& S, const DevWork& w, 
     double dd, dm;
     if (y && sizeof(TY) == 4) {
       const float2 q = __ldcg(reinterpret_cast<const float2*>(y) + b);
-      dd = (double)q.x;
-      dm = (double)q.y;
+      dd = to_f64(q.x);
+      dm = to_f64(q.y);
     } else {
       const double2 q = __ldcg(reinterpret_cast<const double2*>(y ? (const void*)y : (const void*)w.dx) + b);
       dd = q.x;
