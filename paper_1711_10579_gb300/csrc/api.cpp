@@ -423,9 +423,9 @@ int SysBuf::resident_for(const Ybus& y, bool fp32, ResidentShape shape, const Re
 
 int SysBuf::upload_resident(const Ybus& y, bool fp32, ResidentPlan& r) {
   ResPlanHost h;
-  if (!res_plan(sym, r.P, r.threads / res_lanes(fp32), h)) return PF_OK;
+  if (!res_plan_fit(sym, fp32, r.P, r.threads / res_lanes(fp32), kResidentSmem, h)) return PF_OK;
   r.smem = res_smem(h, fp32);
-  if (r.smem > kResidentSmem || resident_clusters(fp32, r.P, r.threads, r.smem) < 1) return PF_OK;
+  if (resident_clusters(fp32, r.P, r.threads, r.smem) < 1) return PF_OK;
   auto val = [&](int e) { return &y.val[2 * (size_t)sym.y_src[e]]; };
   std::vector<double2> ell_y(h.ell_y.size(), make_double2(0.0, 0.0));
   for (size_t k = 0; k < ell_y.size(); ++k)
@@ -1057,7 +1057,7 @@ int pf_analyze(const pf_case_desc* desc, pf_case_stats* out) {
     if (P == 0) continue;
     if (y.ybs == 1) {
       ResPlanHost h;
-      if (res_plan(nr, P, resident_threads(nr.n, P) / res_lanes(fp32 != 0), h))
+      if (res_plan_fit(nr, fp32 != 0, P, resident_threads(nr.n, P) / res_lanes(fp32 != 0), kResidentSmem, h))
         b += 4LL * (long long)(h.row.size() + h.ell_col.size() + h.jac.size() + h.rnd.size() +
                                h.rec.size() + h.bnd.size() + h.gat.size() + h.gsrc.size()) +
              16LL * (long long)h.ell_y.size() + (fp32 ? 2LL : 4LL) * (long long)h.jac.size();

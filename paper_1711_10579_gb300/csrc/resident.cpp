@@ -80,8 +80,9 @@ std::vector<std::vector<Item>> chains_of(std::vector<Item>& items) {
 }
 
 // part[i] of every row: 0 .. P-1, or P for the top.  The heaviest subtree's
-// root moves to the top until the subtrees balance over the P bins.
-void cut_tree(const Symbolic& s, int P, std::vector<int>& part) {
+// root moves to the top until the subtrees balance over the P bins.  A pivot of
+// d later neighbours weighs 12 + 4 d + quad d^2.
+void cut_tree(const Symbolic& s, int P, double quad, std::vector<int>& part) {
   const int n = s.n;
   part.assign(n, P > 1 ? P : 0);
   if (P == 1) return;
@@ -91,7 +92,7 @@ void cut_tree(const Symbolic& s, int P, std::vector<int>& part) {
   for (int k = 0; k < n; ++k) {
     const int d = s.lu_rowptr[k + 1] - s.lu_diag[k] - 1;
     if (d > 0) parent[k] = s.lu_col[s.lu_diag[k] + 1];
-    w[k] = 12.0 + 4.0 * d + (double)d * d;  // mismatch and Jacobian; sweeps; updates
+    w[k] = 12.0 + 4.0 * d + quad * d * d;  // mismatch and Jacobian; sweeps; updates
   }
   for (int k = 0; k < n; ++k) {
     sub[k] += w[k];
@@ -162,13 +163,13 @@ void cut_tree(const Symbolic& s, int P, std::vector<int>& part) {
 
 }  // namespace
 
-bool res_plan(const Symbolic& s, int P, int slots, ResPlanHost& out) {
+bool res_plan(const Symbolic& s, int P, int slots, double quad, ResPlanHost& out) {
   const int n = s.n, nnz = s.nnz_lu();
   out = ResPlanHost();
   out.P = P;
   out.slots = slots;
   std::vector<int> part;
-  cut_tree(s, P, part);
+  cut_tree(s, P, quad, part);
   const int Q = P > 1 ? P + 1 : 1;  // parts and the top
   std::vector<std::vector<int>> piv(Q), bnd(Q);
   for (int i = 0; i < n; ++i) piv[part[i]].push_back(i);
@@ -414,6 +415,16 @@ bool res_plan(const Symbolic& s, int P, int slots, ResPlanHost& out) {
     out.max_tab = std::max(out.max_tab, out.cta[0].ntab + A.rb + A.nrb - A.rf);
   }
   return true;
+}
+
+bool res_plan_fit(const Symbolic& s, bool fp32, int P, int slots, size_t limit, ResPlanHost& out) {
+  for (const double quad : {0.3, 1.0}) {
+    ResPlanHost h;
+    if (!res_plan(s, P, slots, quad, h) || res_smem(h, fp32) > limit) continue;
+    out = std::move(h);
+    return true;
+  }
+  return false;
 }
 
 }  // namespace pf

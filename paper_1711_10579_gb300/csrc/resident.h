@@ -126,7 +126,13 @@ inline size_t res_smem(const ResPlanHost& p, bool fp32) {
 // The plan of P CTAs of `slots` slots for an analysed case (2x2 blocks; an
 // exact factor, or with P = 1 an ILU(0) pattern); false if a part exceeds the
 // items' index ranges.
-bool res_plan(const Symbolic& s, int P, int slots, ResPlanHost& out);
+bool res_plan(const Symbolic& s, int P, int slots, double quad, ResPlanHost& out);
+// The plan that fits `limit` bytes of shared memory a CTA: cut by quad = 0.3,
+// which weighs the rows' assembly more than the blocks of the dense pivots, or
+// where a CTA's blocks then do not fit by quad = 1.  Measured (us, 0.3 / 1):
+// 10,000 buses mixed 431 / 463 and 500 / 545, 7,000 369 / 371, 2,749 FP64 495 /
+// 496, 10,000 FP64 1,303 / 1,347.
+bool res_plan_fit(const Symbolic& s, bool fp32, int P, int slots, size_t limit, ResPlanHost& out);
 
 // Launch of B scenarios on clusters of R.P CTAs (resident.cu); w holds the
 // state [scenario][row], and lin is set for batches: info.linear_iterations

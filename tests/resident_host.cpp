@@ -120,7 +120,7 @@ extern "C" int resident_check(int n, int m, const int* f, const int* t, int P, i
   if (ilu) analyze(y, Ordering::RCM, false, s);
   else analyze(y, Ordering::MinDegree, true, s);
   ResPlanHost p;
-  if (!res_plan(s, P, T, p)) return 100;
+  if (!res_plan(s, P, T, n % 2 ? 1.0 : 0.3, p)) return 100;
   *parts = 0;
   for (const ResPart& R : p.part) *parts += R.np > 0;
 
