@@ -296,7 +296,7 @@ int pf_solve(pf_case c, const pf_opts* opts, double* vmag, double* vang,
  * pattern (Newton-Raphson: one launch with each scenario's factor in the
  * shared memory of a CTA or cluster where it fits and the batch is small, else
  * phase kernels in one CUDA graph whose loop ends on the device when no
- * scenario runs; Newton-Krylov: one persistent launch).
+ * scenario runs; Newton-Krylov: one launch).
  * Scenario b uses p_load[b][*], q_load[b][*] (per bus or per slot; a load
  * scale per bus and scenario is these arrays scaled) and, single phase
  * only, p_gen[b][n]; NULL = the case's own values.  Outputs vmag[b][*],
@@ -480,8 +480,8 @@ int pf_branch_flows(pf_case c, int B, const double* vmag, const double* vang, do
  * out: the chosen shape, for PF_NR that of the factorisation, which alone
  * also applies to the sweeps when passed back explicitly), or 0, 0 where the
  * resident solves were faster than the phase kernels in those shapes.
- * Without tuning, a batch uses about one CTA per SM (at most 8 scenarios per
- * CTA), or the resident solves (pf_solve_batch).
+ * Without tuning, a batch uses about one CTA per SM (at most 32 scenarios per
+ * CTA; three phase and PF_NK 8), or the resident solves (pf_solve_batch).
  * Blocking; allocates the batch workspace.
  */
 int pf_autotune(pf_case c, int B, pf_opts* opts);
