@@ -251,10 +251,10 @@ __device__ __forceinline__ Blk<double> jac_block(const DevWork& w, int i, int j,
   return o;
 }
 
-// Diagonal Jacobian block of row i: V, I of the row, its mismatch power S and
-// loads, the Ybus diagonal.
+// Diagonal Jacobian block of row i: V and I of the row, its loads, the Ybus
+// diagonal.
 __device__ __forceinline__ Blk<float> diag_block(const DevSys& S, int i, int t, double2 Vi, double2,
-                                                 double vm, double2 I, double2, double pl, double ql,
+                                                 double vm, double2 I, double pl, double ql,
                                                  float2 y) {
   if (t == PF_SLACK) return {1.f, 0.f, 0.f, 1.f};
   const float vix = to_f32_trunc(Vi.x), viy = to_f32_trunc(Vi.y);
@@ -276,20 +276,37 @@ __device__ __forceinline__ Blk<float> diag_block(const DevSys& S, int i, int t, 
   return o;
 }
 __device__ __forceinline__ Blk<double> diag_block(const DevSys& S, int i, int t, double2 Vi,
-                                                  double2 Ui, double vm, double2 I, double2 Sc,
+                                                  double2 Ui, double vm, double2 I,
                                                   double pl, double ql, double2 y) {
   if (t == PF_SLACK) return {1.0, 0.0, 0.0, 1.0};
-  const double dshape = fma(2.0 * S.zip[3 * i + 2], vm, S.zip[3 * i + 1]);
+  // dS/d delta = j V conj(I - Y_ii V), dS/d|V| = U conj(I + Y_ii V) and the
+  // load's slope
   const double yvx = dot2(y.x, Vi.x, -y.y, Vi.y), yvy = dot2(y.x, Vi.y, y.y, Vi.x);
-  const double dx = dot2(Vi.x, yvx, Vi.y, yvy), dy = dot2(Vi.y, yvx, -Vi.x, yvy);
-  const double ax = I.x + yvx, ay = I.y + yvy;
-  const double ex = dot2(Ui.x, ax, Ui.y, ay), ey = dot2(Ui.y, ax, -Ui.x, ay);
-  Blk<double> o{-(Sc.y - dy), fma(pl, dshape, ex), Sc.x - dx, fma(ql, dshape, ey)};
+  const double ox = I.x - yvx, oy = I.y - yvy, ax = I.x + yvx, ay = I.y + yvy;
+  Blk<double> o{dot2(Vi.x, oy, -Vi.y, ox), dot2(Ui.x, ax, Ui.y, ay), dot2(Vi.x, ox, Vi.y, oy),
+                dot2(Ui.y, ax, -Ui.x, ay)};
+  const double zi = S.zip[3 * i + 1], zz = S.zip[3 * i + 2];
+  if (nonzero(zi, zz)) {
+    const double dshape = fma(2.0 * zz, vm, zi);
+    o.b = fma(pl, dshape, o.b);
+    o.d = fma(ql, dshape, o.d);
+  }
   if (t == PF_PV) {
     o.b = o.c = 0.0;
     o.d = 1.0;
   }
   return o;
+}
+
+// FP64 -> TF, to the nearest by integer instructions (ties away from zero;
+// infinities become NaN: their scenario has diverged).
+template <typename TF>
+__device__ __forceinline__ TF narrow(double v) {
+  if constexpr (sizeof(TF) == 8) {
+    return v;
+  } else {
+    return to_f32_trunc(__longlong_as_double(__double_as_longlong(v) + (1ll << 28)));
+  }
 }
 
 // The mismatch of Eq. 8-9 of this CTA's rows (into the right-hand side y and,
@@ -336,19 +353,21 @@ __device__ __forceinline__ unsigned long long assemble(const DevSys& S, const De
       I.y = fma(yv.y, v.x, I.y);
     }
     if (!on) continue;
-    const double2 Sc = make_double2(dot2(Vi.x, I.x, Vi.y, I.y), dot2(Vi.y, I.x, -Vi.x, I.y));
-    const double shape = fma(fma(zz, vmi, zi), vmi, zp);
-    const double f0 = (t != PF_SLACK) ? fma(-pl, shape, pg) - Sc.x : 0.0;
+    double shape = zp;
+    if (nonzero(zi, zz)) shape = load_shape(zz, zi, zp, vmi);
     const double qgen = (t == kPQLimit) ? w.qsw[i] : S.q_gen[i];
-    const double f1 = (t >= PF_PQ) ? fma(-ql, shape, qgen) - Sc.y : 0.0;
+    double f0 = fma(-Vi.x, I.x, fma(-Vi.y, I.y, fma(-pl, shape, pg)));
+    double f1 = fma(-Vi.y, I.x, fma(Vi.x, I.y, fma(-ql, shape, qgen)));
+    f0 = t != PF_SLACK ? f0 : 0.0;
+    f1 = t >= PF_PQ ? f1 : 0.0;
     if (keep_f) reinterpret_cast<double2*>(w.F)[i] = make_double2(f0, f1);
-    reinterpret_cast<V2*>(y)[r.z] = mk2((TF)f0, (TF)f1);
+    reinterpret_cast<V2*>(y)[r.z] = mk2(narrow<TF>(f0), narrow<TF>(f1));
     m = max(m, max(abs_bits(f0), abs_bits(f1)));
     Blk<TF> D;
     if constexpr (sizeof(TF) == 4) {
-      D = diag_block(S, i, t, Vi, Vi, vmi, I, Sc, pl, ql, __ldg(R.diag32 + rl));
+      D = diag_block(S, i, t, Vi, Vi, vmi, I, pl, ql, __ldg(R.diag32 + rl));
     } else {
-      D = diag_block(S, i, t, Vi, ld_state<CL>(w.U + i), vmi, I, Sc, pl, ql, yd);
+      D = diag_block(S, i, t, Vi, ld_state<CL>(w.U + i), vmi, I, pl, ql, yd);
     }
     if (jm) st_blk(jm + 4 * (size_t)r.w, D);
     if ((r.x & kResRowLevel0) && !inv2(D)) *bad = true;
