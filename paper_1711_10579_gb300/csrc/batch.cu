@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(kRowThreads, (BS == 2 && sizeof(TF) == 4) ? 5 
       if constexpr (BS == 6) {
         mismatch_jacobian_3ph<TF>(S, w, i, t.gs, nrm, nullptr);
       } else {
-        mismatch_jacobian_1ph<TF>(S, w, i, t.gs, nrm, nullptr);
+        mismatch_jacobian_1ph<TF, true>(S, w, i, t.gs, nrm, nullptr);
       }
       m = max(m, abs_bits(nrm));
     }

@@ -267,8 +267,10 @@ __device__ __forceinline__ bool nonzero(double a, double b) {
 // has no unknown and PV buses no |V| unknown: their rows become identity rows
 // and their columns zero, which keeps the system of Eq. 10 unchanged.  With
 // reactive limits enforced the types are the scenario's (w.bt): a PV bus at
-// its limit is PQ with generation w.qsw.
-template <typename TF>
+// its limit is PQ with generation w.qsw.  LEAN: the batched kernel's mismatch.
+// The persistent kernel keeps the other rounding: a mixed Newton-Krylov step can
+// end so close to the limit that the last bits decide whether one more follows.
+template <typename TF, bool LEAN>
 __device__ void mismatch_jacobian_1ph(const DevSys& S, const DevWork& w, int i, int gs,
                                       double& nrm, TF* jcopy) {
   const int B = w.B;
@@ -293,18 +295,27 @@ __device__ void mismatch_jacobian_1ph(const DevSys& S, const DevWork& w, int i, 
   // FP64 mismatch of Eq. 8-9 from the current I = sum_j Y_ij V_j and S = V
   // conj(I): the operations of a row are what the batched kernel takes its time
   // for, so only the bus type's equations are formed (the lanes of a warp share
-  // the row) and constant-power loads take no polynomial.
+  // the row) and constant-power loads take no polynomial (10,000 buses x 9,728
+  // mixed, 6 evaluations: 28.7 -> 26.0 ms; x 608 FP64 5.7 -> 4.7 ms).
   double2 I = make_double2(0.0, 0.0);
   auto mismatch = [&]() {
     double f0 = 0.0, f1 = 0.0;
-    if (t != PF_SLACK) {
-      double shape = zp;
-      if (nonzero(zi, zz)) shape = load_shape(zz, zi, zp, vmi);
-      f0 = fma(-Vi.x, I.x, fma(-Vi.y, I.y, fma(-pl, shape, pg)));
-      if (t >= PF_PQ) {
-        const double qgen = (t == kPQLimit) ? __ldcg(w.qsw + b) : S.q_gen[i];
-        f1 = fma(-Vi.y, I.x, fma(Vi.x, I.y, fma(-ql, shape, qgen)));
+    if constexpr (LEAN) {
+      if (t != PF_SLACK) {
+        double shape = zp;
+        if (nonzero(zi, zz)) shape = load_shape(zz, zi, zp, vmi);
+        f0 = fma(-Vi.x, I.x, fma(-Vi.y, I.y, fma(-pl, shape, pg)));
+        if (t >= PF_PQ) {
+          const double qgen = (t == kPQLimit) ? __ldcg(w.qsw + b) : S.q_gen[i];
+          f1 = fma(-Vi.y, I.x, fma(Vi.x, I.y, fma(-ql, shape, qgen)));
+        }
       }
+    } else {
+      const double2 Sc = cmulc(Vi, I);
+      const double shape = fma(fma(zz, vmi, zi), vmi, zp);
+      const double qgen = (t == kPQLimit) ? __ldcg(w.qsw + b) : S.q_gen[i];
+      f0 = (t != PF_SLACK) ? fma(-pl, shape, pg) - Sc.x : 0.0;
+      f1 = (t >= PF_PQ) ? fma(-ql, shape, qgen) - Sc.y : 0.0;
     }
     w.F[b * 2] = f0;
     w.F[b * 2 + 1] = f1;
@@ -1262,7 +1273,8 @@ struct FactorPipe {
 // next step's first records are requested before each barrier.  FP64 is bound
 // by its pipe (a warp instruction per 64 cycles and sub-partition), so a
 // pivot's block is inverted once, by the item that updates it last (a level
-// earlier), not for each of its L entries: @@
+// earlier), not for each of its L entries: with the items sorted by work, 5
+// factorisations of 10,000 buses x 608 take 9.5 ms instead of 12.9 ms.
 template <typename TF>
 __device__ __noinline__ void factor_pipe(const FactorArgs<TF> S, const Team tm, int l0, int l1) {
   if (l0 >= l1) return;

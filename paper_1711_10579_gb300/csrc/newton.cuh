@@ -122,7 +122,7 @@ __device__ __forceinline__ void newton_solve(const DevSys& S, const DevWork& w, 
       if constexpr (THREE) {
         mismatch_jacobian_3ph<TF>(S, w, i, gs, nrm, jcopy);
       } else {
-        mismatch_jacobian_1ph<TF>(S, w, i, gs, nrm, jcopy);
+        mismatch_jacobian_1ph<TF, false>(S, w, i, gs, nrm, jcopy);
       }
       return nrm;
     });
