@@ -360,8 +360,8 @@ int pf_drain(pf_ctx ctx, int timeout_ms);
  * launch shape) run as group launches: one launch solves several queued
  * requests of any cases and sizes, on the cluster of a resident single solve
  * of the case where its factor fits shared memory, else on one CTA each (a
- * cluster of 8 CTAs for grids of 4,000 buses or feeders of 2,000 nodes and
- * more),
+ * cluster of 2 to 8 CTAs for grids of 4,000 buses or feeders of 2,000 nodes and
+ * more, by size and by how many CTAs are in flight),
  * and each request retires when its own solve ends.  Runs of queued requests of one case are coalesced into batched
  * solves (pf_submit).  Newton-Krylov requests and requests with reactive
  * limits run as one launch each.

@@ -5,7 +5,7 @@
 // queued request that fits (free job slots and the context's HBM budget),
 // of any cases and sizes, and each of its CTAs or clusters solves one request
 // on its own: the resident solve of the case where it has one (resident.cu,
-// feeder.cu), else newton.cuh's (newton_group_kernel), the largest on 8-CTA
+// feeder.cu), else newton.cuh's (newton_group_kernel), the largest on
 // clusters; each kernel and launch shape is a launch of its own.  A job's
 // descriptor, inputs and outputs
 // live in pinned host memory; the CTA raises the job's done flag when its
@@ -46,10 +46,19 @@ constexpr int kSlots = 8;         // per-request launches (Newton-Krylov, reacti
 constexpr size_t kMaxQueue = 1 << 20;
 constexpr size_t kGroupSmemMax = 200 * 1024;  // a job's solve vector in shared memory up to this
 // Requests without a resident plan of at least this many rows (buses; nodes of
-// a feeder) run on a cluster of kBigCluster CTAs instead of one CTA: they are
-// the tail of the latency (8,000 nodes mixed: 14.5 / 9.6 / 6.4 / 4.8 ms on 1 /
-// 2 / 4 / 8 CTAs; a 37,000-bus grid 29.5 / 22.9 / 17.5 / 15.4 ms).
+// a feeder) run on a cluster of CTAs instead of one CTA: they are the tail of
+// the latency (8,000 nodes mixed: 14.5 / 9.6 / 6.4 / 4.8 ms on 1 / 2 / 4 / 8
+// CTAs; a 37,000-bus grid 29.5 / 22.9 / 17.5 / 15.4 ms).  While the CTAs in
+// flight make at most kWaves waves they take kBigCluster; a wide cluster costs
+// more CTA time, so beyond that 2 CTAs from kBigRows*, 4 from kMidRows* and
+// kBigCluster from kHugeRows*.  Measured: 24 requests of twelve grids (up to
+// 10,000 buses) 4.5 ms wide, 6.4 ms narrow; 2,000 requests a second of grids to
+// 65,000 buses: always wide 1,723 solves/s and a growing queue, by this rule
+// sustained (p50 5.1 ms, p99 41 ms; always narrow 4.4 and 40 ms).
 constexpr int kBigRows1ph = 4000, kBigRows3ph = 2000, kBigCluster = 8;
+constexpr int kMidRows1ph = 16000, kMidRows3ph = 5000;
+constexpr int kHugeRows1ph = 40000, kHugeRows3ph = 12000;
+constexpr double kWaves = 1.5;
 
 // Coalesced batches: kBatchMin or more queued Newton-Raphson requests of one
 // case with the same solve options and their own loads run as one batched
@@ -76,11 +85,14 @@ bool grouped(const Request& r) {
          !r.o.block_threads && !r.o.scen_per_cta && !r.o.cluster_size;
 }
 
-// CTAs of a request that the group kernel of newton.cuh solves.
-int group_cluster(const Request& r) {
-  return r.c->data.n >= (r.c->data.kind == PF_SINGLE_PHASE ? kBigRows1ph : kBigRows3ph)
-             ? kBigCluster
-             : 1;
+// CTAs of a request that the group kernel of newton.cuh solves (busy: more
+// than kWaves waves in flight).
+int group_cluster(const Request& r, bool busy) {
+  const bool one = r.c->data.kind == PF_SINGLE_PHASE;
+  const int n = r.c->data.n;
+  if (n < (one ? kBigRows1ph : kBigRows3ph)) return 1;
+  if (!busy || n >= (one ? kHugeRows1ph : kHugeRows3ph)) return kBigCluster;
+  return n >= (one ? kMidRows1ph : kMidRows3ph) ? 4 : 2;
 }
 
 size_t slots_of(const Request& r) {
@@ -118,6 +130,7 @@ struct Job {
   Staging io;
   Request* req = nullptr;
   int stream = -1;
+  int ctas = 0;  // of its launch
   bool warm_in = false, warm_out = false;
   int want_n = 0;  // sizes to grow the buffers to (largest case of the kind seen)
   long long want_nnz = 0;
@@ -423,6 +436,9 @@ struct Server {
       any = true;
     }
     if (claimed.empty()) return any;
+    int ctas = 0;  // in flight
+    for (int k = 0; k < kJobs; ++k)
+      if (jobs[k].req && jobs[k].stream >= 0) ctas += jobs[k].ctas;
     // one launch per kernel and launch shape
     struct Group {
       GroupList list;
@@ -447,7 +463,9 @@ struct Server {
       Group want;
       want.bs = r->c->bs;
       want.fp32 = r->o.precision == PF_MIXED;
-      want.cluster = plan ? plan->P : group_cluster(*r);
+      want.cluster = plan ? plan->P : group_cluster(*r, ctas + kBigCluster > kWaves * ctx->num_sms);
+      jobs[k].ctas = want.cluster;
+      ctas += want.cluster;
       want.threads = plan ? plan->threads : 0;
       want.list.n = 0;
       auto it = std::find_if(grp.begin(), grp.end(), [&](const Group& g) {
