@@ -1238,8 +1238,10 @@ __device__ __forceinline__ bool finite_bits(double x) {
   return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;
 }
 
-// U_kk^-1 of a 2x2 block, adjugate over determinant; false for a zero or
-// non-finite determinant or inverse (1 / 0 leaves no entry finite).
+// U_kk^-1 of a 2x2 block, adjugate over determinant; false for a zero
+// determinant or a non-finite inverse (1 / 0 leaves no entry finite).  The
+// determinant has the square of the entries' range: FP32 blocks below about
+// 1e-19 count as singular, and above about 1e19 the inverse is zero.
 template <typename TF>
 __device__ __forceinline__ bool inv_2x2(const TF (&a)[4], TF (&di)[4]) {
   const TF det = a[0] * a[3] - a[1] * a[2];
@@ -1249,6 +1251,19 @@ __device__ __forceinline__ bool inv_2x2(const TF (&a)[4], TF (&di)[4]) {
   di[2] = -a[2] * rd;
   di[3] = a[0] * rd;
   return finite_bits(di[0]) && finite_bits(di[1]) && finite_bits(di[2]) && finite_bits(di[3]);
+}
+
+// factor_pipe's U_kk^-1.  FP32: the elimination with row exchanges of
+// factor_run, for blocks of any size, so that a mixed batch rounds as it does
+// there; the last FP32 step of a solve is not always refined, and two roundings
+// of the inverse put voltages of the same mismatch up to 1e-7 apart.  FP64: the
+// adjugate (1e-13 apart).
+__device__ __forceinline__ bool inv_pipe(const float (&a)[4], float (&di)[4]) {
+  float t[4] = {a[0], a[1], a[2], a[3]};
+  return blk_inv<2>(t, di);
+}
+__device__ __forceinline__ bool inv_pipe(const double (&a)[4], double (&di)[4]) {
+  return inv_2x2(a, di);
 }
 
 // The pivot whose diagonal block a target record finishes (-1: none), from the
@@ -1353,7 +1368,7 @@ __device__ __noinline__ void factor_pipe(const FactorArgs<TF> S, const Team tm, 
     bool ok = true;
     if (!r.w) {
       const TF a[BB] = {di[0], di[1], di[2], di[3]};
-      ok = inv_2x2(a, di);
+      ok = inv_pipe(a, di);
     }
     if (r.x == r.z) {
       if (!ok) S.flag[gs] = 1;
@@ -1399,7 +1414,7 @@ __device__ __noinline__ void factor_pipe(const FactorArgs<TF> S, const Team tm, 
       blk_store<2>(gblk(r.x & ~kFillFirst), c);
     } else {  // only its inverse is read from here on
       TF di[BB];
-      if (!inv_2x2(c, di)) S.flag[gs] = 1;
+      if (!inv_pipe(c, di)) S.flag[gs] = 1;
       blk_store<2>(S.uinv + ((size_t)k * S.B + gs) * BB, di);
     }
   };

@@ -1,4 +1,6 @@
 """The phase kernels of batches (explicit shapes): factorisation and sweeps."""
+import dataclasses
+
 import numpy as np
 import pytest
 
@@ -35,6 +37,33 @@ def test_phase_kernels_match_oracle(env, n, S, B, prec):
         vm, va, info = pf.pf_solve_batch(c, pl, ql, pg, o)
         assert np.all(info["status"] == 0) and np.all(info["mismatch"] <= 1e-8)
         for b in (0, B // 2, B - 1):
+            r = O.newton_polar(case.with_loads(pl[b], ql[b], pg[b]))
+            assert np.max(np.abs(vm[b] - r["vm"])) <= 1e-6
+            assert np.max(np.abs(va[b] - r["va"])) <= 1e-6
+    finally:
+        pf.pf_destroy_case(c)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("S", [1, 2, 4, 8, 16])
+def test_mixed_batch_in_a_large_power_base(env, S):
+    """The same grid per unit of a power base 1e22 times larger: admittances and
+    powers of 1e-22, whose 2x2 determinants are below the FP32 range.  The
+    voltages are the oracle's in the ordinary base, within 1e-6."""
+    pf, ctx = env
+    case = mesh(33)
+    k = 1e-22
+    small = dataclasses.replace(case, br_r=case.br_r / k, br_x=case.br_x / k, br_b=case.br_b * k,
+                                p_load=case.p_load * k, q_load=case.q_load * k,
+                                p_gen=case.p_gen * k, q_gen=case.q_gen * k)
+    B = 2 * S + 1
+    pl, ql, pg = cases.scenario_loads(case, B, seed=5)
+    c = pf.pf_create_case(ctx, small)
+    try:
+        o = pf.make_opts(precision=pf.PF_MIXED, scen_per_cta=S, tol=1e-8 * k)
+        vm, va, info = pf.pf_solve_batch(c, pl * k, ql * k, pg * k, o)
+        assert np.all(info["status"] == 0)
+        for b in (0, B - 1):
             r = O.newton_polar(case.with_loads(pl[b], ql[b], pg[b]))
             assert np.max(np.abs(vm[b] - r["vm"])) <= 1e-6
             assert np.max(np.abs(va[b] - r["va"])) <= 1e-6
