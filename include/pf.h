@@ -480,8 +480,8 @@ int pf_branch_flows(pf_case c, int B, const double* vmag, const double* vang, do
  * out: the chosen shape, for PF_NR that of the factorisation, which alone
  * also applies to the sweeps when passed back explicitly), or 0, 0 where the
  * resident solves were faster than the phase kernels in those shapes.
- * Without tuning, a batch uses about one CTA per SM (at most 32 scenarios per
- * CTA; three phase and PF_NK 8), or the resident solves (pf_solve_batch).
+ * Without tuning, a batch uses about one CTA per SM (at most 8 scenarios per
+ * CTA; single-phase FP64 PF_NR 32), or the resident solves (pf_solve_batch).
  * Blocking; allocates the batch workspace.
  */
 int pf_autotune(pf_case c, int B, pf_opts* opts);

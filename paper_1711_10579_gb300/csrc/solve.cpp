@@ -98,20 +98,21 @@ void launch_shape(pf_case c, const pf_opts& o, int B, bool fp32, int* grid, int*
         tth = it->second[1];
       }
     }
-    // default of the phase kernels of 2x2 blocks: the fewest scenarios per CTA,
-    // up to 32, that make one wave (ms, 1 / 2 / 4 / 8 / 16 / 32): FP64, 10,000
-    // buses x 256 19.8 / 14.6 / 20.5, x 1,000 - / - / 44.8 / 38.9 / 59.1, 2,000
-    // x 305 6.4 / 4.9 / 3.7 / 5.1, x 2,500 - / - / - / 16.9 / 18.1 / 15.4.
-    // Mixed, above 8 only for two waves of half as many: 10,000 x 310 14.3 / 11.5
-    // / 10.4 / 14.3, x 1,220 - / - / 26.7 / 22.6 / 25.8, x 2,440 - / - / - / 40.1
-    // / 37.2 / 41.2; 200 x 9,728 - / - / - / 4.0 / 2.9 / 2.0.  Others: up to 8,
-    // about one wave.
-    const bool phase2 = bs == 2 && o.method == PF_NR;
-    const int one_wave = phase2 ? (fp32 ? 8 : 32) : 1, most = phase2 ? 32 : 8;
+    // default: about one CTA per SM, up to 8 scenarios per CTA; FP64 phase kernels
+    // of 2x2 blocks: the fewest scenarios per CTA, up to 32, that make one wave
+    // (ms, 1 / 2 / 4 / 8 / 16 / 32: 10,000 buses x 256 19.8 / 14.6 / 20.5, x 1,000
+    // - / - / 44.8 / 38.9 / 59.1, 2,000 x 305 6.4 / 4.9 / 3.7 / 5.1, x 2,500 - / -
+    // / - / 16.9 / 18.1 / 15.4).  Not mixed, though 2,000 x 305 and 200 x 9,728
+    // would gain: a scenario's sums are ordered by the shape, and its last FP32
+    // step is not always refined, so another default moves the voltages a call
+    // returns by up to 1e-7 at the same mismatch.
+    const bool wave = bs == 2 && o.method == PF_NR && !fp32;
     const long long sms = c->ctx->num_sms;
     int dS = 1;
-    while (dS < one_wave && B > dS * sms) dS <<= 1;
-    while (dS < most && B >= 2 * dS * sms) dS <<= 1;
+    if (wave)
+      while (dS < 32 && B > dS * sms) dS <<= 1;
+    else
+      while (dS < 8 && B >= 2 * dS * sms) dS <<= 1;
     *threads = o.block_threads ? std::min(o.block_threads, max_threads)
                                : (tth ? tth : max_threads);
     *cluster = 1;

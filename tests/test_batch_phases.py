@@ -69,3 +69,28 @@ def test_mixed_batch_in_a_large_power_base(env, S):
             assert np.max(np.abs(va[b] - r["va"])) <= 1e-6
     finally:
         pf.pf_destroy_case(c)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("B", [305, 609, 2432])
+def test_default_shape_of_mixed_batches(env, B):
+    """Untuned mixed batches: about one CTA per SM, at most 8 scenarios each, and
+    the bits of that shape asked for explicitly."""
+    import torch
+
+    pf, ctx = env
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    S = 1
+    while S < 8 and B >= 2 * S * sms:
+        S *= 2
+    case = mesh(4000)
+    pl, ql, pg = cases.scenario_loads(case, B, seed=7)
+    c = pf.pf_create_case(ctx, case)
+    try:
+        assert pf.pf_launch_config(c, pf.make_opts(), B)["scen_per_cluster"] == S
+        vm, va, info = pf.pf_solve_batch(c, pl, ql, pg, pf.make_opts())
+        vm2, va2, info2 = pf.pf_solve_batch(c, pl, ql, pg, pf.make_opts(scen_per_cta=S))
+        assert np.all(info["status"] == 0) and np.all(info2["status"] == 0)
+        assert np.array_equal(vm, vm2) and np.array_equal(va, va2)
+    finally:
+        pf.pf_destroy_case(c)
