@@ -141,9 +141,12 @@ typedef struct {
   int gmres_max_iter; /* NK: inner iterations per Newton step; default 300 */
   double gmres_rtol;  /* NK: inner relative-residual floor; default 1e-6 */
   int warm_start;     /* 1 = start from the case's last converged voltages */
-  int cluster_size;   /* single-solve launch: CTAs per cluster (0 = chosen by
-                         size); with block_threads and scen_per_cta 0 also the
-                         CTAs per scenario of a resident batch */
+  int cluster_size;   /* CTAs per cluster of a single solve (0 = chosen by size).
+                         With block_threads and scen_per_cta 0 it asks PF_NR for
+                         resident solves (pf_solve_batch) of that many CTAs per
+                         scenario, for grids in mixed precision too, whose
+                         voltages then differ from the default's by up to 4e-7
+                         (relative) within the same tol */
   int block_threads;  /* threads per CTA (0 = autotuned) */
   int scen_per_cta;   /* batched launch: scenarios per CTA (0 = autotuned) */
   int nk_fallback;    /* PF_NK through pf_solve / pf_solve_batch: redo every
@@ -293,10 +296,11 @@ int pf_solve(pf_case c, const pf_opts* opts, double* vmag, double* vang,
 
 /*
  * B scenarios of one topology solved together over the shared symbolic
- * pattern (Newton-Raphson: one launch with each scenario's factor in the
- * shared memory of a CTA or cluster where it fits and the batch is small, else
- * phase kernels in one CUDA graph whose loop ends on the device when no
- * scenario runs; Newton-Krylov: one launch).
+ * pattern (Newton-Raphson: one launch of resident solves, each scenario's factor
+ * in the shared memory of a CTA or cluster, where it fits and the batch is small,
+ * in mixed precision up to 32 buses or 1,000 nodes; else phase kernels in one
+ * CUDA graph whose loop ends on the device when no scenario runs;
+ * Newton-Krylov: one launch).
  * Scenario b uses p_load[b][*], q_load[b][*] (per bus or per slot; a load
  * scale per bus and scenario is these arrays scaled) and, single phase
  * only, p_gen[b][n]; NULL = the case's own values.  Outputs vmag[b][*],

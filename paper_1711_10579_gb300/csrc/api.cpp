@@ -342,12 +342,26 @@ static int feeder_least(int n, bool fp32) {
   return 0;
 }
 
+// Mixed-precision cases of more rows stay on the kernels of newton.cuh and
+// batch.cu unless the caller asks for CTAs per scenario.  A mixed solve stops
+// after an FP32 step that is refined only where convergence stalls, so at the
+// same mismatch its voltages depend on the order of the FP32 sums.  Against
+// those kernels (relative, largest of a solve): grids of 14-32 buses at most
+// 3.9e-8 (170 grids x 1,200 load scenarios), of 33-130 1.4e-7, of 3,824 3.3e-7;
+// feeders of 300-1,050 nodes 3.0e-8 (330 feeders x 64), of 1,100-2,000 1.4e-7.
+constexpr int kMixedRows1ph = 32, kMixedRows3ph = 1000;
+
+static bool resident_default(int n, bool fp32, bool three) {
+  return !fp32 || n <= (three ? kMixedRows3ph : kMixedRows1ph);
+}
+
 // Single solves: latency, so more CTAs than memory asks for, one per 400
 // rows (feeders: 100 nodes).  Measured (us, P = 1 / 2 / 4 / 8 / 16): 500 buses
 // mixed 140 / 145 / 133 / 140 / 180; 2,749 buses FP64 - / - / 770 / 657 / 641;
 // feeders of 100 nodes mixed 143 / 170 / 157 / 161 / 184, of 400 314 / 259 /
 // 215 / 231 / 257, of 1,000 FP64 - / 1,343 / 1,044 / 1,060 / 919.
 int resident_single(const Symbolic& s, bool fp32, bool three) {
+  if (!resident_default(s.n, fp32, three)) return 0;
   int P = three ? feeder_least(s.n, fp32) : resident_least(s, fp32);
   while (P > 0 && P < 16 && s.n > (three ? 100 : 400) * P) P <<= 1;
   return P;
@@ -364,14 +378,13 @@ int resident_single(const Symbolic& s, bool fp32, bool three) {
 // Resident up to 8 clusters per resident CTA of the GPU, whatever the batch
 // where 8 fit an SM; beyond, the phase kernels' 32 scenarios per warp win.
 // Measured (ms, resident against phase kernels in their best shape): mixed, 14
-// buses x 9,728 0.26 / 0.43, 200 x 9,728 1.76 / 2.01, 500 x 2,000 0.96 / 1.79
-// and x 9,728 4.7 / 4.0, 1,000 x 2,400 2.17 / 3.10, 2,000 x 1,000 2.40 / 3.47
-// and x 3,000 6.8 / 7.0, 5,000 (4 CTAs) x 256 3.4 / 4.7 and x 1,000 11.9 / 8.3;
-// FP64, 60 x 9,728 1.40 / 1.46, 200 x 3,000 1.70 / 2.15 and x 9,728 5.4 / 4.7,
-// 500 x 2,000 2.98 / 3.80, 1,000 x 1,200 3.9 / 4.3 and x 2,400 7.9 / 7.1, 2,000
-// (2 CTAs) x 256 3.2 / 4.2 and x 1,000 11.0 / 7.7.
+// buses x 9,728 0.26 / 0.43; FP64, 60 x 9,728 1.40 / 1.46, 200 x 3,000 1.70 /
+// 2.15 and x 9,728 5.4 / 4.7, 500 x 2,000 2.98 / 3.80, 1,000 x 1,200 3.9 / 4.3
+// and x 2,400 7.9 / 7.1, 2,000 (2 CTAs) x 256 3.2 / 4.2 and x 1,000 11.0 / 7.7.
 ResidentShape resident_batch(const Symbolic& s, bool fp32, bool three, int B, int num_sms, int P) {
   const bool asked = P > 0;  // CTAs per scenario given by the caller
+  if (!resident_default(s.n, fp32, three) && (three || !asked)) return {0, 0};
+  if (B == 1) return {P, 0};
   if (three) {
     // feeders: CTAs of at most 256 nodes, so that two fit an SM.  Measured (ms,
     // resident against phase kernels): 1,000 nodes mixed x 500 3.6 / 4.7, FP64
@@ -485,15 +498,8 @@ int SysBuf::upload_resident(const Ybus& y, bool fp32, ResidentPlan& r) {
   return PF_OK;
 }
 
-// Mixed-precision feeders of more nodes stay on the persistent kernel: its
-// voltages there are up to 1.3e-7 (relative) off the solution (170 feeders of
-// 2,000-4,000 nodes; up to 2.8e-8 below 2,000), and this kernel's, which are a
-// hundred times closer, would move what such a call returns by as much.
-constexpr int kFeederMixedMax = 2000;
-
 int SysBuf::upload_feeder(const Ybus& y, bool fp32, ResidentPlan& r) {
   FeedPlanHost h;
-  if (fp32 && sym.n > kFeederMixedMax) return PF_OK;
   if (!feed_plan(sym, bus_type, r.P, r.threads / kFeedLanes, h)) return PF_OK;
   r.smem = feed_smem(h, fp32);
   if (r.smem > kResidentSmem || feeder_clusters(fp32, r.P, r.threads, r.smem) < 1) return PF_OK;

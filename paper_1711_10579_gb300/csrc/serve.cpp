@@ -662,11 +662,15 @@ struct Server {
     // it, and never write it
     if (!c->warm_valid || warm_writers[c] > 0) o.warm_start = 0;
     // per-request solves without a resident plan run on 8-CTA clusters so that
-    // every slot fits
+    // every slot fits (in full CTAs: a cluster size alone asks for a resident
+    // solve)
     const ResidentPlan* plan = nullptr;
     rc = resident_plan(c, o, 1, RunMode::Solve, &plan);
     if (rc != PF_OK) return rc;
-    if (!o.cluster_size && !plan) o.cluster_size = 8;
+    if (!o.cluster_size && !plan) {
+      o.cluster_size = 8;
+      if (!o.block_threads) o.block_threads = 512;
+    }
     rc = run_solve_q(c, o, 1, d_in[0], d_in[1], d_in[2], &ws, s.st, nullptr, nullptr, nullptr,
                      /*warm_out=*/false);
     if (rc != PF_OK) return rc;

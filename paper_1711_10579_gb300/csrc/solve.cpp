@@ -122,9 +122,9 @@ void launch_shape(pf_case c, const pf_opts& o, int B, bool fp32, int* grid, int*
 }
 
 // The resident plan a solve runs on, or null: Newton-Raphson on a grid (or a
-// radial feeder) whose factor fits the shared memory of a cluster, GMRES on a
-// grid whose ILU(0) factor fits one CTA's, with no explicit shape of the other
-// kernels asked for.
+// radial feeder) whose factor fits the shared memory of a cluster (mixed: small
+// ones, resident_single), GMRES on a grid whose ILU(0) factor fits one CTA's,
+// with no explicit shape of the other kernels asked for.
 int resident_plan(pf_case c, const pf_opts& o, int B, RunMode mode, const ResidentPlan** out) {
   *out = nullptr;
   if (mode != RunMode::Solve || o.block_threads || o.scen_per_cta) return PF_OK;
@@ -152,8 +152,7 @@ int resident_plan(pf_case c, const pf_opts& o, int B, RunMode mode, const Reside
     return PF_OK;
   }
   const ResidentShape shape =
-      B == 1 ? ResidentShape{o.cluster_size, 0}
-             : resident_batch(c->nr.sym, fp32, c->bs == 6, B, c->ctx->num_sms, o.cluster_size);
+      resident_batch(c->nr.sym, fp32, c->bs == 6, B, c->ctx->num_sms, o.cluster_size);
   return c->nr.resident_for(c->y, fp32, shape, out);
 }
 

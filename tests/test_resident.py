@@ -200,6 +200,51 @@ def test_resident_batch_threads(env, n, B, prec):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("kind,n", [("mesh", 33), ("mesh", 500), ("mesh", 3906), ("feeder", 1106)])
+def test_mixed_solves_keep_their_kernels(env, kind, n):
+    """Mixed solves of more than 32 buses or 1,000 nodes: alone, in a batch, served
+    and under reactive limits the bits of the persistent and the phase kernels
+    (explicit threads), whose FP32 sums are in another order than the resident
+    kernels'."""
+    pf, ctx = env
+    B = 4
+    if kind == "mesh":
+        case = cases.with_q_limits(mesh(n), 2)
+        loads = cases.scenario_loads(case, B, seed=3)
+        full = 512
+    else:
+        case = cases.feeder_case(n, 43)
+        loads = (*[a.reshape(B, -1) for a in cases.feeder_scenario_loads(case, B, seed=3)], None)
+        full = 256
+    one = [None if a is None else a[:1] for a in loads]
+    row = [None if a is None else a[0] for a in loads]
+    c = pf.pf_create_case(ctx, case)
+    try:
+        def same(x, y):
+            assert np.all(x[2]["status"] == 0) and np.all(y[2]["status"] == 0)
+            assert np.array_equal(x[0], y[0]) and np.array_equal(x[1], y[1])
+
+        alone = pf.pf_solve_batch(c, *one, pf.make_opts())
+        same(alone, pf.pf_solve_batch(c, *one, pf.make_opts(block_threads=full)))
+        same(pf.pf_solve(c, pf.make_opts()), pf.pf_solve(c, pf.make_opts(block_threads=full)))
+        same(pf.pf_solve_batch(c, *loads, pf.make_opts()),
+             pf.pf_solve_batch(c, *loads, pf.make_opts(scen_per_cta=1)))
+        t = pf.pf_submit(ctx, c, *row, pf.make_opts())
+        pf.pf_drain(ctx)
+        vm, va, info = pf.pf_poll(ctx, t, c.slots)
+        same((vm, va, info), (alone[0][0], alone[1][0], {"status": alone[2]["status"][0]}))
+        if kind == "mesh":
+            limited = pf.pf_solve_batch(c, *one, pf.make_opts(q_limits=1))
+            same(limited, pf.pf_solve_batch(c, *one, pf.make_opts(q_limits=1, block_threads=full)))
+            t = pf.pf_submit(ctx, c, *row, pf.make_opts(q_limits=1))
+            pf.pf_drain(ctx)
+            vm, va, info = pf.pf_poll(ctx, t, c.slots)
+            same((vm, va, info), (limited[0][0], limited[1][0], {"status": limited[2]["status"][0]}))
+    finally:
+        pf.pf_destroy_case(c)
+
+
+@pytest.mark.gpu
 def test_resident_reports_failures(env):
     """A scenario past the loading nose next to one that converges, and an
     iteration limit."""
