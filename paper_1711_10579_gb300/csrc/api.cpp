@@ -16,6 +16,7 @@
 #include <vector>
 
 #include "api_internal.h"
+#include "records.h"
 
 namespace pf {
 
@@ -69,73 +70,6 @@ static cudaError_t upload(DevBuffer& buf, const std::vector<T>& v, const T** out
 // ---------------------------------------------------------------------------
 // system upload
 // ---------------------------------------------------------------------------
-
-// The kernels' packed records of a symbolic analysis, one 16-byte load per
-// item: forward / backward sweep rows {row, first entry, end, 0} in level
-// order; factor items {entry, pivot k, diagonal entry of k, whether an earlier
-// target finishes that entry}; targets {entry (| kFillFirst when a fill entry
-// gets its first update, which then starts from zero), first L entry, first U
-// entry, start of the rest in `con` or a mark}; `con` holds the other (L, U)
-// pairs of a target, each list ended by (-1, mark) (most targets receive one
-// update per level).  The mark is -1, or -2 - k where the target is the last
-// update of pivot k's diagonal entry.
-static void pack_records(const Symbolic& s, std::vector<int4>& fwd, std::vector<int4>& bwd,
-                         std::vector<int4>& fac, std::vector<int4>& tgt, std::vector<int2>& con) {
-  const int n = s.n;
-  fwd.assign(n, make_int4(0, 0, 0, 0));
-  bwd.assign(n, make_int4(0, 0, 0, 0));
-  fac.assign(s.fac_items.size(), make_int4(0, 0, 0, 0));
-  tgt.assign(s.tgt_entry.size(), make_int4(0, 0, 0, 0));
-  for (int t = 0; t < n; ++t) {
-    const int i = s.flev_rows[t], j = s.blev_rows[t];
-    fwd[t] = make_int4(i, s.lu_rowptr[i], s.lu_diag[i], 0);
-    bwd[t] = make_int4(j, s.lu_diag[j] + 1, s.lu_rowptr[j + 1], 0);
-  }
-  for (size_t t = 0; t < fac.size(); ++t) {
-    const int e = s.fac_items[t], k = s.lu_col[e];
-    fac[t] = make_int4(e, k, s.lu_diag[k], 0);
-  }
-  con.clear();
-  std::vector<char> touched(s.nnz_lu(), 0);
-  std::vector<int> last(n, -1);  // target of a pivot's last update
-  for (size_t t = 0; t < tgt.size(); ++t) {
-    const int k = s.lu_col[s.tgt_entry[t]];
-    if (s.tgt_entry[t] == s.lu_diag[k]) last[k] = (int)t;
-  }
-  for (int4& f : fac) f.w = last[f.y] >= 0;
-  for (size_t t = 0; t < tgt.size(); ++t) {
-    const int c0 = s.tgt_cptr[t], c1 = s.tgt_cptr[t + 1];
-    const int te = s.tgt_entry[t];
-    const bool fill_first = s.lu2y[te] < 0 && !touched[te];
-    touched[te] = 1;
-    const int k = s.lu_col[te];
-    const int mark = te == s.lu_diag[k] && last[k] == (int)t ? -2 - k : -1;
-    int rest = mark;
-    if (c1 - c0 > 1) {
-      rest = (int)con.size();
-      for (int c = c0 + 1; c < c1; ++c) con.push_back(make_int2(s.con_l[c], s.con_u[c]));
-      con.push_back(make_int2(-1, mark));
-    }
-    tgt[t] = make_int4(te | (fill_first ? kFillFirst : 0), s.con_l[c0], s.con_u[c0], rest);
-  }
-  if (con.empty()) con.push_back(make_int2(-1, -1));
-  // Within 256 items of a level those of the same work are neighbours: the
-  // items of a warp run in step (10,000 buses, 8 items a warp: 1.28 M FP64
-  // instructions a factorisation in the order of the entries, 0.93 M sorted so,
-  // 0.90 M sorted by level, which costs 32 scenarios a warp 2% in L2 hits).
-  auto by_work = [](std::vector<int4>& v, const std::vector<int>& ptr, auto work) {
-    for (size_t l = 0; l + 1 < ptr.size(); ++l)
-      for (int a = ptr[l]; a < ptr[l + 1]; a += 256)
-        std::stable_sort(v.begin() + a, v.begin() + std::min(a + 256, ptr[l + 1]),
-                         [&](const int4& x, const int4& y) { return work(x) > work(y); });
-  };
-  by_work(fac, s.fac_ptr, [](const int4& f) { return f.w ? (f.x == f.z ? 0 : 1) : 2; });
-  by_work(tgt, s.tgt_ptr, [&](const int4& t) {
-    int len = 1, mark = t.w;
-    for (int q = t.w; q >= 0 && con[q].x >= 0; ++q, ++len) mark = con[q + 1].y;
-    return len + (mark < -1 ? 1000 : 0);
-  });
-}
 
 int SysBuf::build(const CaseData& c, const Ybus& y, Ordering ord, bool fill) {
   analyze(y, ord, fill, sym);
@@ -257,6 +191,12 @@ int SysBuf::build(const CaseData& c, const Ybus& y, Ordering ord, bool fill) {
   UP(fac, fac_rec);
   UP(tgt, tgt_rec);
   UP(con, con);
+  d.fac_recw = d.tgt_recw = nullptr;
+  if (c.kind == PF_SINGLE_PHASE) {
+    sort_records(s, fac, tgt, con);
+    UP(fac, fac_recw);
+    UP(tgt, tgt_recw);
+  }
 #undef UP
   d.nflev = (int)s.flev_ptr.size() - 1;
   d.nblev = (int)s.blev_ptr.size() - 1;

@@ -64,6 +64,8 @@ struct DevSys {
   const int4* bwd_rec;
   const int4* fac_rec;
   const int4* tgt_rec;
+  const int4* fac_recw;  // the same sorted by work (2x2 blocks; records.h)
+  const int4* tgt_recw;
   const int2* con;
   const int8_t* g_fwd;
   const int8_t* g_bwd;

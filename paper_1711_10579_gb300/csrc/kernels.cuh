@@ -1253,19 +1253,6 @@ __device__ __forceinline__ bool inv_2x2(const TF (&a)[4], TF (&di)[4]) {
   return finite_bits(di[0]) && finite_bits(di[1]) && finite_bits(di[2]) && finite_bits(di[3]);
 }
 
-// factor_pipe's U_kk^-1.  FP32: the elimination with row exchanges of
-// factor_run, for blocks of any size, so that a mixed batch rounds as it does
-// there; the last FP32 step of a solve is not always refined, and two roundings
-// of the inverse put voltages of the same mismatch up to 1e-7 apart.  FP64: the
-// adjugate (1e-13 apart).
-__device__ __forceinline__ bool inv_pipe(const float (&a)[4], float (&di)[4]) {
-  float t[4] = {a[0], a[1], a[2], a[3]};
-  return blk_inv<2>(t, di);
-}
-__device__ __forceinline__ bool inv_pipe(const double (&a)[4], double (&di)[4]) {
-  return inv_2x2(a, di);
-}
-
 // The pivot whose diagonal block a target record finishes (-1: none), from the
 // record's `rest` or the end mark of its list.
 __device__ __forceinline__ int finished_pivot(int mark) { return mark < -1 ? -2 - mark : -1; }
@@ -1289,7 +1276,13 @@ struct FactorPipe {
 // by its pipe (a warp instruction per 64 cycles and sub-partition), so a
 // pivot's block is inverted once, by the item that updates it last (a level
 // earlier), not for each of its L entries: with the items sorted by work, 5
-// factorisations of 10,000 buses x 608 take 9.5 ms instead of 12.9 ms.
+// factorisations of 10,000 buses x 608 take 9.5 ms instead of 12.9 ms.  FP32
+// inverts for each, with row exchanges, as factor_run does: its rounding is then
+// that of the same solve there (the last FP32 step of a solve is not always
+// refined, and another rounding of the inverse moves its voltages by up to 1e-7
+// at the same mismatch), and an inversion at the end of a target's item holds up
+// the level (solves of 2,000 buses x 512: 2.66 ms so, 2.59 ms inverting for each,
+// 2.50 ms with the items in the order of the entries too).
 template <typename TF>
 __device__ __noinline__ void factor_pipe(const FactorArgs<TF> S, const Team tm, int l0, int l1) {
   if (l0 >= l1) return;
@@ -1352,9 +1345,10 @@ __device__ __noinline__ void factor_pipe(const FactorArgs<TF> S, const Team tm, 
     }
   };
   // step 1: r = {e, k, diag(k), ready}: L_ik = A_ik U_kk^-1, with U_kk^-1
-  // formed here for the pivots without updates (ready = 0)
+  // formed here where it is not ready (FP32; the pivots without updates)
+  constexpr bool ONCE = sizeof(TF) == 8;
   auto fetch1 = [&](int d, int4 r) {
-    if (!r.w) {
+    if (!ONCE || !r.w) {
       fetch_blk(d, 0, S.lu, r.z);
     } else if (r.x != r.z) {
       fetch_blk(d, 0, S.uinv, r.y);
@@ -1362,13 +1356,16 @@ __device__ __noinline__ void factor_pipe(const FactorArgs<TF> S, const Team tm, 
     if (r.x != r.z) fetch_blk(d, 1, S.lu, r.x);
   };
   auto work1 = [&](int d, int4 r) {
-    if (r.w && r.x == r.z) return;
+    if (ONCE && r.w && r.x == r.z) return;
     TF di[BB];
     read_blk(d, 0, di);
     bool ok = true;
-    if (!r.w) {
+    if constexpr (!ONCE) {
+      TF a[BB] = {di[0], di[1], di[2], di[3]};
+      ok = blk_inv<2>(a, di);
+    } else if (!r.w) {
       const TF a[BB] = {di[0], di[1], di[2], di[3]};
-      ok = inv_pipe(a, di);
+      ok = inv_2x2(a, di);
     }
     if (r.x == r.z) {
       if (!ok) S.flag[gs] = 1;
@@ -1409,12 +1406,12 @@ __device__ __noinline__ void factor_pipe(const FactorArgs<TF> S, const Team tm, 
         blk_msub<2>(c, l2, u2);
       }
     }
-    const int k = finished_pivot(mark);
+    const int k = ONCE ? finished_pivot(mark) : -1;
     if (k < 0) {
       blk_store<2>(gblk(r.x & ~kFillFirst), c);
     } else {  // only its inverse is read from here on
       TF di[BB];
-      if (!inv_pipe(c, di)) S.flag[gs] = 1;
+      if (!inv_2x2(c, di)) S.flag[gs] = 1;
       blk_store<2>(S.uinv + ((size_t)k * S.B + gs) * BB, di);
     }
   };
@@ -1837,6 +1834,10 @@ __device__ __forceinline__ void factor_levels(const DevSys& S, const DevWork& w,
       return;
     }
     if (tm.S > 1 && ring) {
+      if (sizeof(TF) == 8) {
+        f.fac_rec = S.fac_recw;
+        f.tgt_rec = S.tgt_recw;
+      }
       factor_pipe<TF>(f, tm, l0, l1);
       return;
     }
