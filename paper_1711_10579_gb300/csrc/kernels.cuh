@@ -70,16 +70,6 @@ __device__ __forceinline__ double recip(double x) {
   return __fma_rn(r, __fma_rn(e, e, e), r);
 }
 
-// FP32 -> FP64 by integer instructions (the conversion is an FP64 one);
-// denormals become zeros of their sign.
-__device__ __forceinline__ double to_f64(float v) {
-  const unsigned u = (unsigned)__float_as_int(v), ex = u & 0x7f800000u, sign = u & 0x80000000u;
-  unsigned hi = ((u & 0x7fffffffu) >> 3) + (896u << 20);
-  hi = ex == 0x7f800000u ? hi | 0x7ff00000u : hi;  // infinities and NaN
-  hi = ex == 0u ? 0u : hi;
-  return __hiloint2double((int)(hi | sign), ex == 0u ? 0 : (int)(u << 29));
-}
-
 // |v| as an ordered bit pattern: non-negative doubles order like their bits,
 // and a NaN of either sign maps above +inf.  Integer work only.
 __device__ __forceinline__ unsigned long long abs_bits(double v) {
@@ -89,19 +79,8 @@ __device__ __forceinline__ unsigned long long abs_bits(double v) {
 // sin a and cos a: the table method in 64-bit fixed point on the integer
 // pipes (fixtrig.h; four FP64-free conversions and a dozen 64-bit integer
 // products), sincos() beyond |a| <= 4.
-// The library's in a function of its own: inlined, part of it is executed
-// under a false predicate, which takes the FP64 pipe all the same.
-static __device__ __noinline__ double2 sincos_lib(double a) {
-  double2 r;
-  sincos(a, &r.y, &r.x);
-  return r;
-}
 __device__ __forceinline__ void sincos_tab(const long long* tab, double a, double* s, double* c) {
-  if (!fx::sincos_q(tab, a, s, c)) {
-    const double2 r = sincos_lib(a);
-    *s = r.y;
-    *c = r.x;
-  }
+  if (!fx::sincos_q(tab, a, s, c)) sincos(a, s, c);
 }
 
 // The FP64 refinement of a mixed-precision Newton-Raphson step is taken
@@ -254,8 +233,7 @@ __device__ __forceinline__ T group_sum(T v, int G, unsigned gmask) {
 // ---------------------------------------------------------------------------
 
 // The voltage dependence of a load other than constant power, in a function of
-// its own: a branch the other rows jump over instead of two predicated FP64
-// instructions, which take the pipe all the same.
+// its own, which the other rows jump over.
 static __device__ __noinline__ double load_shape(double zz, double zi, double zp, double vm) {
   return fma(fma(zz, vm, zi), vm, zp);
 }
@@ -296,7 +274,10 @@ __device__ void mismatch_jacobian_1ph(const DevSys& S, const DevWork& w, int i, 
   // conj(I): the operations of a row are what the batched kernel takes its time
   // for, so only the bus type's equations are formed (the lanes of a warp share
   // the row) and constant-power loads take no polynomial (10,000 buses x 9,728
-  // mixed, 6 evaluations: 28.7 -> 26.0 ms; x 608 FP64 5.7 -> 4.7 ms).
+  // mixed, 6 evaluations: 28.7 -> 26.4 ms; x 608 FP64 5.8 -> 4.9 ms).  Every load
+  // is issued before the sum: the row of a small batch is a chain of latencies
+  // (500 x 255 mixed, all evaluations of a solve: 414 -> 400 us).
+  const double qgen = (t == kPQLimit) ? __ldcg(w.qsw + b) : S.q_gen[i];
   double2 I = make_double2(0.0, 0.0);
   auto mismatch = [&]() {
     double f0 = 0.0, f1 = 0.0;
@@ -306,14 +287,12 @@ __device__ void mismatch_jacobian_1ph(const DevSys& S, const DevWork& w, int i, 
         if (nonzero(zi, zz)) shape = load_shape(zz, zi, zp, vmi);
         f0 = fma(-Vi.x, I.x, fma(-Vi.y, I.y, fma(-pl, shape, pg)));
         if (t >= PF_PQ) {
-          const double qgen = (t == kPQLimit) ? __ldcg(w.qsw + b) : S.q_gen[i];
           f1 = fma(-Vi.y, I.x, fma(Vi.x, I.y, fma(-ql, shape, qgen)));
         }
       }
     } else {
       const double2 Sc = cmulc(Vi, I);
       const double shape = fma(fma(zz, vmi, zi), vmi, zp);
-      const double qgen = (t == kPQLimit) ? __ldcg(w.qsw + b) : S.q_gen[i];
       f0 = (t != PF_SLACK) ? fma(-pl, shape, pg) - Sc.x : 0.0;
       f1 = (t >= PF_PQ) ? fma(-ql, shape, qgen) - Sc.y : 0.0;
     }
@@ -2140,8 +2119,8 @@ __device__ __forceinline__ double update_row(const DevSys& S, const DevWork& w, 
     double dd, dm;
     if (y && sizeof(TY) == 4) {
       const float2 q = __ldcg(reinterpret_cast<const float2*>(y) + b);
-      dd = to_f64(q.x);
-      dm = to_f64(q.y);
+      dd = (double)q.x;
+      dm = (double)q.y;
     } else {
       const double2 q = __ldcg(reinterpret_cast<const double2*>(y ? (const void*)y : (const void*)w.dx) + b);
       dd = q.x;
