@@ -485,12 +485,8 @@ struct PhaseClock {
 template <int BS, typename TF>
 cudaError_t set_smem(const Plan<BS, TF>& p) {
   cudaError_t e = cudaSuccess;
-  if (p.ring > 48 * 1024)
-    e = cudaFuncSetAttribute(k_factor<BS, TF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)p.ring);
-  if (e == cudaSuccess && p.red > 48 * 1024)
-    e = cudaFuncSetAttribute(k_solve<BS, TF>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)p.red);
+  if (p.ring > 48 * 1024) e = allow_launches((const void*)k_factor<BS, TF>);
+  if (e == cudaSuccess && p.red > 48 * 1024) e = allow_launches((const void*)k_solve<BS, TF>);
   return e;
 }
 

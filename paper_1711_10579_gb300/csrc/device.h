@@ -207,4 +207,10 @@ struct GroupList {
 enum ProfPhase { kProfSetup = 0, kProfMismatch, kProfStop, kProfFactor, kProfSolve,
                  kProfResidual, kProfUpdate, kProfOutput, kProfPhases };
 
+// Lets `kern` take all the dynamic shared memory a CTA of the current device has
+// beside its static arrays, and clusters of 16 CTAs.  Both belong to the function
+// and are seen by every host thread's launches, so they are set once per function
+// and device and never lowered to one launch's size (newton.cu).
+cudaError_t allow_launches(const void* kern);
+
 }  // namespace pf

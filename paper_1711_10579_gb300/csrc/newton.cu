@@ -44,6 +44,32 @@ cudaError_t noalloc_scratch(void** ptr) {
   return cudaSuccess;
 }
 
+cudaError_t allow_launches(const void* kern) {
+  static std::mutex mu;
+  static struct {
+    const void* kern;
+    int dev;
+  } done[512];  // no host heap: pf_solve_noalloc comes here
+  static int ndone = 0;
+  int dev = 0, most = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lk(mu);
+  for (int k = 0; k < ndone; ++k)
+    if (done[k].kern == kern && done[k].dev == dev) return cudaSuccess;
+  cudaFuncAttributes a;
+  e = cudaFuncGetAttributes(&a, kern);
+  if (e == cudaSuccess)
+    e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             most - (int)a.sharedSizeBytes);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e == cudaSuccess && ndone < 512) done[ndone++] = {kern, dev};
+  return e;
+}
+
 size_t dynamic_smem_bytes(int bs, size_t tf, bool nk, int n, const DevOpts& o, int threads) {
   size_t b = o.y_in_smem ? (size_t)n * bs * tf : 0;
   if (nk) {

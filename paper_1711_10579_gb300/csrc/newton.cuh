@@ -764,19 +764,11 @@ cudaError_t launch_t(const DevSys& S, const DevWork& w, const DevOpts& o, int gr
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = dynamic_smem_bytes(BS, sizeof(TF), NK, S.n, o, threads);
-  // (static + dynamic shared memory above 48 KB needs the opt-in)
-  if (cfg.dynamicSmemBytes > 0) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)cfg.dynamicSmemBytes);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = allow_launches((const void*)kern);
+  if (e != cudaSuccess) return e;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   if (CL) {
-    if (cluster > 8) {
-      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-      if (e != cudaSuccess) return e;
-    }
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = cluster;
     attr[0].val.clusterDim.y = 1;
@@ -791,7 +783,7 @@ cudaError_t launch_t(const DevSys& S, const DevWork& w, const DevOpts& o, int gr
 template <int BS, typename TF, bool NK>
 int max_cluster_t(int threads) {
   auto kern = newton_kernel<BS, TF, true, NK>;
-  cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  allow_launches((const void*)kern);
   for (int c = 16; c >= 1; c >>= 1) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(c);
@@ -814,11 +806,8 @@ template <int BS, typename TF, bool CL>
 cudaError_t launch_group_t(const GroupJob* desc, const GroupList& list, size_t smem,
                                   int cluster, cudaStream_t st) {
   auto kern = newton_group_kernel<BS, TF, CL>;
-  if (smem > 0) {  // (static + dynamic shared memory above 48 KB needs the opt-in)
-    cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
+  const cudaError_t e = allow_launches((const void*)kern);
+  if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(list.n * cluster);
   cfg.blockDim = dim3(BS == 2 ? 512 : 256);

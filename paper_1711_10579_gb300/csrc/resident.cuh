@@ -89,9 +89,7 @@ __device__ __forceinline__ void put_info(pf_info* out, int st, int it, int lin, 
 template <class Kern>
 cudaError_t configure_clusters(Kern kern, int P, int threads, size_t smem, int clusters,
                                cudaStream_t st, cudaLaunchConfig_t& cfg, cudaLaunchAttribute* attr) {
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e == cudaSuccess && P > 8)
-    e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  const cudaError_t e = allow_launches((const void*)kern);
   cfg.gridDim = dim3(clusters * P);
   cfg.blockDim = dim3(threads);
   cfg.dynamicSmemBytes = smem;
