@@ -315,40 +315,43 @@ int resident_single(const Symbolic& s, bool fp32, bool three) {
 // FP64 x 255 685 / 482 / 439 / 636; 2,000 mixed x 512 (one CTA an SM) 4,558 /
 // 2,471 / 1,584 / 1,322.
 //
-// Resident up to 8 clusters per resident CTA of the GPU, whatever the batch
-// where 8 fit an SM; beyond, the phase kernels' 32 scenarios per warp win.
+// Resident up to 8 CTAs per resident CTA of the GPU, whatever the batch where 8
+// scenarios fit an SM; beyond, the phase kernels' 32 scenarios per warp win.  CTAs
+// per scenario that the caller asks for (`asked`) are taken within the same bounds.
 // Measured (ms, resident against phase kernels in their best shape): mixed, 14
 // buses x 9,728 0.26 / 0.43; FP64, 60 x 9,728 1.40 / 1.46, 200 x 3,000 1.70 /
 // 2.15 and x 9,728 5.4 / 4.7, 500 x 2,000 2.98 / 3.80, 1,000 x 1,200 3.9 / 4.3
 // and x 2,400 7.9 / 7.1, 2,000 (2 CTAs) x 256 3.2 / 4.2 and x 1,000 11.0 / 7.7.
-ResidentShape resident_batch(const Symbolic& s, bool fp32, bool three, int B, int num_sms, int P) {
-  const bool asked = P > 0;  // CTAs per scenario given by the caller
-  if (!resident_default(s.n, fp32, three) && (three || !asked)) return {0, 0};
-  if (B == 1) return {P, 0};
+ResidentShape resident_batch(const Symbolic& s, bool fp32, bool three, int B, int num_sms, int asked) {
+  if (!resident_default(s.n, fp32, three) && (three || asked == 0)) return {0, 0};
+  if (B == 1) return {asked, 0};
+  // the shape on P CTAs per scenario, or {0, 0} for too large a batch
+  auto shape = [&](int P) -> ResidentShape {
+    if (P == 0) return {0, 0};
+    if (three) return {(double)B * P > (s.n > 280 * P ? 4.0 : 13.0) * num_sms ? 0 : P, 0};
+    int threads = resident_threads(s.n, P), per_sm = 1;
+    const double blocks =
+        (P > 1 ? 1.15 : 1.0) * ((double)s.nnz_lu() * 4 + 2.0 * s.n) * (fp32 ? 4 : 8) / P + 4096;
+    while (per_sm < 8 && (double)B * P > (double)per_sm * num_sms &&
+           2 * per_sm * (blocks + 64.0 * std::min(threads, 256 / per_sm)) <= 224 * 1024) {
+      per_sm <<= 1;
+      threads = std::min(threads, 512 / per_sm);
+    }
+    const double most = per_sm >= 8 && P == 1 ? 1e30 : (P > 1 && !fp32 ? 5.0 : 8.0) * per_sm;
+    return {(double)B * P > most * num_sms ? 0 : P, threads};
+  };
+  int P = 0;
   if (three) {
     // feeders: CTAs of at most 256 nodes, so that two fit an SM.  Measured (ms,
     // resident against phase kernels): 1,000 nodes mixed x 500 3.6 / 4.7, FP64
     // x 250 5.0 / 5.8; 8,000 nodes FP64 x 16 5.4 / 16.3, x 61 16.3 / 16.8
-    if (!asked) {
-      P = feeder_least(s.n, fp32);
-      while (P > 0 && P < 16 && s.n > 256 * P) P <<= 1;
-      if ((double)B * P > (s.n > 280 * P ? 4.0 : 13.0) * num_sms) P = 0;
-    }
-    return {P, 0};
+    P = feeder_least(s.n, fp32);
+    while (P > 0 && P < 16 && s.n > 256 * P) P <<= 1;
+  } else {
+    P = resident_least(s, fp32);
   }
-  if (!asked) P = resident_least(s, fp32);
-  if (P == 0) return {0, 0};
-  int threads = resident_threads(s.n, P), per_sm = 1;
-  const double blocks =
-      (P > 1 ? 1.15 : 1.0) * ((double)s.nnz_lu() * 4 + 2.0 * s.n) * (fp32 ? 4 : 8) / P + 4096;
-  while (per_sm < 8 && (double)B * P > (double)per_sm * num_sms &&
-         2 * per_sm * (blocks + 64.0 * std::min(threads, 256 / per_sm)) <= 224 * 1024) {
-    per_sm <<= 1;
-    threads = std::min(threads, 512 / per_sm);
-  }
-  const double most = per_sm >= 8 ? 1e30 : (P > 1 && !fp32 ? 5.0 : 8.0) * per_sm;
-  if (!asked && (double)B * P > most * num_sms) P = 0;
-  return {P, threads};
+  const ResidentShape own = shape(P);
+  return asked == 0 || own.P == 0 ? own : shape(asked);
 }
 
 int SysBuf::resident_for(const Ybus& y, bool fp32, ResidentShape shape, const ResidentPlan** out) {

@@ -164,9 +164,10 @@ struct pf_case_s {
 namespace pf {
 
 // CTAs of a resident single solve (0: the case does not run on one by default),
-// and the shape of a batch of B (P > 0: on P CTAs per scenario; B = 1 with P).
+// and the shape of a batch of B (asked > 0: on that many CTAs per scenario; B = 1
+// only so).
 int resident_single(const Symbolic& s, bool fp32, bool three);
-ResidentShape resident_batch(const Symbolic& s, bool fp32, bool three, int B, int num_sms, int P = 0);
+ResidentShape resident_batch(const Symbolic& s, bool fp32, bool three, int B, int num_sms, int asked = 0);
 
 enum class RunMode { Solve, Eval, Step };
 enum class InspectKind { Mismatch, Jacobian, Step };

@@ -320,3 +320,22 @@ def test_resident_krylov_matches_oracle(env, n, m):
             assert np.max(np.abs(va[b] - r["va"])) <= 1e-6
     finally:
         pf.pf_destroy_case(c)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("kind,n,P,B", [("mesh", 500, 16, 3000), ("mesh", 2000, 4, 2000),
+                                        ("feeder", 1000, 16, 500)])
+def test_asked_ctas_keep_the_batch_rule(env, kind, n, P, B, prec):
+    """CTAs per scenario asked for: resident in a small batch; a batch too large for
+    resident solves runs as without them."""
+    pf, ctx = env
+    c = pf.pf_create_case(ctx, mesh(n) if kind == "mesh" else cases.feeder_case(n, 5))
+    try:
+        o, plain = (pf.make_opts(precision=prec, cluster_size=q) for q in (P, 0))
+        small = pf.pf_launch_config(c, o, 3)
+        assert small["cluster"] == P and small["grid"] == 3 * P
+        assert pf.pf_launch_config(c, o, B)["cluster"] == 1
+        assert pf.pf_launch_config(c, o, B) == pf.pf_launch_config(c, plain, B)
+    finally:
+        pf.pf_destroy_case(c)
