@@ -144,9 +144,10 @@ typedef struct {
   int cluster_size;   /* CTAs per cluster of a single solve (0 = chosen by size).
                          With block_threads and scen_per_cta 0 it asks PF_NR for
                          resident solves (pf_solve_batch) of that many CTAs per
-                         scenario, for grids in mixed precision too, whose
-                         voltages then differ from the default's by up to 4e-7
-                         (relative) within the same tol */
+                         scenario, instead of a tuned shape and for grids in
+                         mixed precision too, whose voltages then differ from the
+                         default's by up to 4e-7 (relative) within the same tol;
+                         batches too large for resident solves ignore it */
   int block_threads;  /* threads per CTA (0 = autotuned) */
   int scen_per_cta;   /* batched launch: scenarios per CTA (0 = autotuned) */
   int nk_fallback;    /* PF_NK through pf_solve / pf_solve_batch: redo every
@@ -483,7 +484,8 @@ int pf_branch_flows(pf_case c, int B, const double* vmag, const double* vang, do
  * block_threads == 0 use the stored shapes; *opts (in: method, precision;
  * out: the chosen shape, for PF_NR that of the factorisation, which alone
  * also applies to the sweeps when passed back explicitly), or 0, 0 where the
- * resident solves were faster than the phase kernels in those shapes.
+ * batch can run as resident solves (PF_NR, PF_NK) and these were faster than
+ * the kernels in those shapes.
  * Without tuning, a batch uses about one CTA per SM (at most 8 scenarios per
  * CTA; single-phase FP64 PF_NR 32), or the resident solves (pf_solve_batch).
  * Blocking; allocates the batch workspace.

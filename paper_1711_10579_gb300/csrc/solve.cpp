@@ -128,11 +128,19 @@ void launch_shape(pf_case c, const pf_opts& o, int B, bool fp32, int* grid, int*
 int resident_plan(pf_case c, const pf_opts& o, int B, RunMode mode, const ResidentPlan** out) {
   *out = nullptr;
   if (mode != RunMode::Solve || o.block_threads || o.scen_per_cta) return PF_OK;
+  if (B > 1 && !o.cluster_size) {  // the tuned choice, where there is one
+    std::lock_guard<std::mutex> lk(c->tuned_mu);
+    auto it = c->tuned.find({B, o.method, o.precision});
+    if (it != c->tuned.end() && !it->second[4]) return PF_OK;
+  }
   if (o.method == PF_NK) {
     // Not mixed: FP32 sums in another order move the mismatch of a step by 10%,
     // and where it lands that close to the limit (2.5% of load scenarios of the
     // 2,000-bus grid) the solve ends a step earlier or later, its voltages 1e-7
-    // apart from the persistent kernel's.
+    // apart from the persistent kernel's.  Any batch (ms, here against the
+    // persistent kernel's best shape): 50 buses x 4,864 7.4 / 18.3, 200 x 4,864
+    // 72 / 127, 500 x 2 to x 2,432 11.7 to 187 / 39.8 to 287, 1,000 x 1,216 349 /
+    // 791.
     if (c->bs != 2 || o.krylov != 0 || o.cluster_size || o.precision == PF_MIXED) return PF_OK;
     const int n = c->data.n;
     if (((size_t)c->nk.sym.nnz_lu() * 4 + 2 * (size_t)n) * 8 > kResidentSmem) return PF_OK;
@@ -142,11 +150,6 @@ int resident_plan(pf_case c, const pf_opts& o, int B, RunMode mode, const Reside
     return rc;
   }
   const bool fp32 = o.precision == PF_MIXED;
-  if (B > 1) {
-    std::lock_guard<std::mutex> lk(c->tuned_mu);
-    auto it = c->tuned.find({B, o.method, o.precision});
-    if (it != c->tuned.end() && !it->second[4]) return PF_OK;
-  }
   if (B == 1 && !o.cluster_size) {
     *out = c->nr.res_single[fp32 ? 1 : 0];
     return PF_OK;
@@ -614,23 +617,23 @@ int autotune(pf_case c, int B, pf_opts* io) {
   }
   io->scen_per_cta = bestS;
   io->block_threads = bestT;
-  // the phase kernels in those shapes against the resident solves
+  // the kernels in those shapes against the resident solves
   pf_opts t = o;
-  t.scen_per_cta = t.block_threads = 0;
+  t.scen_per_cta = t.block_threads = t.cluster_size = 0;
+  auto choose = [&](int resident) {
+    std::lock_guard<std::mutex> lk(c->tuned_mu);
+    c->tuned[{B, o.method, o.precision}][4] = resident;
+  };
   const ResidentPlan* plan = nullptr;
-  const bool fp32 = o.precision == PF_MIXED;
-  if (nr)
-    rc = c->nr.resident_for(
-        c->y, fp32, resident_batch(c->nr.sym, fp32, c->bs == 6, B, c->ctx->num_sms), &plan);
+  choose(1);
+  rc = resident_plan(c, t, B, RunMode::Solve, &plan);
+  choose(0);
   if (rc != PF_OK || !plan) return rc;
   float ms[2] = {1e30f, 1e30f};
   e = cudaEventCreate(&e0);
   if (e == cudaSuccess) e = cudaEventCreate(&e1);
   for (int k = 0; k < 4 && rc == PF_OK && e == cudaSuccess; ++k) {
-    {
-      std::lock_guard<std::mutex> lk(c->tuned_mu);
-      c->tuned[{B, o.method, o.precision}][4] = k & 1;
-    }
+    choose(k & 1);
     e = cudaEventRecord(e0, st);
     if (e == cudaSuccess)
       rc = run_solve(c, t, B, nullptr, nullptr, nullptr, ws, st, RunMode::Solve, nullptr, nullptr);
@@ -642,10 +645,7 @@ int autotune(pf_case c, int B, pf_opts* io) {
   cudaEventDestroy(e1);
   if (rc == PF_OK && e != cudaSuccess) rc = cuda_error(e, "timing the resident solves");
   const bool resident = rc == PF_OK && ms[1] < ms[0];
-  {
-    std::lock_guard<std::mutex> lk(c->tuned_mu);
-    c->tuned[{B, o.method, o.precision}][4] = resident ? 1 : 0;
-  }
+  choose(resident ? 1 : 0);
   if (resident) io->scen_per_cta = io->block_threads = 0;  // the stored choice
   return rc;
 }

@@ -339,3 +339,28 @@ def test_asked_ctas_keep_the_batch_rule(env, kind, n, P, B, prec):
         assert pf.pf_launch_config(c, o, B) == pf.pf_launch_config(c, plain, B)
     finally:
         pf.pf_destroy_case(c)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("method,prec,n,B", [("nk", 0, 60, 40), ("nk", 1, 60, 40), ("nr", 0, 300, 64),
+                                             ("nr", 1, 300, 64)])
+def test_tuned_choice_is_what_runs(env, method, prec, n, B):
+    """After pf_autotune the launch is the returned shape, or the resident solves
+    where it returned none; CTAs per scenario asked for come before it."""
+    pf, ctx = env
+    c = pf.pf_create_case(ctx, mesh(n))
+    m = pf.PF_NK if method == "nk" else pf.PF_NR
+    try:
+        got = pf.pf_autotune(c, B, pf.make_opts(method=m, precision=prec, nk_fallback=0))
+        shape = pf.pf_launch_config(c, pf.make_opts(method=m, precision=prec), B)
+        if got.scen_per_cta:
+            assert shape["scen_per_cluster"] == got.scen_per_cta
+            assert shape["threads"] == got.block_threads
+        else:
+            assert shape["scen_per_cluster"] == 1 and shape["grid"] == B * shape["cluster"]
+            assert got.block_threads == 0
+        if method == "nr":
+            asked = pf.pf_launch_config(c, pf.make_opts(method=m, precision=prec, cluster_size=2), B)
+            assert asked["cluster"] == 2 and asked["grid"] == 2 * B
+    finally:
+        pf.pf_destroy_case(c)
