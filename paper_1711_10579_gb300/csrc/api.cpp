@@ -377,8 +377,21 @@ int SysBuf::resident_for(const Ybus& y, bool fp32, ResidentShape shape, const Re
   return PF_OK;
 }
 
+// Whether the determinants of a grid's 2x2 pivots are in the FP32 range: the own
+// admittance of every bus but the slack within 2^+-30 pu.
+static bool fp32_units(const Symbolic& s, const Ybus& y, const std::vector<int8_t>& bus_type) {
+  for (int i = 0; i < s.n; ++i) {
+    if (bus_type[i] == PF_SLACK) continue;
+    const double* v = &y.val[2 * (size_t)s.y_src[s.lu2y[s.lu_diag[i]]]];
+    const double a = std::fabs(v[0]) + std::fabs(v[1]);
+    if (!(a >= std::ldexp(1.0, -30) && a <= std::ldexp(1.0, 30))) return false;
+  }
+  return true;
+}
+
 int SysBuf::upload_resident(const Ybus& y, bool fp32, ResidentPlan& r) {
   ResPlanHost h;
+  if (fp32 && !fp32_units(sym, y, bus_type)) return PF_OK;
   if (!res_plan_fit(sym, fp32, r.P, r.threads / res_lanes(fp32), kResidentSmem, h)) return PF_OK;
   r.smem = res_smem(h, fp32);
   if (resident_clusters(fp32, r.P, r.threads, r.smem) < 1) return PF_OK;

@@ -364,3 +364,35 @@ def test_tuned_choice_is_what_runs(env, method, prec, n, B):
             assert asked["cluster"] == 2 and asked["grid"] == 2 * B
     finally:
         pf.pf_destroy_case(c)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("kind,n,P", [("mesh", 2, 0), ("mesh", 14, 0), ("mesh", 32, 0), ("mesh", 33, 0),
+                                      ("mesh", 500, 4), ("feeder", 40, 0), ("feeder", 300, 0)])
+def test_solves_in_a_large_power_base(env, kind, n, P, prec):
+    """The same grid per unit of a power base 1e22 times larger: admittances and
+    powers of 1e-22, whose 2x2 determinants are below the FP32 range.  Within
+    1e-6 of the oracle's voltages in the ordinary base."""
+    pf, ctx = env
+    k = 1e-22
+    if kind == "mesh":
+        case = mesh(n)
+        ref = O.newton_polar(case)
+        ref = ref["vm"] * np.exp(1j * ref["va"])
+        small = dataclasses.replace(case, br_r=case.br_r / k, br_x=case.br_x / k, br_b=case.br_b * k,
+                                    p_load=case.p_load * k, q_load=case.q_load * k,
+                                    p_gen=case.p_gen * k, q_gen=case.q_gen * k)
+    else:
+        case = cases.feeder_case(n, 5)
+        ref = O.newton_cim(case)["V"].reshape(-1)
+        small = dataclasses.replace(case, br_z=case.br_z / k, p_load=case.p_load * k,
+                                    q_load=case.q_load * k)
+    c = pf.pf_create_case(ctx, small)
+    try:
+        vm, va, info = pf.pf_solve(c, pf.make_opts(precision=prec, cluster_size=P, tol=1e-8 * k))
+        assert info["status"] == 0
+        on = np.abs(ref) > 0
+        assert np.max(np.abs(vm * np.exp(1j * va) - ref)[on]) <= 1e-6
+    finally:
+        pf.pf_destroy_case(c)
