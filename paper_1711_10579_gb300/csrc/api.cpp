@@ -49,6 +49,10 @@ cudaError_t DevBuffer::alloc(void** out, size_t nbytes) {
   *out = nullptr;
   if (nbytes == 0) nbytes = 16;
   nbytes = (nbytes + 255) & ~size_t(255);
+  if (count_only) {
+    bytes += nbytes;
+    return cudaSuccess;
+  }
   cudaError_t e = cudaMalloc(out, nbytes);
   if (e == cudaSuccess) {
     ptrs.push_back(*out);
@@ -62,7 +66,7 @@ static cudaError_t upload(DevBuffer& buf, const std::vector<T>& v, const T** out
   void* p;
   cudaError_t e = buf.alloc(&p, v.size() * sizeof(T));
   if (e != cudaSuccess) return e;
-  if (!v.empty()) e = cudaMemcpy(p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
+  if (!v.empty() && !buf.count_only) e = cudaMemcpy(p, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
   *out = static_cast<const T*>(p);
   return e;
 }
@@ -354,7 +358,20 @@ ResidentShape resident_batch(const Symbolic& s, bool fp32, bool three, int B, in
   return asked == 0 || own.P == 0 ? own : shape(asked);
 }
 
-int SysBuf::resident_for(const Ybus& y, bool fp32, ResidentShape shape, const ResidentPlan** out) {
+int SysBuf::build_single(const Ybus& y, bool three) {
+  for (int fp32 = 0; fp32 < 2; ++fp32) {
+    const ResidentPlan* plan = nullptr;
+    for (int P = resident_single(sym, fp32 != 0, three); P > 0 && P <= 16 && !plan; P <<= 1) {
+      const int rc = resident_for(y, fp32 != 0, {P, 0}, &plan);
+      if (rc != PF_OK) return rc;
+    }
+    res_single[fp32] = plan;
+  }
+  return PF_OK;
+}
+
+int SysBuf::resident_for(const Ybus& y, bool fp32, ResidentShape shape, const ResidentPlan** out,
+                         bool put) {
   std::lock_guard<std::mutex> lk(g_mu);
   *out = nullptr;
   if (shape.P == 0) return PF_OK;
@@ -367,13 +384,16 @@ int SysBuf::resident_for(const Ybus& y, bool fp32, ResidentShape shape, const Re
     slot = std::make_unique<ResidentPlan>();
     slot->P = shape.P;
     slot->threads = shape.threads;
-    const int rc = y.ybs == 1 ? upload_resident(y, fp32, *slot) : upload_feeder(y, fp32, *slot);
+    const int rc = y.ybs == 1 ? upload_resident(y, fp32, *slot, put) : upload_feeder(y, fp32, *slot, put);
     if (rc != PF_OK) {
       res_cache.erase(key);
       return rc;
     }
+  } else if (put && slot->fits && !slot->ok) {
+    const int rc = y.ybs == 1 ? upload_resident(y, fp32, *slot, put) : upload_feeder(y, fp32, *slot, put);
+    if (rc != PF_OK) return rc;
   }
-  if (slot->ok) *out = slot.get();
+  if (slot->fits) *out = slot.get();
   return PF_OK;
 }
 
@@ -389,12 +409,14 @@ static bool fp32_units(const Symbolic& s, const Ybus& y, const std::vector<int8_
   return true;
 }
 
-int SysBuf::upload_resident(const Ybus& y, bool fp32, ResidentPlan& r) {
+int SysBuf::upload_resident(const Ybus& y, bool fp32, ResidentPlan& r, bool put) {
   ResPlanHost h;
   if (fp32 && !fp32_units(sym, y, bus_type)) return PF_OK;
   if (!res_plan_fit(sym, fp32, r.P, r.threads / res_lanes(fp32), kResidentSmem, h)) return PF_OK;
   r.smem = res_smem(h, fp32);
-  if (resident_clusters(fp32, r.P, r.threads, r.smem) < 1) return PF_OK;
+  if (!mem.count_only && resident_clusters(fp32, r.P, r.threads, r.smem) < 1) return PF_OK;
+  r.fits = true;
+  if (!put) return PF_OK;
   auto val = [&](int e) { return &y.val[2 * (size_t)sym.y_src[e]]; };
   std::vector<double2> ell_y(h.ell_y.size(), make_double2(0.0, 0.0));
   for (size_t k = 0; k < ell_y.size(); ++k)
@@ -454,11 +476,14 @@ int SysBuf::upload_resident(const Ybus& y, bool fp32, ResidentPlan& r) {
   return PF_OK;
 }
 
-int SysBuf::upload_feeder(const Ybus& y, bool fp32, ResidentPlan& r) {
+int SysBuf::upload_feeder(const Ybus& y, bool fp32, ResidentPlan& r, bool put) {
   FeedPlanHost h;
   if (!feed_plan(sym, bus_type, r.P, r.threads / kFeedLanes, h)) return PF_OK;
   r.smem = feed_smem(h, fp32);
-  if (r.smem > kResidentSmem || feeder_clusters(fp32, r.P, r.threads, r.smem) < 1) return PF_OK;
+  if (r.smem > kResidentSmem) return PF_OK;
+  if (!mem.count_only && feeder_clusters(fp32, r.P, r.threads, r.smem) < 1) return PF_OK;
+  r.fits = true;
+  if (!put) return PF_OK;
   const int n = sym.n;
   auto val = [&](int e) { return &y.val[18 * (size_t)sym.y_src[e]]; };
   auto free_phase = [&](int i, int a) { return ((bus_type[i] >> a) & 1) && !(bus_type[i] & 8); };
@@ -784,14 +809,8 @@ int pf_create_case(pf_ctx ctx, const pf_case_desc* desc, pf_case* out) {
     rc = c->nr.lanes_for(pf::noalloc_threads(c->bs), 1, unused);
     if (rc != PF_OK) return rc;
     // and the resident plans of single solves
-    for (int fp32 = 0; fp32 < 2; ++fp32) {
-      const ResidentPlan* plan = nullptr;
-      for (int P = resident_single(c->nr.sym, fp32 != 0, c->bs == 6); P > 0 && P <= 16 && !plan; P <<= 1) {
-        rc = c->nr.resident_for(c->y, fp32 != 0, {P, 0}, &plan);
-        if (rc != PF_OK) return rc;
-      }
-      c->nr.res_single[fp32] = plan;
-    }
+    rc = c->nr.build_single(c->y, c->bs == 6);
+    if (rc != PF_OK) return rc;
   }
   {
     const int ki = c->data.kind == PF_SINGLE_PHASE ? 0 : 1;
@@ -999,42 +1018,21 @@ int pf_analyze(const pf_case_desc* desc, pf_case_stats* out) {
   int rc = copy_case(desc, d, err);
   if (rc == PF_OK) rc = build_ybus(d, y, err);
   if (rc != PF_OK) return set_error(rc, err);
-  Symbolic nr, nk;
-  analyze(y, Ordering::MinDegree, true, nr);
-  analyze(y, Ordering::RCM, false, nk);
-  fill_stats(d, nr, nk, out);
-  // what pf_create_case uploads: both systems' arrays and Ybus values
-  long long b = 0;
-  for (const Symbolic* s : {&nr, &nk}) {
-    b += 4LL * ((long long)s->y_rowptr.size() + s->y_col.size() + s->lu_rowptr.size() +
-                s->lu_col.size() + s->lu_diag.size() + s->lu2y.size() + s->fac_ptr.size() +
-                s->fac_items.size() + s->tgt_ptr.size() + s->tgt_entry.size() +
-                s->tgt_cptr.size() + s->con_l.size() + s->con_u.size() +
-                s->flev_ptr.size() + s->flev_rows.size() +
-                s->blev_ptr.size() + s->blev_rows.size() + s->perm.size());
-    b += (long long)y.val.size() * 8 + (long long)d.n * (1 + 8 * 9);
-  }
-  for (int fp32 = 0; fp32 < 2; ++fp32) {  // the plans of resident single solves
-    const int P = resident_single(nr, fp32 != 0, y.ybs == 3);
-    if (P == 0) continue;
-    if (y.ybs == 1) {
-      ResPlanHost h;
-      if (res_plan_fit(nr, fp32 != 0, P, resident_threads(nr.n, P) / res_lanes(fp32 != 0), kResidentSmem, h))
-        b += 4LL * (long long)(h.row.size() + h.ell_col.size() + h.jac.size() + h.rnd.size() +
-                               h.rec.size() + h.bnd.size() + h.gat.size() + h.gsrc.size()) +
-             16LL * (long long)h.ell_y.size() + (fp32 ? 2LL : 4LL) * (long long)h.jac.size();
-    } else {
-      FeedPlanHost h;
-      std::vector<int8_t> bt(d.n);
-      for (int i = 0; i < d.n; ++i)
-        bt[i] = !d.bus_type.empty() && d.bus_type[nr.perm[i]] == PF_PV ? 16 : 7;
-      if (feed_plan(nr, bt, P, feeder_groups(nr.n, P), h))
-        b += 4LL * (long long)(h.item.size() + h.ell_col.size() + h.node.size() + h.rnd.size() +
-                               h.rec.size()) +
-             48LL * (long long)h.ell_y.size() + (fp32 ? 152LL : 288LL) * d.n;
-    }
-  }
-  out->device_bytes = b;
+  // what pf_create_case uploads, counted
+  const int bs = d.kind == PF_SINGLE_PHASE ? 2 : 6;
+  SysBuf nr, nk;
+  DevBuffer warm;
+  nr.mem.count_only = nk.mem.count_only = warm.count_only = true;
+  DevSys unused;
+  rc = nr.build(d, y, Ordering::MinDegree, true);
+  if (rc == PF_OK) rc = nr.lanes_for(noalloc_threads(bs), 1, unused);
+  if (rc == PF_OK) rc = nr.build_single(y, bs == 6);
+  if (rc == PF_OK) rc = nk.build(d, y, Ordering::RCM, false);
+  if (rc != PF_OK) return rc;
+  void* p;
+  for (size_t each : {8, 8, 3 * 16}) warm.alloc(&p, d.n * each);
+  fill_stats(d, nr.sym, nk.sym, out);
+  out->device_bytes = (long long)(nr.mem.bytes + nk.mem.bytes + warm.bytes);
   return PF_OK;
 }
 
@@ -1225,7 +1223,7 @@ int pf_launch_config(pf_case c, const pf_opts* opts, int B, int* grid, int* clus
   if (opts) o = *opts; else pf_opts_default(&o);
   cudaSetDevice(c->ctx->device);
   const ResidentPlan* plan = nullptr;
-  const int rc = resident_plan(c, o, B, RunMode::Solve, &plan);
+  const int rc = resident_plan(c, o, B, RunMode::Solve, &plan, false);
   if (rc != PF_OK) return rc;
   if (plan) {
     *grid = B * plan->P;

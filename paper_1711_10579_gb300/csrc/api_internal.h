@@ -21,10 +21,12 @@ namespace pf {
 int set_error(int code, const std::string& msg);
 int cuda_error(cudaError_t e, const char* what);
 
-// A set of cudaMalloc'ed blocks released together.
+// A set of cudaMalloc'ed blocks released together (count_only: their sizes
+// alone, for pf_analyze).
 struct DevBuffer {
   std::vector<void*> ptrs;
   size_t bytes = 0;
+  bool count_only = false;
   ~DevBuffer();
   void release();
   cudaError_t alloc(void** out, size_t nbytes);
@@ -47,7 +49,8 @@ struct ResidentPlan {
   FeedDev feed{};
   const void* d_dev = nullptr;  // a copy of dev / feed in device memory (group launches)
   size_t smem = 0;
-  bool ok = false;  // fits the device (else the case runs the other kernels)
+  bool fits = false;  // the device (else the case runs the other kernels)
+  bool ok = false;    // uploaded
 };
 
 // One ordering of a case: host symbolic analysis plus its device copy.
@@ -63,15 +66,19 @@ struct SysBuf {
   // and cached); lanes_cached only looks them up and fails if absent.
   int lanes_for(int threads, int S, DevSys& out);
   int lanes_cached(int threads, int S, DevSys& out);
-  // The resident plan of a shape, built and uploaded on first use; null if the
-  // case does not fit it (or shape.P is 0).
-  int resident_for(const Ybus& y, bool fp32, ResidentShape shape, const ResidentPlan** out);
+  // The resident plan of a shape, built and uploaded on first use (put = false:
+  // its shape only, nothing uploaded); null if the case does not fit it (or
+  // shape.P is 0).
+  int resident_for(const Ybus& y, bool fp32, ResidentShape shape, const ResidentPlan** out,
+                   bool put = true);
+  // The plans of single solves, uploaded into res_single.
+  int build_single(const Ybus& y, bool three);
   // The plan of single solves (FP64, FP32), built with the case, or null.
   const ResidentPlan* res_single[2] = {nullptr, nullptr};
 
  private:
-  int upload_resident(const Ybus& y, bool fp32, ResidentPlan& r);
-  int upload_feeder(const Ybus& y, bool fp32, ResidentPlan& r);
+  int upload_resident(const Ybus& y, bool fp32, ResidentPlan& r, bool put);
+  int upload_feeder(const Ybus& y, bool fp32, ResidentPlan& r, bool put);
   std::map<std::array<int, 3>, std::unique_ptr<ResidentPlan>> res_cache;  // P, threads, fp32
 
   void finish_view(const std::array<const int8_t*, 2>& g, int threads, DevSys& out) const;
@@ -175,7 +182,8 @@ enum class InspectKind { Mismatch, Jacobian, Step };
 // Launches one solve of B scenarios on `ws` (asynchronous on `st`).
 // Outputs go to out_vm / out_va / out_info when given, else to the
 // workspace's staging buffers.
-int resident_plan(pf_case c, const pf_opts& o, int B, RunMode mode, const ResidentPlan** out);
+int resident_plan(pf_case c, const pf_opts& o, int B, RunMode mode, const ResidentPlan** out,
+                  bool put = true);
 int run_solve(pf_case c, const pf_opts& o, int B, const double* d_p_load,
               const double* d_q_load, const double* d_p_gen, Workspace* ws,
               cudaStream_t st, RunMode mode, double* out_vm, double* out_va,

@@ -125,7 +125,8 @@ void launch_shape(pf_case c, const pf_opts& o, int B, bool fp32, int* grid, int*
 // radial feeder) whose factor fits the shared memory of a cluster (mixed: small
 // ones, resident_single), GMRES on a grid whose ILU(0) factor fits one CTA's,
 // with no explicit shape of the other kernels asked for.
-int resident_plan(pf_case c, const pf_opts& o, int B, RunMode mode, const ResidentPlan** out) {
+int resident_plan(pf_case c, const pf_opts& o, int B, RunMode mode, const ResidentPlan** out,
+                  bool put) {
   *out = nullptr;
   if (mode != RunMode::Solve || o.block_threads || o.scen_per_cta) return PF_OK;
   if (B > 1 && !o.cluster_size) {  // the tuned choice, where there is one
@@ -145,7 +146,7 @@ int resident_plan(pf_case c, const pf_opts& o, int B, RunMode mode, const Reside
     const int n = c->data.n;
     if (((size_t)c->nk.sym.nnz_lu() * 4 + 2 * (size_t)n) * 8 > kResidentSmem) return PF_OK;
     const ResidentPlan* plan = nullptr;
-    const int rc = c->nk.resident_for(c->y, false, {1, 0}, &plan);
+    const int rc = c->nk.resident_for(c->y, false, {1, 0}, &plan, put);
     if (plan && resident_nk_smem(plan->smem, n, o.gmres_restart) <= kResidentSmem) *out = plan;
     return rc;
   }
@@ -156,7 +157,7 @@ int resident_plan(pf_case c, const pf_opts& o, int B, RunMode mode, const Reside
   }
   const ResidentShape shape =
       resident_batch(c->nr.sym, fp32, c->bs == 6, B, c->ctx->num_sms, o.cluster_size);
-  return c->nr.resident_for(c->y, fp32, shape, out);
+  return c->nr.resident_for(c->y, fp32, shape, out, put);
 }
 
 int run_solve(pf_case c, const pf_opts& o, int B, const double* d_p_load, const double* d_q_load,

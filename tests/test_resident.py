@@ -396,3 +396,29 @@ def test_solves_in_a_large_power_base(env, kind, n, P, prec):
         assert np.max(np.abs(vm * np.exp(1j * va) - ref)[on]) <= 1e-6
     finally:
         pf.pf_destroy_case(c)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kind,n", [("mesh", 1), ("mesh", 14), ("mesh", 33), ("mesh", 2749), ("mesh", 10000),
+                                    ("feeder", 40), ("feeder", 1106), ("feeder", 8000)])
+def test_analysis_counts_what_a_case_holds(env, kind, n):
+    """pf_analyze, which needs no GPU, against the created case; asking for a launch
+    configuration uploads nothing, the batch itself does."""
+    pf, ctx = env
+    case = mesh(n) if kind == "mesh" else cases.feeder_case(n, 3)
+    c = pf.pf_create_case(ctx, case)
+    try:
+        held = lambda: pf.pf_case_get_stats(c)["device_bytes"]
+        created = held()
+        assert pf.pf_analyze(case)["device_bytes"] == created
+        o = pf.make_opts(precision=pf.PF_FP64)
+        shape = pf.pf_launch_config(c, o, 3)
+        assert held() == created
+        if n == 2749:  # a batch runs on fewer CTAs than one solve: another plan
+            assert shape["cluster"] > 1 and shape["scen_per_cluster"] == 1
+            pl, ql, pg = _loads(case, 3, seed=1)
+            assert np.all(pf.pf_solve_batch(c, pl, ql, pg, o)[2]["status"] == 0)
+            assert held() > created
+            assert pf.pf_launch_config(c, o, 3) == shape
+    finally:
+        pf.pf_destroy_case(c)
