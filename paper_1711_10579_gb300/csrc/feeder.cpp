@@ -98,7 +98,11 @@ bool feed_plan(const Symbolic& s, const std::vector<int8_t>& btype, int P, int g
     double best = 1e300;
     std::vector<std::vector<int>> bins;
     while (!heap.empty()) {
-      if ((int)heap.size() >= P) {
+      // no bins are better than even ones, nor than the heaviest subtree's
+      const double least = std::max((double)heap.top().first, (double)(n - ntop) / P) + 0.25 * ntop;
+      if ((int)heap.size() >= P && least >= best) {
+        if (ntop > best) break;
+      } else if ((int)heap.size() >= P) {
         auto h = heap;
         std::vector<std::vector<int>> bb(P);
         std::priority_queue<std::pair<int, int>, std::vector<std::pair<int, int>>,

@@ -27,11 +27,12 @@ class RoundPacker {
                      [](const std::vector<Item>& a, const std::vector<Item>& b) {
                        return a.size() > b.size();
                      });
-    std::vector<std::vector<const Item*>> col(T_);
+    const int T = std::min(T_, (int)chains.size());  // no more slots are used
+    std::vector<std::vector<const Item*>> col(T);
     std::priority_queue<std::pair<int, int>, std::vector<std::pair<int, int>>,
                         std::greater<std::pair<int, int>>>
         pq;
-    for (int t = 0; t < T_; ++t) pq.push({0, t});
+    for (int t = 0; t < T; ++t) pq.push({0, t});
     size_t height = 0;
     for (const auto& ch : chains) {
       const auto top = pq.top();
@@ -42,7 +43,7 @@ class RoundPacker {
     }
     for (size_t r = 0; r < height; ++r) {
       int cnt = 0;
-      for (int t = 0; t < T_; ++t)
+      for (int t = 0; t < T; ++t)
         if (col[t].size() > r) cnt = t + 1;
       out_.rnd.push_back((int)(out_.rec.size() / 2));
       out_.rnd.push_back(cnt | (r + 1 == height ? kResSync : 0));
@@ -114,7 +115,13 @@ void cut_tree(const Symbolic& s, int P, double quad, std::vector<int>& part) {
   double best = 1e300, topw = 0.0;
   std::vector<int> top, best_top;
   for (int step = 0; step <= n && !heap.empty(); ++step) {
-    if ((int)heap.size() >= P || step == n) {
+    // the top runs after the parts, its rows one after another
+    const double after = 2.0 * topw + 40.0 * P * top.size() / 16.0;
+    // no bins are better than even ones, nor than the heaviest subtree's
+    const double least = std::max(heap.top().first, (total - topw) / P);
+    if (((int)heap.size() >= P || step == n) && (least + after) * (1.0 + 1e-9) >= best) {
+      if (topw + 40.0 * top.size() > best) break;
+    } else if ((int)heap.size() >= P || step == n) {
       std::vector<std::pair<double, int>> all;
       auto h = heap;
       while (!h.empty()) {
@@ -135,8 +142,7 @@ void cut_tree(const Symbolic& s, int P, double quad, std::vector<int>& part) {
         worst = std::max(worst, l.first);
         load.push(l);
       }
-      // the top runs after the parts, its rows one after another
-      const double cost = worst + 2.0 * topw + 40.0 * P * top.size() / 16.0;
+      const double cost = worst + after;
       if (cost < best) {
         best = cost;
         best_bins = bb;

@@ -114,6 +114,28 @@ def test_feeder_schedule_refuses_pv_nodes(host):
     assert host.feeder_check(40, *args(), 1, 8, C.byref(err), C.byref(levels)) == 100
 
 
+def test_analysis_of_a_comb_is_quick():
+    """A corridor of 10,000 buses with a bus at each (0.06 s; a cut that packs its
+    parts anew for every bus of the corridor takes seconds)."""
+    import time
+
+    from paper_1711_10579_gb300 import pf
+
+    n, h = 20_000, 10_000
+    one = cases.two_bus_case(0.0, 0.0, 0.1, 0.1)
+    f = np.r_[np.arange(h - 1), np.arange(h)].astype(np.int32)
+    t = np.r_[np.arange(1, h), np.arange(h, n)].astype(np.int32)
+    z = np.zeros(n)
+    case = dataclasses.replace(one, n_bus=n, br_from=f, br_to=t, br_r=np.full(n - 1, 0.01),
+                               br_x=np.full(n - 1, 0.1), br_b=np.zeros(n - 1),
+                               bus_type=np.r_[0, np.full(n - 1, 2)].astype(np.int32), v_set=z + 1.0,
+                               p_gen=z, q_gen=z, p_load=z, q_load=z,
+                               zip=np.tile([1.0, 0.0, 0.0], (n, 1)))
+    t0 = time.perf_counter()
+    assert pf.pf_analyze(case)["n_bus"] == n
+    assert time.perf_counter() - t0 < 1.5
+
+
 # ----------------------------------------------------------------------------
 # the kernels
 # ----------------------------------------------------------------------------
