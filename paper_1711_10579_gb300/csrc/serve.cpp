@@ -48,17 +48,18 @@ constexpr size_t kGroupSmemMax = 200 * 1024;  // a job's solve vector in shared 
 // Requests without a resident plan of at least this many rows (buses; nodes of
 // a feeder) run on a cluster of CTAs instead of one CTA: they are the tail of
 // the latency (8,000 nodes mixed: 14.5 / 9.6 / 6.4 / 4.8 ms on 1 / 2 / 4 / 8
-// CTAs; a 37,000-bus grid 29.5 / 22.9 / 17.5 / 15.4 ms).  While the CTAs in
-// flight make at most kWaves waves they take kBigCluster; a wide cluster costs
-// more CTA time, so beyond that 2 CTAs from kBigRows*, 4 from kMidRows* and
-// kBigCluster from kHugeRows*.  Measured: 24 requests of twelve grids (up to
-// 10,000 buses) 4.5 ms wide, 6.4 ms narrow; 2,000 requests a second of grids to
-// 65,000 buses: always wide 1,723 solves/s and a growing queue, by this rule
-// sustained (p50 5.1 ms, p99 41 ms; always narrow 4.4 and 40 ms).
-constexpr int kBigRows1ph = 4000, kBigRows3ph = 2000, kBigCluster = 8;
+// CTAs; a 37,000-bus grid 29.5 / 22.9 / 17.5 / 15.4 ms).  2 CTAs from kBigRows*, 4
+// from kMidRows*, kHugeCluster from kHugeRows*; while the CTAs in flight make at
+// most kWaves waves, feeders kHugeCluster and grids 4 from kBigRows* on.  A wider
+// cluster costs more CTA time.  Measured: 24 requests of twelve grids (up to
+// 10,000 buses), and 2,000 requests a second of grids to 65,000 buses (five streams
+// of 20 s, p50 / p99): never wide 6.35 ms, 5.5 / 38.3 ms; by this rule 4.77 ms,
+// 4.7 / 38.4 ms; grids on 8 CTAs too, up to 1.5 waves, 4.40 ms, 4.9 / 40.3 ms.
+constexpr int kBigRows1ph = 4000, kBigRows3ph = 2000;
 constexpr int kMidRows1ph = 16000, kMidRows3ph = 5000;
 constexpr int kHugeRows1ph = 40000, kHugeRows3ph = 12000;
-constexpr double kWaves = 1.5;
+constexpr int kHugeCluster = 8;
+constexpr double kWaves = 1.0;
 
 // Coalesced batches: kBatchMin or more queued Newton-Raphson requests of one
 // case with the same solve options and their own loads run as one batched
@@ -91,7 +92,8 @@ int group_cluster(const Request& r, bool busy) {
   const bool one = r.c->data.kind == PF_SINGLE_PHASE;
   const int n = r.c->data.n;
   if (n < (one ? kBigRows1ph : kBigRows3ph)) return 1;
-  if (!busy || n >= (one ? kHugeRows1ph : kHugeRows3ph)) return kBigCluster;
+  if (n >= (one ? kHugeRows1ph : kHugeRows3ph)) return kHugeCluster;
+  if (!busy) return one ? 4 : kHugeCluster;
   return n >= (one ? kMidRows1ph : kMidRows3ph) ? 4 : 2;
 }
 
@@ -463,7 +465,7 @@ struct Server {
       Group want;
       want.bs = r->c->bs;
       want.fp32 = r->o.precision == PF_MIXED;
-      want.cluster = plan ? plan->P : group_cluster(*r, ctas + kBigCluster > kWaves * ctx->num_sms);
+      want.cluster = plan ? plan->P : group_cluster(*r, ctas + kHugeCluster > kWaves * ctx->num_sms);
       jobs[k].ctas = want.cluster;
       ctas += want.cluster;
       want.threads = plan ? plan->threads : 0;
