@@ -43,12 +43,12 @@ ORACLE_SAMPLE = 16  # results of the timed step checked against the oracle
 # by the 4,864 scenarios (a launch's traffic is taken as these bytes per
 # scenario times its scenarios).  Valid only for the kernel sources it was measured on
 # (sha256 prefix of csrc/batch.cu + csrc/kernels.cuh); otherwise null.
-NCU_SOURCES = "dd32d8eb986dc819"
+NCU_SOURCES = "be7cd090a9eedb0d"
 NCU_TRAFFIC = {
-    "k_factor": (8_075_490_560 + 5_484_717_312) / 4864,
-    "k_solve": (6_198_120_192 + 843_736_320) / 4864,
-    "k_mismatch": (3_847_756_032 + 3_717_548_800) / 4864,
-    "k_update": (1_167_814_400 + 1_493_330_176) / 4864,
+    "k_factor": (8_097_284_352 + 5_486_695_936) / 4864,
+    "k_solve": (6_197_995_008 + 843_632_640) / 4864,
+    "k_mismatch": (3_848_719_872 + 3_722_118_656) / 4864,
+    "k_update": (1_167_891_200 + 1_493_378_560) / 4864,
 }
 WORKLOAD = (f"mesh10000 x {B_MAIN} load scenarios per step, batched Newton-Raphson, "
             "FP32 LU + FP64 mismatch/refinement/update, one CUDA graph per batch")
@@ -786,8 +786,8 @@ def profile_launches(count, B=608, S=0, threads=0, grid="mesh10000"):
 
 def profile_single(count, precision="mixed", method="nr", grid="mesh10000"):
     """``count`` single solves of a grid (default: the main step's) in the
-    kernel a single solve runs on (resident.cu; Newton-Krylov mixed: the
-    persistent kernel), for ncu."""
+    kernel a single solve runs on (FP64: resident.cu, resident_nk.cu; mixed
+    grids of more than 32 buses: the persistent kernel), for ncu."""
     import __graft_entry__
 
     __graft_entry__.build()

@@ -11,7 +11,8 @@
 // Measured (us, persistent kernel or phase kernels -> here): single solves of
 // 14 buses 276 -> 98 (a whole host call), 10,000 mixed 3,330 -> 426, 2,749 FP64
 // 2,140 -> 490; batches of 2,000 x 512 mixed 2,530 -> 1,262, 14 x 9,728 428 ->
-// 244, 500 x 255 mixed with reactive limits 2,070 -> 496.
+// 244, 500 x 255 mixed with reactive limits 2,070 -> 496.  Mixed grids of more
+// than 32 buses come here only where the caller asks (resident_default says why).
 #include "resident_blocks.cuh"
 
 namespace pf {
