@@ -363,8 +363,8 @@ int pf_drain(pf_ctx ctx, int timeout_ms);
  * Counters of the context's serving runtime since it started (all zero before
  * the first pf_submit).  Newton-Raphson requests (no reactive limits, default
  * launch shape) run as group launches: one launch solves several queued
- * requests of any cases and sizes, on the cluster of a resident single solve
- * of the case where its factor fits shared memory, else on one CTA each (a
+ * requests of any cases and sizes, each on the CTAs of a resident single solve
+ * where the case has one by default (pf_solve_batch), else on one CTA (a
  * cluster of 2 to 8 CTAs for grids of 4,000 buses or feeders of 2,000 nodes and
  * more, by size and by how many CTAs are in flight),
  * and each request retires when its own solve ends.  Runs of queued requests of one case are coalesced into batched
